@@ -83,7 +83,7 @@ def record_traffic(csv_path, size, command):
     head, units = rows[0], rows[1]
     k = head.index("Kernel Name")
     import re
-    pat = re.compile(r"tiled_pass_kernel<\d+, \d+, \d+, \d+, ([12]), \d+>")
+    pat = re.compile(r"tiled_pass_kernel<\d+, \d+, \d+, \d+, [12](, \d+)+>")
     hit = [r for r in rows[2:] if pat.search(r[k])]
     if not hit:
         raise SystemExit("no sampling launch of the colour pass in " + csv_path)

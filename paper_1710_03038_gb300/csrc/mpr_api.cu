@@ -1137,6 +1137,8 @@ mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bo
         a.rk[2 * i] = a.key.x + (uint32_t)i * 0x9E3779B9u;
         a.rk[2 * i + 1] = a.key.y + (uint32_t)i * 0xBB67AE85u;
     }
+    a.rk[18] ^= 0x80000000u;
+    a.rk[19] ^= 0x80000000u;
     a.q = (float)c->p.q;
     a.inv_q = (float)(1.0 / c->p.q);
     a.two_pi_q = (float)(2.0 * kPiD * c->p.q);

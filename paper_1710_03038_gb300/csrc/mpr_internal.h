@@ -95,7 +95,9 @@ struct SweepArgs {
     ChainDev ch;
     Control* ctl;
     uint2 key;
-    uint32_t rk[20];           // Philox round keys k_i = key + i * (0x9E3779B9, 0xBB67AE85)
+    uint32_t rk[20];           // Philox round keys k_i = key + i * (0x9E3779B9, 0xBB67AE85); the last
+                               // two with the top bit flipped (the tiled pass reads words 0 and 2
+                               // of a block as signed numbers)
     float q, inv_q, two_pi_q, J;
     int n_chains;
     int chain_group;

@@ -15,7 +15,7 @@
 // tile leaves at most one step partly idle.  Per launch the block
 //  - prepares, for every own-colour gap site, the constant part of its local
 //    field (sines and cosines of its sample neighbours, summed up, down, left,
-//    right), its random-stream counter word, and the byte offsets of its four
+//    right), its share of the random stream's first rounds, and the byte offsets of its four
 //    neighbours' entries in the block's table of other-colour gap cells
 //    (interior segment, then the 1-cell ring; entry 0 holds zeros for
 //    neighbours that are not gaps);
@@ -39,6 +39,14 @@
 // black gap sites (their site energy after their update) plus the bonds
 // between red gap sites and black sample sites.
 //
+// Variants.  What a launch needs is known when it is made, so it is compiled in:
+// ACC (sampling sweep), ENERGY (this pass records energies) and GROUPS: kRagged
+// (some pairs of a group may be missing), kWhole (every group has 2P chains: no test
+// of a pair's existence) and kOnly (the 2P chains of the one group are all there are:
+// slots lie 2P floats apart, a constant).  2048^2 x 32, ms per equilibration sweep: all
+// three read at run time 0.2867, ENERGY compiled in 0.2655, kOnly 0.2556.  Passes
+// that record energies run as kRagged: one variant less for rare passes.
+//
 // Models.  kModelMPR: the MPR bond with the q-consistent over-relaxation;
 // kModelLIT: the over-relaxation as printed (q = 1 field; the table cell
 // carries a second float4 with (cos phi, sin phi)); kModelGMRF: the GMRF bond
@@ -54,6 +62,7 @@ namespace mpr {
 namespace tiled {
 
 enum Model : int { kModelMPR = 0, kModelLIT = 1, kModelGMRF = 2 };
+enum Groups : int { kRagged = 0, kWhole = 1, kOnly = 2 };
 
 
 // bytes of one (entry, pair) table cell
@@ -71,7 +80,7 @@ struct Cfg {
     static constexpr size_t a16(size_t v) { return (v + 15) / 16 * 16; }
     // per own site: byte offsets of the four neighbour entries
     static constexpr size_t off_rows = 0;
-    // per own site: sample field (x, y), counter word, unused
+    // per own site: sample field (x, y), random-stream words
     static constexpr size_t off_k = off_rows + sizeof(uint4) * NMAX;
     // per own site (kModelLIT): the q = 1 sample field
     static constexpr size_t off_f1 = off_k + sizeof(uint4) * NMAX;
@@ -101,7 +110,7 @@ __device__ __forceinline__ float2 gmrf_bond2(float2 phi, float v) {
     return fma2(mul2(d, d), f2(0.050660591821168885f), f2(-1.0f));
 }
 
-template <int TX, int TY, int NW, int P, bool ACC, int MODEL>
+template <int TX, int TY, int NW, int P, bool ACC, int MODEL, bool ENERGY, int GROUPS>
 __global__ void __launch_bounds__(NW * 32, 1024 / (NW * 32))  // 64 registers: 32 warps per SM
 tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     using Cf = Cfg<TX, TY, NW, MODEL>;
@@ -130,10 +139,9 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     const TileDesc T = a.tiles[tile];
     const int c = a.colour;
     const int n_own = c ? T.cnt[1] : T.cnt[0];
-    const bool energy = (a.flags & kEnergy) != 0;
     const int n_oth = c ? T.cnt[0] : T.cnt[1];
     // nothing to update and no red-gap / black-sample bond energy to add
-    if (n_own == 0 && !(energy && n_oth > 0)) return;
+    if (n_own == 0 && !(ENERGY && n_oth > 0)) return;
     const int t_img = T.img;
     const int off_own = c ? T.off[1] : T.off[0], off_oth = c ? T.off[0] : T.off[1];
     const int n_halo = c ? T.halo_cnt[1] : T.halo_cnt[0];
@@ -141,16 +149,16 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     const ImgDev& I = a.img[t_img];
     const int r0 = a.chain0 + blockIdx.y * a.chain_group;
     const int ng = min(a.chain_group, a.chain_end - r0);
-    const bool has0 = 2 * p < ng;      // this lane's pair exists
-    const bool has1 = 2 * p + 1 < ng;  // and has a second chain
+    const bool has0 = GROUPS != kRagged || 2 * p < ng;      // this lane's pair exists
+    const bool has1 = GROUPS != kRagged || 2 * p + 1 < ng;  // and has a second chain
     const uint32_t sweep = a.ctl->sweep;
     const uint32_t c3 = (uint32_t)t_img | a.img_tag | ((uint32_t)c << 31);
     const uint32_t c2 = (uint32_t)(r0 >> 1) + (uint32_t)p;  // chain >> 1 of the pair
     const UpdateConst uk{a.q, a.inv_q, a.two_pi_q, a.J};
-    const long long cp = T.cp;  // floats from one slot to the next
+    const long long cp = GROUPS == kOnly ? 2 * P : T.cp;  // floats from one slot to the next
     // this lane's pair at slot 0 (8-byte aligned: state_off, cp, r0 are even)
     float* st = a.state + T.state_off + r0 + 2 * p;
-        float* sto = st + (long long)off_own * cp;  // this lane's pair at the own segment
+    float* sto = st + (long long)off_own * cp;  // this lane's pair at the own segment
     const int cpi = (int)cp;
     // angles of the first warp step, in flight during the table fill
     float2 vn = make_float2(0.0f, 0.0f);
@@ -176,6 +184,8 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
         const float* src = st + (long long)(off_oth + e_lo) * cp;
         const long long src_step = (long long)NTP * cp;
         uint32_t dst = cell_lo;
+        constexpr int kUnroll = GROUPS == kOnly ? 4 : 1;
+#pragma unroll kUnroll
         for (int e = e_lo; e < n_oth; e += NTP, src += src_step, dst += kDstStep)
             cp_async8_s(dst, src);
     }
@@ -198,8 +208,8 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
             own_rows[j] = make_uint4((r.x & 0xFFFFu) * kRow, (r.x >> 16) * kRow,
                                      (r.y & 0xFFFFu) * kRow, (r.y >> 16) * kRow);
             const uint32_t pos = a.slot_pos[b + j];
-            own_k[j] = make_uint4(__float_as_uint(f.x), __float_as_uint(f.y),
-                                  (pos & 0xFFFF0000u) | ((pos & 0xFFFFu) >> 1), 0u);
+            const uint2 pw = philox_site_words((pos & 0xFFFF0000u) | ((pos & 0xFFFFu) >> 1), c3, a.rk);
+            own_k[j] = make_uint4(__float_as_uint(f.x), __float_as_uint(f.y), pw.x, pw.y);
             if (MODEL == kModelLIT) own_f1[j] = make_float4(f.z, f.w, 0.0f, 0.0f);
         }
     }
@@ -220,6 +230,9 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     if (has0) {
         const float4* fcs = a.slot_cs + slot_off + off_oth;
         unsigned char* t = tab + (size_t)((1 + e_lo) * P + p) * CB;
+        // unrolled: the conversions of four entries overlap (0.2963 -> 0.2918 ms per
+        // equilibration sweep at 2048^2 x 32; by eight 0.2881 against 0.2867 by four)
+#pragma unroll 4
         for (int e = e_lo; e < n_ent; e += NTP, t += (size_t)NTP * P * CB) {
             const float2 v = *reinterpret_cast<const float2*>(t);
             if (MODEL != kModelGMRF) {
@@ -234,12 +247,12 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
                     reinterpret_cast<float4*>(t)[1] = make_float4(w0, w1, u0, u1);
                 }
                 *reinterpret_cast<float4*>(t) = make_float4(c0, c1, s0, s1);
-                if (energy && e < n_oth) {
+                if (ENERGY && e < n_oth) {
                     const float4 f = fcs[e];
                     const float2 d = fma2(f2(f.x), make_float2(c0, c1), mul2(f2(f.y), make_float2(s0, s1)));
                     esum = fma2(f2(-a.J), d, esum);
                 }
-            } else if (energy && e < n_oth) {
+            } else if (ENERGY && e < n_oth) {
                 // GMRF: bonds to the sample neighbours from the sample plane
                 const uint32_t pos = a.slot_pos[slot_off + off_oth + e];
                 const int X = (int)(pos & 0xFFFFu), Y = (int)(pos >> 16);
@@ -261,6 +274,7 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
             ? f2(proposal_width(1.0f))
             : make_float2(has0 ? a.ch.alpha[ch0] : 0.0f, has1 ? a.ch.alpha[ch0 + 1] : 0.0f);
     const float c_acc = 1.4426950408889634f * I.invT;  // log2(e) / T
+    const PhiloxPair pair_words = philox_pair_words(sweep, c2, a.rk);
     unsigned cnt0 = 0, cnt1 = 0;
     const int n_steps = (n_own + SPW - 1) / SPW;
     const unsigned char* tabp = tab + p * CB;  // this lane's column of the table
@@ -278,19 +292,18 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
         const int jj = in ? j : 0;  // idle lanes recompute slot 0 and store nothing
         const uint4 rw = own_rows[jj];
         const uint4 kk = own_k[jj];
-        const uint4 w = philox4x32_10_rk(make_uint4(kk.z, sweep, c2, c3), a.rk);
-        const PairRand u = pair_uniforms(w);
+        const PairRand u = pair_uniforms_flipped(philox_finish(kk.z, kk.w, pair_words, a.rk));
         PairOut o;
         if (MODEL == kModelGMRF) {
             const float2 gu = tab_f2(tabp + rw.x), gd = tab_f2(tabp + rw.y);
             const float2 gl = tab_f2(tabp + rw.z), gr = tab_f2(tabp + rw.w);
             const float2 sum = add2(add2(add2(add2(f2(__uint_as_float(kk.x)), gu), gd), gl), gr);
             o = gmrf_pair<false>(vc, sum, __uint_as_float(kk.y), u, a.J, alpha_s, c_acc);
-            if (energy) {
+            if (ENERGY) {
                 // the site's bonds after its update: gap neighbours from the table,
                 // sample neighbours from the sample plane
-                const int Y = (int)(kk.z >> 16);
-                const int X = 2 * (int)(kk.z & 0xFFFFu) + ((Y ^ c) & 1);
+                const uint32_t pos = a.slot_pos[slot_off + off_own + jj];
+                const int X = (int)(pos & 0xFFFFu), Y = (int)(pos >> 16);
                 const float* sp = a.samp + I.site_off + (long long)Y * I.Lx + X;
                 const bool hn[4] = {Y > 0, Y + 1 < I.Ly, X > 0, X + 1 < I.Lx};
                 const long long dn[4] = {-(long long)I.Lx, (long long)I.Lx, -1, 1};
@@ -333,35 +346,36 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
                                                  make_float2(hd.z, hd.w)),
                                             make_float2(hl.z, hl.w)),
                                        make_float2(hr.z, hr.w));
-                if (energy) o = literal_pair<true>(vc, C, S, C1, S1, u, uk, alpha_s, c_acc);
-                else o = literal_pair<false>(vc, C, S, C1, S1, u, uk, alpha_s, c_acc);
+                o = literal_pair<ENERGY>(vc, C, S, C1, S1, u, uk, alpha_s, c_acc);
             } else {
-                if (energy) o = hybrid_pair<true>(vc, C, S, u, uk, alpha_s, c_acc);
-                else o = hybrid_pair<false>(vc, C, S, u, uk, alpha_s, c_acc);
+                o = hybrid_pair<ENERGY>(vc, C, S, u, uk, alpha_s, c_acc);
             }
         }
         const bool act1 = act && has1;
         // a missing second chain is the padding chain of the layout: storing there is harmless
         if (act) *reinterpret_cast<float2*>(sto + j * cpi) = o.phi;
         if (ACC) {
-            // this pair's part of the site's realisation sums, added to that of
-            // pair p + 8 first (half the lanes on each shared-memory word), then
-            // in fixed point
+            // this pair's part of the site's realisation sums, in fixed point.  With 16
+            // pairs, pairs p and p + 8 add theirs first in one exchange: the lower lane
+            // gives its sum of squares for the other's sum, so that one shuffle and one
+            // shared-memory add per lane do both (0.3239 -> 0.3220 ms per sampling sweep
+            // at 2048^2 x 32)
             const float x0 = act ? o.phi.x : 0.0f, x1 = act1 ? o.phi.y : 0.0f;
-            float sa = x0 + x1, sb = fmaf(x0, x0, x1 * x1);
-            constexpr int kAdders = P >= 16 ? 8 : P;
+            const float sa = x0 + x1, sb = fmaf(x0, x0, x1 * x1);
             if (P >= 16) {
-                sa += __shfl_xor_sync(0xffffffffu, sa, 8);
-                sb += __shfl_xor_sync(0xffffffffu, sb, 8);
-            }
-            if (in && p < kAdders) {
+                const bool lower = p < 8;
+                const float v = (lower ? sa : sb) + __shfl_xor_sync(0xffffffffu, lower ? sb : sa, 8);
+                if (in)
+                    atomicAdd(&accs[(lower ? 0 : Cf::NMAX) + j],
+                              __float2uint_rn(v * (lower ? 16777216.0f : 2097152.0f)));
+            } else if (in) {
                 atomicAdd(&accs[j], __float2uint_rn(sa * 16777216.0f));
                 atomicAdd(&accs[Cf::NMAX + j], __float2uint_rn(sb * 2097152.0f));
             }
         }
         cnt0 += (act && o.acc0) ? 1u : 0u;
         cnt1 += (act1 && o.acc1) ? 1u : 0u;
-        if (energy) esum = add2(esum, make_float2(act ? o.e.x : 0.0f, act1 ? o.e.y : 0.0f));
+        if (ENERGY) esum = add2(esum, make_float2(act ? o.e.x : 0.0f, act1 ? o.e.y : 0.0f));
     }
 
     if (ACC) {
@@ -383,7 +397,7 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     for (int o = P; o < 32; o <<= 1) {
         cnt0 += __shfl_xor_sync(0xffffffffu, cnt0, o);
         cnt1 += __shfl_xor_sync(0xffffffffu, cnt1, o);
-        if (energy) {
+        if (ENERGY) {
             e0 += __shfl_xor_sync(0xffffffffu, e0, o);
             e1 += __shfl_xor_sync(0xffffffffu, e1, o);
         }
@@ -403,22 +417,22 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
         }
         const long long b0 = (long long)(t_img * a.n_chains + r0 + 2 * tid) * kSpread + spread;
         if (n0) atomicAdd(a.ch.acc_cnt + b0, n0);
-        if (energy) atomicAdd(a.ch.e_cur + b0, E0);
+        if (ENERGY) atomicAdd(a.ch.e_cur + b0, E0);
         if (2 * tid + 1 < ng) {
             if (n1) atomicAdd(a.ch.acc_cnt + b0 + kSpread, n1);
-            if (energy) atomicAdd(a.ch.e_cur + b0 + kSpread, E1);
+            if (ENERGY) atomicAdd(a.ch.e_cur + b0 + kSpread, E1);
         }
     }
 }
 
-template <int TX, int TY, int NW, int P, bool ACC, int MODEL>
+template <int TX, int TY, int NW, int P, bool ACC, int MODEL, bool ENERGY, int GROUPS>
 cudaError_t launch_one(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     using Cf = Cfg<TX, TY, NW, MODEL>;
     static_assert(Cf::smem_max <= 227 * 1024, "shared memory");
+    const auto kernel = tiled_pass_kernel<TX, TY, NW, P, ACC, MODEL, ENERGY, GROUPS>;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(tiled_pass_kernel<TX, TY, NW, P, ACC, MODEL>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)Cf::smem_max);
         if (e != cudaSuccess) return e;
         attr_set = true;
@@ -426,18 +440,40 @@ cudaError_t launch_one(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     if (setup_only) return cudaSuccess;
     if (a.gt < 1 || a.gt > Cf::GT) return cudaErrorInvalidValue;
     dim3 grid(a.n_list, (a.chain_end - a.chain0 + a.chain_group - 1) / a.chain_group);
-    tiled_pass_kernel<TX, TY, NW, P, ACC, MODEL><<<grid, Cf::NT, Cf::smem_for(a.gt, P), s>>>(a);
+    kernel<<<grid, Cf::NT, Cf::smem_for(a.gt, P), s>>>(a);
     return cudaGetLastError();
+}
+
+template <int TX, int TY, int NW, int P, bool ACC, int MODEL>
+cudaError_t launch_acc(const SweepArgs& a, cudaStream_t s, bool setup_only) {
+    // the variants for whole groups exist for 16 x 16 tiles, the shape of every
+    // automatic choice
+    constexpr bool kVariants = TX == 16 && TY == 16 && MODEL != kModelLIT;
+    constexpr int kW = kVariants ? kWhole : kRagged, kO = kVariants ? kOnly : kRagged;
+    if (setup_only) {
+        cudaError_t e = launch_one<TX, TY, NW, P, ACC, MODEL, true, kRagged>(a, s, true);
+        if (e == cudaSuccess) e = launch_one<TX, TY, NW, P, ACC, MODEL, false, kRagged>(a, s, true);
+        if (e == cudaSuccess) e = launch_one<TX, TY, NW, P, ACC, MODEL, false, kW>(a, s, true);
+        if (e == cudaSuccess) e = launch_one<TX, TY, NW, P, ACC, MODEL, false, kO>(a, s, true);
+        return e;
+    }
+    if (a.flags & kEnergy) return launch_one<TX, TY, NW, P, ACC, MODEL, true, kRagged>(a, s, false);
+    const bool whole = a.chain_group == 2 * P && (a.chain_end - a.chain0) % (2 * P) == 0;
+    // (slots are a multiple of 4 floats apart)
+    if (whole && a.n_chains == 2 * P && P % 2 == 0)
+        return launch_one<TX, TY, NW, P, ACC, MODEL, false, kO>(a, s, false);
+    if (whole) return launch_one<TX, TY, NW, P, ACC, MODEL, false, kW>(a, s, false);
+    return launch_one<TX, TY, NW, P, ACC, MODEL, false, kRagged>(a, s, false);
 }
 
 template <int TX, int TY, int NW, int P, int MODEL>
 cudaError_t launch_cfg(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     if (setup_only) {
-        cudaError_t e = launch_one<TX, TY, NW, P, false, MODEL>(a, s, true);
-        return e != cudaSuccess ? e : launch_one<TX, TY, NW, P, true, MODEL>(a, s, true);
+        cudaError_t e = launch_acc<TX, TY, NW, P, false, MODEL>(a, s, true);
+        return e != cudaSuccess ? e : launch_acc<TX, TY, NW, P, true, MODEL>(a, s, true);
     }
-    if (a.flags & kAccumulate) return launch_one<TX, TY, NW, P, true, MODEL>(a, s, false);
-    return launch_one<TX, TY, NW, P, false, MODEL>(a, s, false);
+    if (a.flags & kAccumulate) return launch_acc<TX, TY, NW, P, true, MODEL>(a, s, false);
+    return launch_acc<TX, TY, NW, P, false, MODEL>(a, s, false);
 }
 
 // pairs per site for a chain group of cg chains: the next power of two of
