@@ -430,12 +430,11 @@ def run_gpu(args):
                 "d2h_bytes_per_step": N * 4},
         "clocks": clocks,
     }
-    # kernel launches of one step: the library's per-sweep count for the realisations
-    # and for the temperature lattices, the Newton steps (and their set-up), the 16
-    # initialisation kernels of the two contexts (map, extremes, sample energy, tile
-    # tables, hot starts, chain set-up) and the prediction
-    t_sweeps = topts.iters * (topts.n_equil + topts.n_meas) + topts.n_equil
-    line["gpu_launches"] = args.steps * (launches[0] * (ne + nm) + launches[1] * t_sweeps
+    # kernel launches of one step: the library's per-sweep count for the realisations,
+    # two runs of the temperature lattices per Newton step (each one launch), the Newton
+    # steps (and their set-up), the 16 initialisation kernels of the two contexts (map,
+    # extremes, sample energy, tile tables, hot starts, chain set-up) and the prediction
+    line["gpu_launches"] = args.steps * (launches[0] * (ne + nm) + 2 * topts.iters
                                          + topts.iters + 1 + 16 + 1)
     if not args.no_plain:
         # the plain single-image path on the same job (one warm-up, one timed step)

@@ -10,6 +10,7 @@
 
 #include "mpr_device.cuh"
 #include "mpr_internal.h"
+#include "mpr_resident.h"
 
 using namespace mpr;
 
@@ -41,6 +42,7 @@ constexpr size_t kAlign = 256;
 constexpr int kHist = 512;  // chain-mean energies kept per image for the equilibration test
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 constexpr double kPiD = 3.14159265358979323846;
+constexpr int kResidentBlocks = 2048;  // upper bound on the blocks that run at once (8 per SM)
 
 // ============================================================ layout
 
@@ -48,7 +50,7 @@ constexpr double kPiD = 3.14159265358979323846;
 struct Layout {
     size_t img, ctl, ch_a, ch_alpha, ch_cnt, ch_last, ch_ecur, ch_elast, ch_esum, ch_esum2;
     size_t zst, gst, outst, eout, samp, slot_map, tiles, counts, halo, tile_list, scratch;
-    size_t slot_pos, slot_ref, slot_cs, acc1, acc2, state, newton, hist, sub;
+    size_t slot_pos, slot_ref, slot_cs, acc1, acc2, state, newton, hist, res_words, res_epoch, res_packets, res_e, res_end, sub;
     size_t total;
     long long n_slots;   // slot space over all images
     long long n_state;   // floats of the state buffer
@@ -99,6 +101,14 @@ void make_geometry(Geometry& g, int n_img, const int* Lx, const int* Ly, int n_c
     }
 }
 
+// Resident sweeps: 2^this words per chain, one per 64 tiles of the largest image.
+int resident_spread_log(const Geometry& g) {
+    int most = 1, s = 0;
+    for (int n : g.ntiles) most = std::max(most, n);
+    while (s < 4 && (64 << s) < most) ++s;
+    return s;
+}
+
 // Per image slot counts: tiled path = padded gap segments, plain = sites.
 Layout make_layout(const Geometry& g, const std::vector<long long>& slots_per_img,
                    size_t sub_bytes, bool staging) {
@@ -143,6 +153,15 @@ Layout make_layout(const Geometry& g, const std::vector<long long>& slots_per_im
     L.state = take(sizeof(float) * L.n_state);
     L.newton = take(sizeof(double) * 4 * g.n_img);
     L.hist = take(sizeof(double) * kHist * g.n_img + sizeof(int) * (g.n_img + 3));
+    // resident sweeps: per-chain words, epoch, boundary and energy packets (none when the
+    // batch has more blocks than one wave)
+    const size_t RT = tiled && g.n_tiles * (long long)((g.n_chains + 31) / 32) <= kResidentBlocks
+                          ? (size_t)g.n_tiles : 0;
+    L.res_words = take(RT ? 2 * (sizeof(unsigned long long) * NC << resident_spread_log(g)) : 0);
+    L.res_epoch = take(RT ? sizeof(uint32_t) : 0);
+    L.res_packets = take(3 * 64 * sizeof(ulonglong2) * RT * ((g.n_chains + 1) / 2));
+    L.res_e = take(3 * sizeof(ulonglong2) * RT * g.n_chains);
+    L.res_end = o;
     L.sub = take(sub_bytes);
     L.total = o;
     return L;
@@ -206,6 +225,10 @@ struct mpr_ctx {
     uint32_t sweep = 0, equil_index = 0;
     long long n_meas_done = 0;
     bool T_set = false;
+    // tiled: every tile and chain group fits the GPU at once, so a run of sweeps is one
+    // launch (resident sweeps) with this much shared memory per block
+    bool resident = false;
+    size_t res_smem = 0;
     mpr_ctx* sub = nullptr;   // unconditional lattices of the temperature estimate
     // instantiated CUDA graphs of sweep sequences, keyed by (n, phase, flags, stats, accumulate)
     std::vector<std::pair<long long, cudaGraphExec_t>> graphs;
@@ -822,6 +845,34 @@ mpr_status split_tiles(mpr_ctx* c, const std::vector<TileDesc>& tiles, cudaStrea
     return MPR_OK;
 }
 
+// Whether runs of sweeps go through the resident kernel: 16 x 16 tiles, the MPR bond
+// or the GMRF, and every (tile, chain group) block on the GPU at once.  The line lies
+// at the device's own limit: below it the resident run was the faster one at every
+// size measured.
+mpr_status choose_resident(mpr_ctx* c, const std::vector<TileDesc>& tiles, cudaStream_t s) {
+    const Geometry& g = c->g;
+    const int flags = model_flags(c->p);
+    c->resident = false;
+    if (g.tx != 16 || g.ty != 16 || (flags & kLiteralOR)) return MPR_OK;
+    ChainRange cr[2];
+    const int n_cr = chain_ranges(c, cr);
+    const long long groups = (cr[0].chain_end + cr[0].group - 1) / cr[0].group + (n_cr - 1);
+    // (with the blocks that record energies)
+    const long long need = (g.n_tiles + (long long)g.n_img * resident_recorders(cr[0].group)) * groups;
+    if (need > kResidentBlocks) return MPR_OK;
+    const int P = tiled_pairs(cr[0].group);
+    const bool gmrf = (flags & kGMRF) != 0;
+    size_t smem = 0;
+    for (const TileDesc& t : tiles) smem = std::max(smem, resident_smem(t, P, gmrf));
+    long long blocks = 0;
+    MPR_CUDA(resident_blocks(smem, gmrf, &blocks));
+    c->resident = need <= blocks;
+    c->res_smem = smem;
+    if (c->resident)
+        MPR_CUDA(cudaMemsetAsync(c->ws + c->L.res_words, 0, c->L.res_end - c->L.res_words, s));
+    return MPR_OK;
+}
+
 mpr_status sub_workspace_size(const mpr_params& p, const mpr_T_opts& o, int n_img, const int* Lx,
                               const int* Ly, size_t* bytes);
 
@@ -1047,6 +1098,7 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
                                  cudaMemcpyDeviceToHost, s));
         MPR_CUDA(cudaStreamSynchronize(s));
         MPR_TRY(split_tiles(c, tiles, s));
+        MPR_TRY(choose_resident(c, tiles, s));
         ChainRange cr[2];
         const bool extra = c->n_light[0] < g.n_tiles || c->n_light[1] < g.n_tiles ||
                            chain_ranges(c, cr) > 1;
@@ -1115,10 +1167,9 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
     return MPR_OK;
 }
 
-mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool accumulate,
-                         cudaStream_t s) {
-    const bool equil = phase == MPR_EQUIL;
-    const bool record = (flags & MPR_RECORD_ENERGY) != 0;
+// The arguments that every sweep launch of a context shares; `flags` holds the
+// phase's and the model's bits.
+SweepArgs sweep_args(const mpr_ctx* c, int phase, bool accumulate) {
     SweepArgs a{};
     a.img = c->d_img;
     a.tiles = c->d_tiles;
@@ -1147,15 +1198,52 @@ mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bo
     a.chain_group = pick_chain_group(c);
     a.chain0 = 0;
     a.chain_end = c->g.n_chains;
-    ChainRange cr[2];
-    const int n_cr = chain_ranges(c, cr);
     a.halo_cap = c->g.halo_cap;
     a.n_img = c->g.n_img;
     a.img_tag = c->img_tag;
-    int base = 0;
-    if (!equil && accumulate) base |= kAccumulate | kAccumulate2;
-    if (!equil && !c->p.freeze_a_in_measure) base |= kAlphaOne;
-    base |= model_flags(c->p);
+    if (phase != MPR_EQUIL && accumulate) a.flags |= kAccumulate | kAccumulate2;
+    if (phase != MPR_EQUIL && !c->p.freeze_a_in_measure) a.flags |= kAlphaOne;
+    a.flags |= model_flags(c->p);
+    return a;
+}
+
+// n sweeps as one launch
+mpr_status launch_resident_run(mpr_ctx* c, int n, int phase, int flags, bool stats, bool accumulate,
+                               cudaStream_t s) {
+    ResidentArgs r{};
+    r.a = sweep_args(c, phase, accumulate);
+    if (flags & MPR_RECORD_ENERGY) r.a.flags |= kEnergy;
+    r.n = n;
+    r.equil = phase == MPR_EQUIL ? 1 : 0;
+    r.stats = stats ? 1 : 0;
+    r.A_targ = c->p.A_targ;
+    r.k_a = c->p.k_a;
+    ChainRange cr[2];
+    const int n_cr = chain_ranges(c, cr);
+    r.group = cr[0].group;
+    r.n_whole = (cr[0].chain_end + cr[0].group - 1) / cr[0].group;
+    r.P = tiled_pairs(cr[0].group);
+    r.P_rest = n_cr > 1 ? tiled_pairs(cr[1].group) : r.P;
+    r.n_tiles = c->g.n_tiles;
+    r.words = at<unsigned long long>(c->ws, c->L.res_words);
+    r.recorders = resident_recorders(cr[0].group);
+    r.spread_log = resident_spread_log(c->g);
+    r.epoch = at<uint32_t>(c->ws, c->L.res_epoch);
+    r.packets = at<ulonglong2>(c->ws, c->L.res_packets);
+    r.energies = at<ulonglong2>(c->ws, c->L.res_e);
+    const cudaError_t e = launch_resident(r, r.n_whole + (n_cr - 1), c->res_smem, s);
+    if (e != cudaSuccess) return fail(MPR_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(e));
+    return MPR_OK;
+}
+
+mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool accumulate,
+                         cudaStream_t s) {
+    const bool equil = phase == MPR_EQUIL;
+    const bool record = (flags & MPR_RECORD_ENERGY) != 0;
+    SweepArgs a = sweep_args(c, phase, accumulate);
+    const int base = a.flags;
+    ChainRange cr[2];
+    const int n_cr = chain_ranges(c, cr);
     const bool tiled = c->g.path == MPR_PATH_TILED;
     for (int k = 0; k < n; ++k) {
         for (int colour = 0; colour < 2; ++colour) {
@@ -1260,7 +1348,7 @@ bool graphs_usable(const mpr_ctx* c, cudaStream_t s) {
     return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
 }
 
-// n sweeps: launched directly, or (sequences of at least 4 sweeps on a stream
+// n sweeps: as one launch (resident sweeps), launched directly, or (sequences of at least 4 sweeps on a stream
 // that may be captured) through a CUDA graph captured once per context and
 // replayed.  Every argument of the launches is fixed for the context's life
 // (temperatures, a, the sweep counter live in device memory), so a graph
@@ -1269,7 +1357,12 @@ mpr_status run_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool 
                       cudaStream_t s) {
     // (a caller that is capturing gets the launches in its own capture)
     const bool graph = n >= 4 && graphs_usable(c, s);
-    if (!graph) {
+    if (c->resident && n > 0) {
+        // (a chain's word holds 2^40 accepted proposals: 2^20 sweeps of 2048 tiles)
+        constexpr int kMost = 1 << 20;
+        for (int k = 0; k < n; k += kMost)
+            MPR_TRY(launch_resident_run(c, std::min(n - k, kMost), phase, flags, stats, accumulate, s));
+    } else if (!graph) {
         MPR_TRY(launch_sweeps(c, n, phase, flags, stats, accumulate, s));
     } else {
         const long long key = ((long long)n << 8) | (phase << 4) | ((flags & 1) << 3) |
@@ -1309,7 +1402,7 @@ mpr_status check_device_status(mpr_ctx* c, cudaStream_t s) {
                                          cudaMemcpyDeviceToHost, s));
     MPR_CUDA(cudaStreamSynchronize(s));
     if (st[0] | st[1])
-        return fail(MPR_ERR_DEVICE, "a kernel gave up waiting for an asynchronous copy (status " +
+        return fail(MPR_ERR_DEVICE, "a kernel gave up waiting (status " +
                                         std::to_string(st[0] | st[1]) + ")");
     return MPR_OK;
 }

@@ -143,6 +143,8 @@ cudaError_t launch_tile_const(const ImgDev* img, const TileDesc* tiles, int n_ti
 // launch whose largest tile has gt table entries; flags: the model bits of
 // SweepFlags (kLiteralOR, kGMRF).
 size_t tiled_pass_smem(int tx, int ty, int gt, int chain_group, int flags);
+// Chain pairs per site of a colour-pass block for a group of that many chains.
+int tiled_pairs(int chain_group);
 // blocks of the colour pass one SM holds by their threads and registers
 int tiled_blocks_per_sm(int tx, int ty);
 

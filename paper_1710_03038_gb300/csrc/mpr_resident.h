@@ -1,0 +1,42 @@
+// Resident sweeps (mpr_resident.cu): arguments and launchers.
+#pragma once
+
+#include "mpr_internal.h"
+
+namespace mpr {
+
+struct ResidentArgs {
+    SweepArgs a;         // as for the colour passes (flags without the per-colour kEnergy rule: set
+                         // when the sweeps record energies)
+    int n;               // sweeps of the run
+    int equil, stats;    // adapt a; add the energies to the chains' sums
+    double A_targ, k_a;
+    int group, n_whole;  // chains per group, groups of that size; the remaining chains follow
+    int P, P_rest;       // chain pairs per site of a whole group and of the remaining chains
+    int n_tiles;
+    int recorders;       // blocks per image and group that record energies (recorded runs only)
+    int spread_log;      // 2^spread_log words per chain and parity: about one per 64 tiles of an image
+    // [parity of the sweep][spread][chain]: tiles done << 40 | accepted proposals (zero
+    // between launches)
+    unsigned long long* words;
+    ulonglong2* packets;   // [3][tile][64 places][chain pairs]: (angle, epoch) words of both chains
+    ulonglong2* energies;  // [3][tile][chain]: (half of a double, epoch) words
+    uint32_t* epoch;       // epoch of the last launch's last pass
+};
+
+// Shared memory of a block of tile t with P chain pairs per site.
+size_t resident_smem(const TileDesc& t, int P, bool gmrf);
+// Blocks that record the energies of a group of that many chains.
+int resident_recorders(int group);
+// Blocks of that size that the device holds at once (0: no cooperative launches, or
+// one block does not fit); sets the kernels' shared-memory limit.
+cudaError_t resident_blocks(size_t smem, bool gmrf, long long* blocks);
+cudaError_t launch_resident(const ResidentArgs& ra, int n_groups, size_t smem, cudaStream_t s);
+
+namespace resident {
+using Kernel = void (*)(ResidentArgs);
+Kernel pick_mpr(bool acc, bool energy);
+Kernel pick_gmrf(bool acc, bool energy);
+}  // namespace resident
+
+}  // namespace mpr

@@ -196,6 +196,8 @@ size_t tiled_pass_smem(int tx, int ty, int gt, int chain_group, int flags) {
     return Cfg<16, 16, 4, kModelMPR>::smem_for(gt, P);
 }
 
+int tiled_pairs(int chain_group) { return tiled::pairs_for_group(chain_group); }
+
 int tiled_blocks_per_sm(int tx, int ty) {
     using namespace tiled;
     if (tx == 32) return 1024 / Cfg<32, 16, 8, kModelMPR>::NT;

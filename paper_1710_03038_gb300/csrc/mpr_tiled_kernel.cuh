@@ -110,6 +110,121 @@ __device__ __forceinline__ float2 gmrf_bond2(float2 phi, float v) {
     return fma2(mul2(d, d), f2(0.050660591821168885f), f2(-1.0f));
 }
 
+// A cell of the table from its pair of angles: (cos q phi_0, cos q phi_1, sin q phi_0,
+// sin q phi_1), then the same of q = 1 for kModelLIT; the angles for kModelGMRF.
+template <int MODEL>
+__device__ __forceinline__ float4 store_cell(unsigned char* t, float q, float2 v) {
+    if (MODEL == kModelGMRF) {
+        *reinterpret_cast<float2*>(t) = v;
+        return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    const float2 qv = mul2(f2(q), v);
+    float s0, c0, s1, c1;
+    __sincosf(qv.x, &s0, &c0);
+    __sincosf(qv.y, &s1, &c1);
+    if (MODEL == kModelLIT) {
+        float u0, w0, u1, w1;
+        __sincosf(v.x, &u0, &w0);
+        __sincosf(v.y, &u1, &w1);
+        reinterpret_cast<float4*>(t)[1] = make_float4(w0, w1, u0, u1);
+    }
+    const float4 cell = make_float4(c0, c1, s0, s1);
+    *reinterpret_cast<float4*>(t) = cell;
+    return cell;
+}
+
+// Energy of the bonds between a gap cell (its table cell, or for kModelGMRF its
+// angles v) and its sample neighbours, added to esum.  (fx, fy): the cell's sample
+// field; slot: its place in the slot arrays.
+template <int MODEL>
+__device__ __forceinline__ float2 add_sample_bonds(const SweepArgs& a, const ImgDev& I, float4 cell,
+                                                   float2 v, float fx, float fy, long long slot,
+                                                   float2 esum) {
+    if (MODEL != kModelGMRF) {
+        const float2 d = fma2(f2(fx), make_float2(cell.x, cell.y),
+                              mul2(f2(fy), make_float2(cell.z, cell.w)));
+        return fma2(f2(-a.J), d, esum);
+    }
+    const uint32_t pos = a.slot_pos[slot];
+    const int X = (int)(pos & 0xFFFFu), Y = (int)(pos >> 16);
+    const float* sp = a.samp + I.site_off + (long long)Y * I.Lx + X;
+    const float vs[4] = {Y > 0 ? sp[-I.Lx] : -1.0f, Y + 1 < I.Ly ? sp[I.Lx] : -1.0f,
+                         X > 0 ? sp[-1] : -1.0f, X + 1 < I.Lx ? sp[1] : -1.0f};
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+        if (vs[m] >= 0.0f) esum = fma2(f2(a.J), gmrf_bond2(v, vs[m]), esum);
+    return esum;
+}
+
+// Alg. 1 at one own site for a pair of chains: the field from the table (tabp: the
+// pair's column; rw: byte offsets of the four neighbours' entries) and the site's
+// constants kk, then the model's update.  slot: the site's place in the slot arrays.
+template <int MODEL, bool ENERGY>
+__device__ __forceinline__ PairOut update_site(const SweepArgs& a, const ImgDev& I,
+                                               const unsigned char* tabp, uint4 rw, uint4 kk,
+                                               float4 f1, float2 vc, const PairRand& u,
+                                               const UpdateConst& uk, float2 alpha_s, float c_acc,
+                                               long long slot) {
+    PairOut o;
+    if (MODEL == kModelGMRF) {
+        const float2 gu = tab_f2(tabp + rw.x), gd = tab_f2(tabp + rw.y);
+        const float2 gl = tab_f2(tabp + rw.z), gr = tab_f2(tabp + rw.w);
+        const float2 sum = add2(add2(add2(add2(f2(__uint_as_float(kk.x)), gu), gd), gl), gr);
+        o = gmrf_pair<false>(vc, sum, __uint_as_float(kk.y), u, a.J, alpha_s, c_acc);
+        if (ENERGY) {
+            // the site's bonds after its update: gap neighbours from the table,
+            // sample neighbours from the sample plane
+            const uint32_t pos = a.slot_pos[slot];
+            const int X = (int)(pos & 0xFFFFu), Y = (int)(pos >> 16);
+            const float* sp = a.samp + I.site_off + (long long)Y * I.Lx + X;
+            const bool hn[4] = {Y > 0, Y + 1 < I.Ly, X > 0, X + 1 < I.Lx};
+            const long long dn[4] = {-(long long)I.Lx, (long long)I.Lx, -1, 1};
+            const float2 gv[4] = {gu, gd, gl, gr};
+            const uint32_t rr[4] = {rw.x, rw.y, rw.z, rw.w};
+            float2 es = f2(0.0f);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                if (!hn[m]) continue;
+                const float vs = sp[dn[m]];
+                if (vs >= 0.0f) es = add2(es, gmrf_bond2(o.phi, vs));
+                else if (rr[m] != 0u) {
+                    const float2 d = add2(o.phi, mul2(gv[m], f2(-1.0f)));
+                    es = add2(es, fma2(mul2(d, d), f2(0.050660591821168885f), f2(-1.0f)));
+                }
+            }
+            o.e = mul2(f2(a.J), es);
+        }
+    } else {
+        const float4 gu = tab_f4(tabp + rw.x), gd = tab_f4(tabp + rw.y);
+        const float4 gl = tab_f4(tabp + rw.z), gr = tab_f4(tabp + rw.w);
+        const float fsx = __uint_as_float(kk.x), fsy = __uint_as_float(kk.y);
+        const float2 C = add2(add2(add2(add2(f2(fsx), make_float2(gu.x, gu.y)),
+                                        make_float2(gd.x, gd.y)),
+                                   make_float2(gl.x, gl.y)),
+                              make_float2(gr.x, gr.y));
+        const float2 S = add2(add2(add2(add2(f2(fsy), make_float2(gu.z, gu.w)),
+                                        make_float2(gd.z, gd.w)),
+                                   make_float2(gl.z, gl.w)),
+                              make_float2(gr.z, gr.w));
+        if (MODEL == kModelLIT) {
+            const float4 hu = tab_f4(tabp + rw.x + 16), hd = tab_f4(tabp + rw.y + 16);
+            const float4 hl = tab_f4(tabp + rw.z + 16), hr = tab_f4(tabp + rw.w + 16);
+            const float2 C1 = add2(add2(add2(add2(f2(f1.x), make_float2(hu.x, hu.y)),
+                                             make_float2(hd.x, hd.y)),
+                                        make_float2(hl.x, hl.y)),
+                                   make_float2(hr.x, hr.y));
+            const float2 S1 = add2(add2(add2(add2(f2(f1.y), make_float2(hu.z, hu.w)),
+                                             make_float2(hd.z, hd.w)),
+                                        make_float2(hl.z, hl.w)),
+                                   make_float2(hr.z, hr.w));
+            o = literal_pair<ENERGY>(vc, C, S, C1, S1, u, uk, alpha_s, c_acc);
+        } else {
+            o = hybrid_pair<ENERGY>(vc, C, S, u, uk, alpha_s, c_acc);
+        }
+    }
+    return o;
+}
+
 template <int TX, int TY, int NW, int P, bool ACC, int MODEL, bool ENERGY, int GROUPS>
 __global__ void __launch_bounds__(NW * 32, 1024 / (NW * 32))  // 64 registers: 32 warps per SM
 tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
@@ -235,33 +350,10 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
 #pragma unroll 4
         for (int e = e_lo; e < n_ent; e += NTP, t += (size_t)NTP * P * CB) {
             const float2 v = *reinterpret_cast<const float2*>(t);
-            if (MODEL != kModelGMRF) {
-                const float2 qv = mul2(f2(a.q), v);
-                float s0, c0, s1, c1;
-                __sincosf(qv.x, &s0, &c0);
-                __sincosf(qv.y, &s1, &c1);
-                if (MODEL == kModelLIT) {
-                    float u0, w0, u1, w1;
-                    __sincosf(v.x, &u0, &w0);
-                    __sincosf(v.y, &u1, &w1);
-                    reinterpret_cast<float4*>(t)[1] = make_float4(w0, w1, u0, u1);
-                }
-                *reinterpret_cast<float4*>(t) = make_float4(c0, c1, s0, s1);
-                if (ENERGY && e < n_oth) {
-                    const float4 f = fcs[e];
-                    const float2 d = fma2(f2(f.x), make_float2(c0, c1), mul2(f2(f.y), make_float2(s0, s1)));
-                    esum = fma2(f2(-a.J), d, esum);
-                }
-            } else if (ENERGY && e < n_oth) {
-                // GMRF: bonds to the sample neighbours from the sample plane
-                const uint32_t pos = a.slot_pos[slot_off + off_oth + e];
-                const int X = (int)(pos & 0xFFFFu), Y = (int)(pos >> 16);
-                const float* sp = a.samp + I.site_off + (long long)Y * I.Lx + X;
-                float vs[4] = {Y > 0 ? sp[-I.Lx] : -1.0f, Y + 1 < I.Ly ? sp[I.Lx] : -1.0f,
-                               X > 0 ? sp[-1] : -1.0f, X + 1 < I.Lx ? sp[1] : -1.0f};
-#pragma unroll
-                for (int m = 0; m < 4; ++m)
-                    if (vs[m] >= 0.0f) esum = fma2(f2(a.J), gmrf_bond2(v, vs[m]), esum);
+            const float4 cell = MODEL == kModelGMRF ? float4{} : store_cell<MODEL>(t, a.q, v);
+            if (ENERGY && e < n_oth) {
+                const float4 f = MODEL == kModelGMRF ? float4{} : fcs[e];
+                esum = add_sample_bonds<MODEL>(a, I, cell, v, f.x, f.y, slot_off + off_oth + e, esum);
             }
         }
     }
@@ -293,64 +385,9 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
         const uint4 rw = own_rows[jj];
         const uint4 kk = own_k[jj];
         const PairRand u = pair_uniforms_flipped(philox_finish(kk.z, kk.w, pair_words, a.rk));
-        PairOut o;
-        if (MODEL == kModelGMRF) {
-            const float2 gu = tab_f2(tabp + rw.x), gd = tab_f2(tabp + rw.y);
-            const float2 gl = tab_f2(tabp + rw.z), gr = tab_f2(tabp + rw.w);
-            const float2 sum = add2(add2(add2(add2(f2(__uint_as_float(kk.x)), gu), gd), gl), gr);
-            o = gmrf_pair<false>(vc, sum, __uint_as_float(kk.y), u, a.J, alpha_s, c_acc);
-            if (ENERGY) {
-                // the site's bonds after its update: gap neighbours from the table,
-                // sample neighbours from the sample plane
-                const uint32_t pos = a.slot_pos[slot_off + off_own + jj];
-                const int X = (int)(pos & 0xFFFFu), Y = (int)(pos >> 16);
-                const float* sp = a.samp + I.site_off + (long long)Y * I.Lx + X;
-                const bool hn[4] = {Y > 0, Y + 1 < I.Ly, X > 0, X + 1 < I.Lx};
-                const long long dn[4] = {-(long long)I.Lx, (long long)I.Lx, -1, 1};
-                const float2 gv[4] = {gu, gd, gl, gr};
-                const uint32_t rr[4] = {rw.x, rw.y, rw.z, rw.w};
-                float2 es = f2(0.0f);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    if (!hn[m]) continue;
-                    const float vs = sp[dn[m]];
-                    if (vs >= 0.0f) es = add2(es, gmrf_bond2(o.phi, vs));
-                    else if (rr[m] != 0u) {
-                        const float2 d = add2(o.phi, mul2(gv[m], f2(-1.0f)));
-                        es = add2(es, fma2(mul2(d, d), f2(0.050660591821168885f), f2(-1.0f)));
-                    }
-                }
-                o.e = mul2(f2(a.J), es);
-            }
-        } else {
-            const float4 gu = tab_f4(tabp + rw.x), gd = tab_f4(tabp + rw.y);
-            const float4 gl = tab_f4(tabp + rw.z), gr = tab_f4(tabp + rw.w);
-            const float fsx = __uint_as_float(kk.x), fsy = __uint_as_float(kk.y);
-            const float2 C = add2(add2(add2(add2(f2(fsx), make_float2(gu.x, gu.y)),
-                                            make_float2(gd.x, gd.y)),
-                                       make_float2(gl.x, gl.y)),
-                                  make_float2(gr.x, gr.y));
-            const float2 S = add2(add2(add2(add2(f2(fsy), make_float2(gu.z, gu.w)),
-                                            make_float2(gd.z, gd.w)),
-                                       make_float2(gl.z, gl.w)),
-                                  make_float2(gr.z, gr.w));
-            if (MODEL == kModelLIT) {
-                const float4 f1 = own_f1[jj];
-                const float4 hu = tab_f4(tabp + rw.x + 16), hd = tab_f4(tabp + rw.y + 16);
-                const float4 hl = tab_f4(tabp + rw.z + 16), hr = tab_f4(tabp + rw.w + 16);
-                const float2 C1 = add2(add2(add2(add2(f2(f1.x), make_float2(hu.x, hu.y)),
-                                                 make_float2(hd.x, hd.y)),
-                                            make_float2(hl.x, hl.y)),
-                                       make_float2(hr.x, hr.y));
-                const float2 S1 = add2(add2(add2(add2(f2(f1.y), make_float2(hu.z, hu.w)),
-                                                 make_float2(hd.z, hd.w)),
-                                            make_float2(hl.z, hl.w)),
-                                       make_float2(hr.z, hr.w));
-                o = literal_pair<ENERGY>(vc, C, S, C1, S1, u, uk, alpha_s, c_acc);
-            } else {
-                o = hybrid_pair<ENERGY>(vc, C, S, u, uk, alpha_s, c_acc);
-            }
-        }
+        const PairOut o = update_site<MODEL, ENERGY>(
+            a, I, tabp, rw, kk, MODEL == kModelLIT ? own_f1[jj] : make_float4(0.0f, 0.0f, 0.0f, 0.0f), vc,
+            u, uk, alpha_s, c_acc, slot_off + off_own + jj);
         const bool act1 = act && has1;
         // a missing second chain is the padding chain of the layout: storing there is harmless
         if (act) *reinterpret_cast<float2*>(sto + j * cpi) = o.phi;

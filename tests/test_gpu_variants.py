@@ -53,3 +53,84 @@ def test_variants_equal_the_plain_path(R, cg, model):
     # the mean of angles rounded to 2^-24 rad, mapped back and rounded to FP32
     for a, b in zip(got[2], want[2]):
         assert np.allclose(a, b, rtol=1e-6, atol=1e-5)
+
+
+# ------------------------------------------------ launches per colour, resident runs
+# Batches whose tiles and chain groups fit the GPU at once run their sweeps in one
+# launch (the tests above); more than about a thousand blocks take a launch per colour.
+
+def big_run(path, R, cg, model="mpr", n=2):
+    z = synthetic.grf((530, 545), nu=0.5, ell=9.0, mean=50, std=10, seed=61).astype(np.float32)
+    g = synthetic.uniform_gaps((530, 545), 0.35, 62).astype(np.uint8)
+    g[100:150, 200:260] = 1  # tiles that are all gap
+    ctx = mpr.Context([z], [g], chains=R, params=mpr.Params(seed=78, path=path, chain_group=cg, model=model))
+    ctx.set_T([0.1])
+    ctx.sweep(n, "equil")
+    ctx.sweep(1, "equil", record_energy=True)
+    ctx.sweep(n, "measure")
+    info = ctx.chain_info()
+    return ctx.get_state()[0], info, ctx.predict()[0]
+
+
+@pytest.mark.parametrize("R,cg,model", [(4, 4, "mpr"), (8, 8, "mpr"), (16, 16, "mpr"), (32, 32, "mpr"),
+                                        (64, 32, "mpr"), (40, 32, "mpr"), (7, 7, "mpr"), (2, 2, "mpr"),
+                                        (16, 16, "gmrf"), (24, 8, "gmrf")])
+def test_launches_per_colour_equal_the_plain_path(R, cg, model):
+    want, got = big_run("plain", R, cg, model), big_run("tiled", R, cg, model)
+    assert torch.equal(got[0], want[0])
+    for k in ("a", "accepted"):
+        assert np.array_equal(got[1][k], want[1][k])
+    assert torch.allclose(got[2], want[2], rtol=1e-6, atol=1e-5)
+
+
+def small_ctx(path, R, seed=5, stream=None):
+    zs, gs = images()
+    ctx = mpr.Context(zs, gs, chains=R, params=mpr.Params(seed=seed, path=path), stream=stream)
+    ctx.set_T([0.2, 0.05, 0.4], stream=stream)
+    return ctx
+
+
+@pytest.mark.parametrize("lengths", [(1, 1, 1, 1, 1, 1), (2, 4), (3, 3), (6,), (5, 1)])
+@pytest.mark.parametrize("phase", ["equil", "measure"])
+def test_resident_runs_join_without_a_seam(lengths, phase):
+    """Six sweeps in runs of any length, states replaced in between by themselves: the
+    plain path's states, acceptances and energies."""
+    out = []
+    for path, parts in (("plain", (6,)), ("tiled", lengths)):
+        ctx = small_ctx(path, 10)
+        ctx.sweep(2, "equil")
+        for n in parts:
+            ctx.set_state(ctx.get_state())
+            ctx.sweep(n, phase, record_energy=True)
+        out.append(([s.cpu().numpy() for s in ctx.get_state()], ctx.chain_info(), ctx.sweep_index()))
+    for a, b in zip(out[0][0], out[1][0]):
+        assert np.array_equal(a, b)
+    assert np.array_equal(out[0][1]["accepted"], out[1][1]["accepted"])
+    assert np.array_equal(out[0][1]["a"], out[1][1]["a"])
+    assert np.allclose(out[0][1]["e_last"], out[1][1]["e_last"], rtol=0, atol=1e-6)
+    assert out[0][2] == out[1][2]
+
+
+def test_resident_runs_in_a_caller_capture_and_on_two_streams():
+    """A captured run replays like a direct one, and contexts on two streams do not
+    disturb each other."""
+    want = []
+    for seed in (5, 6):
+        ctx = small_ctx("tiled", 10, seed)
+        for _ in range(8):
+            ctx.sweep(25, "measure")
+        want.append([s.cpu().numpy() for s in ctx.get_state()])
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    ctxs = [small_ctx("tiled", 10, seed, stream=s) for seed, s in zip((5, 6), streams)]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=streams[0]):
+        ctxs[0].sweep(25, "measure", stream=streams[0])
+    for _ in range(8):
+        with torch.cuda.stream(streams[0]):
+            graph.replay()
+        ctxs[1].sweep(25, "measure", stream=streams[1])
+    torch.cuda.synchronize()
+    for ctx, w in zip(ctxs, want):
+        for a, b in zip(ctx.get_state(), w):
+            assert np.array_equal(a.cpu().numpy(), b)
