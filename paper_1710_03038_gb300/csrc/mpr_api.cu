@@ -552,36 +552,26 @@ __global__ void newton_init_kernel(ImgDev* sub_img, const ImgDev* main_img, doub
 
 // ======================================================= dense views
 
-__device__ __forceinline__ float site_value(const ImgDev& I, const float* state, const float* samp,
-                                            const int* slot_map, int tiled, int chain,
-                                            long long i) {
-    if (tiled) {
-        const int s = slot_map[I.site_off + i];
-        return s >= 0 ? state[state_index(I, chain, s)] : samp[I.site_off + i];
-    }
-    return fabsf(state[state_index(I, chain, i)]);
-}
-
-// H of every (image, chain) (blockIdx.y), FP64 sums of FP32 bond terms.
-__global__ void energy_kernel(const ImgDev* img, const float* state, const float* samp,
-                              const int* slot_map, int tiled, int n_chains, float q, float J,
+// H of every (image, chain) (blockIdx.y) of the plain path, FP64 sums of FP32 bond terms.
+__global__ void energy_kernel(const ImgDev* img, const float* state, int n_chains, float q, float J,
                               int gmrf, double* out) {
     const int ic = blockIdx.y;
     const int im = ic / n_chains, chain = ic - im * n_chains;
     const ImgDev& I = img[im];
+    const float* st = state + state_index(I, chain, 0);
     const long long n = (long long)I.Lx * I.Ly;
     double s = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(i % I.Lx), y = (int)(i / I.Lx);
-        const float v = site_value(I, state, samp, slot_map, tiled, chain, i);
+        const float v = fabsf(st[i]);
         float e = 0.0f;
         if (x + 1 < I.Lx) {
-            const float d = v - site_value(I, state, samp, slot_map, tiled, chain, i + 1);
+            const float d = v - fabsf(st[i + 1]);
             e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
         }
         if (y + 1 < I.Ly) {
-            const float d = v - site_value(I, state, samp, slot_map, tiled, chain, i + I.Lx);
+            const float d = v - fabsf(st[i + I.Lx]);
             e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
         }
         s += (double)e;
@@ -619,27 +609,24 @@ __global__ void state_copy_kernel(const ImgDev* img, float* state, const float* 
     }
 }
 
-// Conditional mean and standard deviation over realisations (Alg. 2 step 6).
+// Conditional mean and standard deviation over realisations (Alg. 2 step 6), plain path.
 __global__ void predict_kernel(const ImgDev* img, const double* acc1, const double* acc2,
-                               const float* zin, const int* slot_map, const float* samp,
-                               int tiled, double n_samples, float* zhat, float* zstd) {
+                               const float* zin, const float* samp, double n_samples, float* zhat,
+                               float* zstd) {
     const ImgDev& I = img[blockIdx.y];
     const long long n = (long long)I.Lx * I.Ly;
     const double range = (double)I.zmax - (double)I.zmin;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const long long s = I.site_off + i;
-        long long slot = -1;
-        if (tiled) slot = slot_map[s];
-        else if (samp[s] < 0.0f) slot = i;
-        if (slot < 0) {
+        if (samp[s] >= 0.0f) {
             zhat[s] = zin[s];
             if (zstd) zstd[s] = 0.0f;
         } else {
-            const double m = acc1[I.slot_off + slot] / n_samples;
+            const double m = acc1[I.slot_off + i] / n_samples;
             zhat[s] = (float)(I.zmin + range * m / (2.0 * kPiD));
             if (zstd) {
-                const double v = fmax(acc2[I.slot_off + slot] / n_samples - m * m, 0.0);
+                const double v = fmax(acc2[I.slot_off + i] / n_samples - m * m, 0.0);
                 zstd[s] = (float)(range * sqrt(v) / (2.0 * kPiD));
             }
         }
@@ -1852,10 +1839,17 @@ mpr_status mpr_energy(mpr_ctx* c, double* e_out, mpr_mem where, mpr_stream strea
     MPR_CUDA(cudaMemsetAsync(d_out, 0, sizeof(double) * nc, s));
     long long maxn = 0;
     for (int i = 0; i < c->g.n_img; ++i) maxn = std::max(maxn, (long long)c->g.Lx[i] * c->g.Ly[i]);
-    energy_kernel<<<dim3(grid_for(maxn, 256, 512), nc), 256, 0, s>>>(
-        c->d_img, c->d_state, c->d_samp, c->d_slot_map, c->g.path == MPR_PATH_TILED ? 1 : 0,
-        c->g.n_chains, (float)c->p.q, (float)c->p.J, c->p.model == MPR_MODEL_GMRF ? 1 : 0, d_out);
-    MPR_CUDA(cudaGetLastError());
+    const int gmrf = c->p.model == MPR_MODEL_GMRF ? 1 : 0;
+    if (c->g.path == MPR_PATH_TILED) {
+        const int most = *std::max_element(c->g.ntiles.begin(), c->g.ntiles.end());
+        MPR_CUDA(launch_energy_tiles(c->d_img, c->d_tiles, c->g.n_img, most, c->g.tx, c->g.ty, c->d_state,
+                                     c->d_samp, c->d_slot_map, c->g.n_chains, (float)c->p.q, (float)c->p.J,
+                                     gmrf, d_out, s));
+    } else {
+        energy_kernel<<<dim3(grid_for(maxn, 256, 512), nc), 256, 0, s>>>(
+            c->d_img, c->d_state, c->g.n_chains, (float)c->p.q, (float)c->p.J, gmrf, d_out);
+        MPR_CUDA(cudaGetLastError());
+    }
     energy_finish_kernel<<<grid_for(nc), 256, 0, s>>>(c->d_img, d_out, c->g.n_chains, nc);
     MPR_CUDA(cudaGetLastError());
     if (where == MPR_HOST) {
@@ -1874,10 +1868,15 @@ mpr_status mpr_predict(mpr_ctx* c, float* z_hat, float* z_std, mpr_mem where, mp
     float* ds = where == MPR_DEVICE ? z_std : (z_std ? c->d_out + N : nullptr);
     long long maxn = 0;
     for (int i = 0; i < c->g.n_img; ++i) maxn = std::max(maxn, (long long)c->g.Lx[i] * c->g.Ly[i]);
-    predict_kernel<<<dim3(grid_for(maxn, 256, 2048), c->g.n_img), 256, 0, s>>>(
-        c->d_img, c->d_acc1, c->d_acc2, c->d_zst, c->d_slot_map, c->d_samp,
-        c->g.path == MPR_PATH_TILED ? 1 : 0, (double)c->n_meas_done * c->g.n_chains, dh, ds);
-    MPR_CUDA(cudaGetLastError());
+    const double n_samples = (double)c->n_meas_done * c->g.n_chains;
+    if (c->g.path == MPR_PATH_TILED) {
+        MPR_CUDA(launch_predict_tiles(c->d_img, c->d_tiles, c->g.n_tiles, c->g.tx, c->g.ty, c->d_slot_pos,
+                                      c->d_acc1, c->d_acc2, c->d_zst, c->d_gst, n_samples, dh, ds, s));
+    } else {
+        predict_kernel<<<dim3(grid_for(maxn, 256, 2048), c->g.n_img), 256, 0, s>>>(
+            c->d_img, c->d_acc1, c->d_acc2, c->d_zst, c->d_samp, n_samples, dh, ds);
+        MPR_CUDA(cudaGetLastError());
+    }
     if (where == MPR_HOST) {
         MPR_CUDA(cudaMemcpyAsync(z_hat, dh, sizeof(float) * N, cudaMemcpyDeviceToHost, s));
         if (z_std) MPR_CUDA(cudaMemcpyAsync(z_std, ds, sizeof(float) * N, cudaMemcpyDeviceToHost, s));
@@ -1948,6 +1947,11 @@ static mpr_status state_copy(mpr_ctx* c, float* phi, mpr_mem where, int dir, cud
     if (where == MPR_DEVICE) {
         long long maxn = 0;
         for (int i = 0; i < c->g.n_img; ++i) maxn = std::max(maxn, (long long)c->g.Lx[i] * c->g.Ly[i]);
+        if (tiled) {
+            MPR_CUDA(launch_state_tiles(c->d_img, c->d_tiles, c->g.n_tiles, c->g.tx, c->g.ty, c->d_slot_pos,
+                                        c->d_samp, c->d_state, c->g.n_chains, phi, dir == 1, s));
+            return MPR_OK;
+        }
         state_copy_kernel<<<dim3(grid_for(maxn, 256, 1024), nc), 256, 0, s>>>(
             c->d_img, c->d_state, c->d_samp, c->d_slot_map, tiled, c->g.n_chains, phi, dir, 0,
             nullptr);

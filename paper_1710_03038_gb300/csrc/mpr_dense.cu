@@ -1,0 +1,232 @@
+// Dense views of the tiled path: prediction, states in and out, energies of the
+// chains.  The state is slot-major with the chains interleaved, so a thread per pixel
+// and chain reads 4 bytes of a 128-byte row at a time; these kernels take one tile
+// per block instead, move whole rows, and turn them in shared memory.
+#include <algorithm>
+
+#include "mpr_device.cuh"
+#include "mpr_internal.h"
+
+namespace mpr {
+
+namespace {
+
+// Conditional mean and standard deviation over realisations (Alg. 2 step 6), a block
+// per tile: the samples by pixel, the gaps by slot, so that every lane of the FP64
+// work is busy.  Bound by the FP64 units (2 lanes per clock and SM): one thread per
+// pixel with FP64 divisions and square root took 1562 us at 4096^2 with 40 % gaps;
+// the divisions are multiplications by 1 / n and 1 / 2 pi here, and the root is one
+// FP64 Newton step from the FP32 estimate (relative error below 1e-13).
+__global__ void __launch_bounds__(128)
+predict_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix,
+                    const uint32_t* __restrict__ slot_pos, const double* __restrict__ acc1,
+                    const double* __restrict__ acc2, const float* __restrict__ zin,
+                    const uint8_t* __restrict__ gap, double inv_n, float* __restrict__ zhat,
+                    float* __restrict__ zstd) {
+    const TileDesc T = tiles[blockIdx.x];
+    const ImgDev& I = img[T.img];
+    const int Lx = I.Lx, Ly = I.Ly;
+    const long long site0 = I.site_off + (long long)T.y0 * Lx + T.x0;
+    for (int i = threadIdx.x; i < npix; i += 128) {
+        const int x = i & ((1 << tx_log) - 1), y = i >> tx_log;
+        if (T.x0 + x >= Lx || T.y0 + y >= Ly) continue;
+        const long long s = site0 + (long long)y * Lx + x;
+        if (gap[s]) continue;
+        zhat[s] = zin[s];
+        if (zstd) zstd[s] = 0.0f;
+    }
+    constexpr double kInvTwoPiD = 0.15915494309189533577;
+    const double per_rad = ((double)I.zmax - (double)I.zmin) * kInvTwoPiD;  // field units per rad
+    const double scale = per_rad * inv_n, zmin = I.zmin;
+    for (int j = threadIdx.x; j < T.cnt[0] + T.cnt[1]; j += 128) {
+        const long long k = T.slot_off + (j < T.cnt[0] ? T.off[0] + j : T.off[1] + j - T.cnt[0]);
+        const uint32_t p = slot_pos[k];
+        const long long s = I.site_off + (long long)(p >> 16) * Lx + (p & 0xFFFFu);
+        const double a = acc1[k];
+        zhat[s] = (float)fma(a, scale, zmin);
+        if (zstd) {
+            const double m = a * inv_n;
+            const double v = fma(-m, m, acc2[k] * inv_n);
+            const float vf = (float)v;
+            float sd = 0.0f;
+            if (vf > 1e30f) {  // (beyond the estimate's range: angles are below 2 pi)
+                sd = (float)(sqrt(v) * per_rad);
+            } else if (vf > 1e-30f) {
+                const double r = (double)rsqrtf(vf), y = v * r;
+                sd = (float)(fma(fma(-y, y, v), 0.5 * r, y) * per_rad);
+            }
+            zstd[s] = sd;
+        }
+    }
+}
+
+// States of 32 chains of a tile <-> dense planes (SET: the gap sites only), through
+// shared memory: rows of 32 chains on one side, rows of the tile on the other
+// (2048^2 x 32 chains out: 1020 us before, a chain at a time).
+template <bool SET>
+__global__ void __launch_bounds__(256)
+state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix,
+                  const uint32_t* __restrict__ slot_pos, const float* __restrict__ samp,
+                  float* __restrict__ state, int n_chains, float* __restrict__ dense) {
+    extern __shared__ float rows[];  // [sites of the tile][33], then the tile's map
+    uint16_t* map = reinterpret_cast<uint16_t*>(rows + npix * 33);  // pixel -> site, 0xFFFF: a sample
+    const TileDesc T = tiles[blockIdx.x];
+    const ImgDev& I = img[T.img];
+    const int Lx = I.Lx, Ly = I.Ly, n = T.cnt[0] + T.cnt[1];
+    const int r0 = blockIdx.y * 32, nr = min(32, n_chains - r0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < npix; i += 256) map[i] = 0xFFFFu;
+    __syncthreads();
+    const auto slot_of = [&](int j) { return j < T.cnt[0] ? T.off[0] + j : T.off[1] + j - T.cnt[0]; };
+    for (int j = threadIdx.x; j < n; j += 256) {
+        const uint32_t p = slot_pos[T.slot_off + slot_of(j)];
+        map[(((int)(p >> 16) - T.y0) << tx_log) + (int)(p & 0xFFFFu) - T.x0] = (uint16_t)j;
+    }
+    float* st = state + T.state_off + r0 + lane;
+    if (!SET && lane < nr) {
+#pragma unroll 4
+        for (int j = warp; j < n; j += 8) rows[j * 33 + lane] = st[(long long)slot_of(j) * T.cp];
+    }
+    __syncthreads();
+    const long long plane = (long long)Lx * Ly;
+    float* d0 = dense + I.site_off * n_chains + r0 * plane;
+    for (int i = threadIdx.x; i < npix; i += 256) {
+        const int x = T.x0 + (i & ((1 << tx_log) - 1)), y = T.y0 + (i >> tx_log);
+        if (x >= Lx || y >= Ly) continue;
+        const long long site = (long long)y * Lx + x;
+        const int m = map[i];
+        float* d = d0 + site;
+        if (SET) {
+            if (m == 0xFFFF) continue;
+            float* row = rows + m * 33;
+#pragma unroll 8
+            for (int r = 0; r < nr; ++r, d += plane) row[r] = *d;
+        } else if (m == 0xFFFF) {
+            const float v = samp[I.site_off + site];
+            for (int r = 0; r < nr; ++r, d += plane) *d = v;
+        } else {
+            const float* row = rows + m * 33;
+#pragma unroll 8
+            for (int r = 0; r < nr; ++r, d += plane) *d = row[r];
+        }
+    }
+    if (SET) {
+        __syncthreads();
+        if (lane < nr)
+            for (int j = warp; j < n; j += 8) st[(long long)slot_of(j) * T.cp] = rows[j * 33 + lane];
+    }
+}
+
+// H of 32 chains of an image (blockIdx.y, z): a lane is a chain, a block walks tiles.
+// The tile's angles and those right of and below it lie in shared memory, a row of 32
+// chains per pixel.  FP32 bond terms as before; their sum in two FP32 words (TwoSum,
+// Knuth: the rounding error of every addition is kept), FP64 from there: an FP64
+// addition per pixel and chain ran at 1/32 of the rate (1000 x 777 x 24: 177 us before).
+__global__ void __launch_bounds__(256)
+energy_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int ty, const float* state,
+                   const float* samp, const int* slot_map, int n_chains, float q, float J, int gmrf,
+                   double* out) {
+    extern __shared__ float ang[];  // [(ty + 1) x (tx + 1)][32]
+    __shared__ double part[8][32];
+    const ImgDev& I = img[blockIdx.z];
+    const int Lx = I.Lx, Ly = I.Ly, tx = 1 << tx_log, ew = tx + 1;
+    const int r0 = blockIdx.y * 32, nr = min(32, n_chains - r0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r = min(lane, nr - 1);  // idle lanes repeat the last chain
+    double sum = 0.0;
+    for (int t = blockIdx.x; t < I.ntiles; t += gridDim.x) {
+        const TileDesc& T = tiles[I.tile0 + t];
+        const int w = min(ew, Lx - T.x0), h = min(ty + 1, Ly - T.y0);  // with the neighbours that exist
+        __syncthreads();
+        for (int y = warp; y < h; y += 8) {
+            const long long s0 = I.site_off + (long long)(T.y0 + y) * Lx + T.x0;
+#pragma unroll 4
+            for (int x = 0; x < w; ++x) {
+                const int s = slot_map[s0 + x];
+                ang[(y * ew + x) * 32 + lane] = s >= 0 ? state[I.state_off + (long long)s * I.sstride + r0 + r]
+                                                       : samp[s0 + x];
+            }
+        }
+        __syncthreads();
+        const int wi = min(tx, Lx - T.x0), hn = min(ty, Ly - T.y0);
+        float hi = 0.0f, lo = 0.0f;
+        for (int y = warp; y < hn; y += 8) {
+            const float* a = ang + y * ew * 32 + lane;
+            float v = a[0];
+            for (int x = 0; x < wi; ++x) {
+                float e = 0.0f, right = 0.0f;
+                if (x + 1 < w) {
+                    right = a[(x + 1) * 32];
+                    const float d = v - right;
+                    e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
+                }
+                if (y + 1 < h) {
+                    const float d = v - a[(ew + x) * 32];
+                    e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
+                }
+                two_sum(hi, lo, e);
+                v = right;
+            }
+        }
+        sum += two_sum_value(hi, lo);
+    }
+    part[warp][lane] = sum;
+    __syncthreads();
+    if (warp == 0 && lane < nr) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += part[k][lane];
+        atomicAdd(out + (long long)blockIdx.z * n_chains + r0 + lane, s);
+    }
+}
+
+int log2_of(int v) {
+    int l = 0;
+    while ((1 << l) < v) ++l;
+    return l;
+}
+
+}  // namespace
+
+cudaError_t launch_predict_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tx, int ty,
+                                 const uint32_t* slot_pos, const double* acc1, const double* acc2,
+                                 const float* z, const uint8_t* gap, double n_samples, float* zhat,
+                                 float* zstd, cudaStream_t s) {
+    predict_tile_kernel<<<n_tiles, 128, 0, s>>>(img, tiles, log2_of(tx), tx * ty, slot_pos, acc1, acc2, z,
+                                                gap, 1.0 / n_samples, zhat, zstd);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tx, int ty,
+                               const uint32_t* slot_pos, const float* samp, float* state, int n_chains,
+                               float* dense, bool set, cudaStream_t s) {
+    const size_t smem = (size_t)tx * ty * (33 * sizeof(float) + sizeof(uint16_t));
+    const auto kernel = set ? state_tile_kernel<true> : state_tile_kernel<false>;
+    if (smem > 48 * 1024) {  // 32 x 16 and 32 x 32 tiles
+        const cudaError_t e =
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    kernel<<<dim3(n_tiles, (n_chains + 31) / 32), 256, smem, s>>>(img, tiles, log2_of(tx), tx * ty, slot_pos,
+                                                                  samp, state, n_chains, dense);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles, int tx,
+                                int ty, const float* state, const float* samp, const int* slot_map,
+                                int n_chains, float q, float J, int gmrf, double* out, cudaStream_t s) {
+    const size_t smem = (size_t)(tx + 1) * (ty + 1) * 32 * sizeof(float);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            energy_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    // about eight blocks per SM over all images and chain groups
+    const int groups = (n_chains + 31) / 32;
+    const int blocks = std::max(1, std::min(max_tiles, 152 * 8 / std::max(1, groups * n_img) + 1));
+    energy_tile_kernel<<<dim3(blocks, groups, n_img), 256, smem, s>>>(
+        img, tiles, log2_of(tx), ty, state, samp, slot_map, n_chains, q, J, gmrf, out);
+    return cudaGetLastError();
+}
+
+}  // namespace mpr

@@ -351,6 +351,17 @@ __device__ __forceinline__ float gmrf_bond(float d) {
 }
 
 // --------------------------------------------------------- reductions
+// (hi, lo) += e without loss: hi takes the rounded sum, lo its rounding error (TwoSum,
+// Knuth, The Art of Computer Programming 2, 4.2.2).
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float e) {
+    const float s = __fadd_rn(hi, e), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(e, b)));
+    hi = s;
+}
+// the pair's value (an infinite or undefined sum has no rounding error)
+__device__ __forceinline__ double two_sum_value(float hi, float lo) {
+    return (double)hi + (fabsf(hi) <= 3.402823466e38f ? (double)lo : 0.0);
+}
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

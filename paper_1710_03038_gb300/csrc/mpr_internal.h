@@ -148,6 +148,19 @@ int tiled_pairs(int chain_group);
 // blocks of the colour pass one SM holds by their threads and registers
 int tiled_blocks_per_sm(int tx, int ty);
 
+// dense views of the tiled path (mpr_dense.cu)
+cudaError_t launch_predict_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tile_x,
+                                 int tile_y, const uint32_t* slot_pos, const double* acc1,
+                                 const double* acc2, const float* z, const uint8_t* gap,
+                                 double n_samples, float* zhat, float* zstd, cudaStream_t s);
+cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tile_x,
+                               int tile_y, const uint32_t* slot_pos, const float* samp, float* state,
+                               int n_chains, float* dense, bool set, cudaStream_t s);
+cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles,
+                                int tile_x, int tile_y, const float* state, const float* samp,
+                                const int* slot_map, int n_chains, float q, float J, int gmrf,
+                                double* out, cudaStream_t s);
+
 // float offset of gap slot k (tiled) or site k (plain) of a realisation
 __host__ __device__ inline long long state_index(const ImgDev& I, int chain, long long k) {
     return I.state_off + (long long)chain * I.stride + k * I.sstride;

@@ -98,59 +98,84 @@ __global__ void noalloc_extremes_kernel(const __grid_constant__ Shapes S, const 
     }
 }
 
-// Phase 2: per image, combine the partials in a fixed order.
-__global__ void noalloc_extremes_final_kernel(const Partial* part, ImgStat* stat) {
-    if (threadIdx.x != 0) return;
-    const int im = blockIdx.x;
-    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-    unsigned long long cnt = 0;
-    for (int b = 0; b < kNoAllocBlocks; ++b) {
-        const Partial& p = part[im * kNoAllocBlocks + b];
-        lo = min(lo, p.zlo);
-        hi = max(hi, p.zhi);
-        cnt += p.n_gap;
-    }
-    stat[im].zmin = lo == 0xFFFFFFFFu ? __int_as_float(0x7FC00000) : unordered_f(lo);
-    stat[im].zmax = lo == 0xFFFFFFFFu ? __int_as_float(0x7FC00000) : unordered_f(hi);
-    stat[im].n_gap = cnt;
-}
+// Phase 2: sample-sample bond sums with the angles of Eq. map computed on the fly
+// exactly as the context's initialisation computes them (FP64 map, rounded to FP32
+// once; FP32 bond terms -J cos(q (v - w)), their sum in two FP32 words per thread and
+// FP64 from there).  A thread walks kRows rows of a column, so that a pixel is mapped
+// once: the one below is the next row's own, the one on the right comes from the next
+// lane.  Mapping both neighbours again for every pixel took 48 us for two images of 433^2
+// and 694^2, most of it FP64.  Every block first combines the image's extremes (all
+// blocks get the same bits).
+constexpr int kRows = 16, kCols = 128;
 
-// Phase 3: sample-sample bond sums with the angles of Eq. map computed on the
-// fly exactly as the context's initialisation computes them (FP64 map,
-// rounded to FP32 once; FP32 bond terms -J cos(q (v - w)) summed in FP64).
-__global__ void noalloc_pairs_kernel(const __grid_constant__ Shapes S, const float* z,
-                                     const uint8_t* gap, const ImgStat* stat, double q, double J,
-                                     Partial* part) {
-    __shared__ double shd[32];
+__global__ void __launch_bounds__(kCols)
+noalloc_pairs_kernel(const __grid_constant__ Shapes S, const float* __restrict__ z,
+                     const uint8_t* __restrict__ gap, ImgStat* stat, float q, float J, Partial* part) {
     __shared__ unsigned long long shu[32];
+    __shared__ double shd[32];
+    __shared__ ImgStat st;
     const int im = blockIdx.y;
+    uint32_t plo = 0xFFFFFFFFu, phi = 0u;
+    unsigned long long pgap = 0;
+    for (int b = threadIdx.x; b < kNoAllocBlocks; b += kCols) {
+        const Partial& p = part[im * kNoAllocBlocks + b];
+        plo = min(plo, p.zlo);
+        phi = max(phi, p.zhi);
+        pgap += p.n_gap;
+    }
+    auto mn = [](unsigned long long a, unsigned long long b) { return a < b ? a : b; };
+    auto mx = [](unsigned long long a, unsigned long long b) { return a > b ? a : b; };
+    auto add_u = [](unsigned long long a, unsigned long long b) { return a + b; };
+    auto add_d = [](double a, double b) { return a + b; };
+    const unsigned long long rlo = block_reduce<unsigned long long>(plo, mn, shu, 0xFFFFFFFFull);
+    const unsigned long long rhi = block_reduce<unsigned long long>(phi, mx, shu, 0ull);
+    const unsigned long long rg = block_reduce<unsigned long long>(pgap, add_u, shu, 0ull);
+    if (threadIdx.x == 0) {
+        st.zmin = rlo == 0xFFFFFFFFull ? __int_as_float(0x7FC00000) : unordered_f((uint32_t)rlo);
+        st.zmax = rlo == 0xFFFFFFFFull ? __int_as_float(0x7FC00000) : unordered_f((uint32_t)rhi);
+        st.n_gap = rg;
+        if (blockIdx.x == 0) stat[im] = st;
+    }
+    __syncthreads();
     const int Lx = S.Lx[im], Ly = S.Ly[im];
-    const long long n = (long long)Lx * Ly;
-    const float* zi = z + S.off[im];
-    const uint8_t* gi = gap + S.off[im];
-    const double zmin = stat[im].zmin;
-    const double scale = 2.0 * kPiD / ((double)stat[im].zmax - zmin);
-    const bool ok = stat[im].zmax > stat[im].zmin;
+    const double zmin = st.zmin;
+    const double scale = 2.0 * kPiD / ((double)st.zmax - zmin);
+    const int nx = (Lx + kCols - 1) / kCols, tasks = nx * ((Ly + kRows - 1) / kRows);
     double s = 0.0;
     unsigned long long cnt = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; ok && i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        if (gi[i]) continue;
-        const int x = (int)(i % Lx), y = (int)(i / Lx);
-        const float v = (float)(((double)zi[i] - zmin) * scale);
-        if (x + 1 < Lx && !gi[i + 1]) {
-            const float w = (float)(((double)zi[i + 1] - zmin) * scale);
-            s -= (double)((float)J * cosf((float)q * (v - w)));
-            ++cnt;
+    for (int task = blockIdx.x; st.zmax > st.zmin && task < tasks; task += gridDim.x) {
+        const int x = (task % nx) * kCols + threadIdx.x, y0 = task / nx * kRows;
+        const bool in = x < Lx, in_right = x + 1 < Lx;
+        const long long o = S.off[im] + (long long)y0 * Lx + x;
+        const int rows = min(kRows, Ly - y0);
+        float hi = 0.0f, lo = 0.0f;
+        bool ok = in && !gap[o];
+        float v = ok ? (float)(((double)z[o] - zmin) * scale) : 0.0f;
+#pragma unroll 2
+        for (int k = 0; k < rows; ++k) {
+            const long long i = o + (long long)k * Lx;
+            // the pixel on the right (the next lane's own) and the one below
+            float right = __shfl_down_sync(0xffffffffu, v, 1);
+            bool ok_right = __shfl_down_sync(0xffffffffu, (int)ok, 1);
+            if ((threadIdx.x & 31) == 31) {
+                ok_right = in_right && !gap[i + 1];
+                if (ok_right) right = (float)(((double)z[i + 1] - zmin) * scale);
+            }
+            const bool ok_below = in && y0 + k + 1 < Ly && !gap[i + Lx];
+            const float below = ok_below ? (float)(((double)z[i + Lx] - zmin) * scale) : 0.0f;
+            if (ok && ok_right) {
+                two_sum(hi, lo, -(J * cosf(q * (v - right))));
+                ++cnt;
+            }
+            if (ok && ok_below) {
+                two_sum(hi, lo, -(J * cosf(q * (v - below))));
+                ++cnt;
+            }
+            v = below;
+            ok = ok_below;
         }
-        if (y + 1 < Ly && !gi[i + Lx]) {
-            const float w = (float)(((double)zi[i + Lx] - zmin) * scale);
-            s -= (double)((float)J * cosf((float)q * (v - w)));
-            ++cnt;
-        }
+        s += two_sum_value(hi, lo);
     }
-    auto add_d = [](double a, double b) { return a + b; };
-    auto add_u = [](unsigned long long a, unsigned long long b) { return a + b; };
     const double rs = block_reduce<double>(s, add_d, shd, 0.0);
     const unsigned long long rc = block_reduce<unsigned long long>(cnt, add_u, shu, 0ull);
     if (threadIdx.x == 0) {
@@ -160,16 +185,20 @@ __global__ void noalloc_pairs_kernel(const __grid_constant__ Shapes S, const flo
     }
 }
 
-__global__ void noalloc_final_kernel(const Partial* part, const ImgStat* stat, double* e_s,
-                                     long long* n_sp, float* zmin, float* zmax) {
-    if (threadIdx.x != 0) return;
+// Phase 3: per image, combine the partials in a fixed order (one thread per partial: a
+// loop of one thread over them took 22 us).
+__global__ void __launch_bounds__(kNoAllocBlocks)
+noalloc_final_kernel(const Partial* part, const ImgStat* stat, double* e_s, long long* n_sp, float* zmin,
+                     float* zmax) {
+    __shared__ unsigned long long shu[32];
+    __shared__ double shd[32];
     const int im = blockIdx.x;
-    double s = 0.0;
-    unsigned long long c = 0;
-    for (int b = 0; b < kNoAllocBlocks; ++b) {
-        s += part[im * kNoAllocBlocks + b].sum;
-        c += part[im * kNoAllocBlocks + b].n_pair;
-    }
+    const Partial& p = part[im * kNoAllocBlocks + threadIdx.x];
+    auto add_u = [](unsigned long long a, unsigned long long b) { return a + b; };
+    auto add_d = [](double a, double b) { return a + b; };
+    const double s = block_reduce<double>(p.sum, add_d, shd, 0.0);
+    const unsigned long long c = block_reduce<unsigned long long>(p.n_pair, add_u, shu, 0ull);
+    if (threadIdx.x != 0) return;
     const bool ok = stat[im].zmax > stat[im].zmin;
     e_s[im] = (ok && c > 0) ? s / (double)c : __longlong_as_double(0x7FF8000000000000LL);
     if (n_sp) n_sp[im] = ok ? (long long)c : 0;
@@ -232,9 +261,8 @@ extern "C" mpr_status mpr_sample_energy_noalloc(int n_img, const int* Lx, const 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     dim3 grid(kNoAllocBlocks, n_img);
     noalloc_extremes_kernel<<<grid, 256, 0, s>>>(S, z, gap, part);
-    noalloc_extremes_final_kernel<<<n_img, 32, 0, s>>>(part, stat);
-    noalloc_pairs_kernel<<<grid, 256, 0, s>>>(S, z, gap, stat, q, J, part);
-    noalloc_final_kernel<<<n_img, 32, 0, s>>>(part, stat, e_s, reinterpret_cast<long long*>(n_sp),
+    noalloc_pairs_kernel<<<grid, kCols, 0, s>>>(S, z, gap, stat, (float)q, (float)J, part);
+    noalloc_final_kernel<<<n_img, kNoAllocBlocks, 0, s>>>(part, stat, e_s, reinterpret_cast<long long*>(n_sp),
                                               z_min, z_max);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
