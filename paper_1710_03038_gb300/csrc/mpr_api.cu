@@ -221,6 +221,7 @@ struct mpr_ctx {
     // tiled: tiles whose table fits the shared memory of a full SM of blocks run
     // in one launch (gt_light entries), the rest in a second one (gt entries)
     int gt_light[2] = {1, 1};
+    int n_cap[2] = {1, 1}, n_cap_light[2] = {1, 1};  // own sites of the largest tile of either launch
     int n_light[2] = {0, 0};
     uint32_t sweep = 0, equil_index = 0;
     long long n_meas_done = 0;
@@ -806,14 +807,19 @@ mpr_status split_tiles(mpr_ctx* c, const std::vector<TileDesc>& tiles, cudaStrea
     std::vector<int> list(2 * (size_t)n);
     bool split = false;
     for (int col = 0; col < 2; ++col) {
-        int gmax = 1, glight = 1, nl = 0;
+        // light: the largest set of tiles, by table entries and own sites, whose common
+        // block size keeps the blocks per SM (the own sites' records are sized for the
+        // light tile with the most)
+        int gmax = 1, cmax = 1, glight = 1, clight = 1, nl = 0;
         std::vector<int> heavy;
         for (int t = 0; t < n; ++t) {
-            const int e = tiles[t].cnt[col ^ 1] + tiles[t].halo_cnt[col] + 1;
+            const int e = tiles[t].cnt[col ^ 1] + tiles[t].halo_cnt[col] + 1, own = tiles[t].cnt[col];
             gmax = std::max(gmax, e);
-            if (tiled_pass_smem(g.tx, g.ty, e, cg, flags) <= budget) {
+            cmax = std::max(cmax, own);
+            if (tiled_pass_smem(g.tx, g.ty, std::max(e, glight), std::max(own, clight), cg, flags) <= budget) {
                 list[(size_t)col * n + nl++] = t;
                 glight = std::max(glight, e);
+                clight = std::max(clight, own);
             } else {
                 heavy.push_back(t);
             }
@@ -821,6 +827,8 @@ mpr_status split_tiles(mpr_ctx* c, const std::vector<TileDesc>& tiles, cudaStrea
         for (size_t k = 0; k < heavy.size(); ++k) list[(size_t)col * n + nl + k] = heavy[k];
         c->gt[col] = gmax;
         c->gt_light[col] = glight;
+        c->n_cap[col] = cmax;
+        c->n_cap_light[col] = clight;
         c->n_light[col] = nl;
         split = split || nl < n;
     }
@@ -1259,12 +1267,14 @@ mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bo
                     a.tile_base = 0;
                     a.n_list = nl;
                     a.gt = nl < nt ? c->gt_light[colour] : c->gt[colour];
+                    a.n_cap = nl < nt ? c->n_cap_light[colour] : c->n_cap[colour];
                     e = launch_tiled_pass(a, c->g.tx, c->g.ty, s);
                 }
                 if (e == cudaSuccess && nl < nt) {
                     a.tile_base = nl;
                     a.n_list = nt - nl;
                     a.gt = c->gt[colour];
+                    a.n_cap = c->n_cap[colour];
                     e = launch_tiled_pass(a, c->g.tx, c->g.ty, s2);
                 }
                 if (e == cudaSuccess && n_cr > 1) {  // the remaining chains, every tile
@@ -1275,6 +1285,7 @@ mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bo
                     a.tile_base = 0;
                     a.n_list = nt;
                     a.gt = c->gt[colour];
+                    a.n_cap = c->n_cap[colour];
                     e = launch_tiled_pass(a, c->g.tx, c->g.ty, s2);
                 }
                 if (fork && e == cudaSuccess) {

@@ -106,6 +106,7 @@ struct SweepArgs {
     int flags;
     int halo_cap;
     int gt;                    // tiled: table entries per chain pair for this pass (largest tile)
+    int n_cap;                 // tiled: own sites of the tile with the most
     const int* tile_list;      // tiled: k-th tile of the launch is tile_list[tile_base + k] (null: k)
     int tile_base;
     int n_list;                // tiled: tiles in the launch
@@ -140,9 +141,9 @@ cudaError_t launch_tile_const(const ImgDev* img, const TileDesc* tiles, int n_ti
                               const float* samp, float q, int gmrf, uint2* slot_ref,
                               float4* slot_cs, cudaStream_t s);
 // Dynamic shared memory of a colour-pass block of tile shape tx x ty for a
-// launch whose largest tile has gt table entries; flags: the model bits of
+// launch whose largest tiles have gt table entries and n_cap own sites; flags: the model bits of
 // SweepFlags (kLiteralOR, kGMRF).
-size_t tiled_pass_smem(int tx, int ty, int gt, int chain_group, int flags);
+size_t tiled_pass_smem(int tx, int ty, int gt, int n_cap, int chain_group, int flags);
 // Chain pairs per site of a colour-pass block for a group of that many chains.
 int tiled_pairs(int chain_group);
 // blocks of the colour pass one SM holds by their threads and registers

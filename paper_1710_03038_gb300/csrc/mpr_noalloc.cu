@@ -101,14 +101,14 @@ __global__ void noalloc_extremes_kernel(const __grid_constant__ Shapes S, const 
 // Phase 2: sample-sample bond sums with the angles of Eq. map computed on the fly
 // exactly as the context's initialisation computes them (FP64 map, rounded to FP32
 // once; FP32 bond terms -J cos(q (v - w)), their sum in two FP32 words per thread and
-// FP64 from there).  A thread walks kRows rows of a column, so that a pixel is mapped
-// once: the one below is the next row's own, the one on the right comes from the next
-// lane.  Mapping both neighbours again for every pixel took 48 us for two images of 433^2
-// and 694^2, most of it FP64.  Every block first combines the image's extremes (all
-// blocks get the same bits).
-constexpr int kRows = 16, kCols = 128;
+// FP64 from there).  A warp takes 31 columns and kRows rows: each lane maps its pixels
+// once, the pixel below is the next row's own, the one on the right the next lane's (the
+// last lane only maps).  Mapping both neighbours again for every pixel took 48 us for two
+// images of 433^2 and 694^2, most of it FP64.  Every block first combines the image's
+// extremes (all blocks get the same bits).
+constexpr int kRows = 8, kPairThreads = 256;
 
-__global__ void __launch_bounds__(kCols)
+__global__ void __launch_bounds__(kPairThreads)
 noalloc_pairs_kernel(const __grid_constant__ Shapes S, const float* __restrict__ z,
                      const uint8_t* __restrict__ gap, ImgStat* stat, float q, float J, Partial* part) {
     __shared__ unsigned long long shu[32];
@@ -117,7 +117,7 @@ noalloc_pairs_kernel(const __grid_constant__ Shapes S, const float* __restrict__
     const int im = blockIdx.y;
     uint32_t plo = 0xFFFFFFFFu, phi = 0u;
     unsigned long long pgap = 0;
-    for (int b = threadIdx.x; b < kNoAllocBlocks; b += kCols) {
+    for (int b = threadIdx.x; b < kNoAllocBlocks; b += kPairThreads) {
         const Partial& p = part[im * kNoAllocBlocks + b];
         plo = min(plo, p.zlo);
         phi = max(phi, p.zhi);
@@ -140,34 +140,31 @@ noalloc_pairs_kernel(const __grid_constant__ Shapes S, const float* __restrict__
     const int Lx = S.Lx[im], Ly = S.Ly[im];
     const double zmin = st.zmin;
     const double scale = 2.0 * kPiD / ((double)st.zmax - zmin);
-    const int nx = (Lx + kCols - 1) / kCols, tasks = nx * ((Ly + kRows - 1) / kRows);
+    const int lane = threadIdx.x & 31, warps = kPairThreads / 32;
+    const int nx = (Lx + 30) / 31, tasks = nx * ((Ly + kRows - 1) / kRows);
     double s = 0.0;
     unsigned long long cnt = 0;
-    for (int task = blockIdx.x; st.zmax > st.zmin && task < tasks; task += gridDim.x) {
-        const int x = (task % nx) * kCols + threadIdx.x, y0 = task / nx * kRows;
-        const bool in = x < Lx, in_right = x + 1 < Lx;
+    for (int task = blockIdx.x * warps + (threadIdx.x >> 5); st.zmax > st.zmin && task < tasks;
+         task += gridDim.x * warps) {
+        const int x = task % nx * 31 + lane, y0 = task / nx * kRows;
+        const bool in = x < Lx, own = in && lane < 31;
         const long long o = S.off[im] + (long long)y0 * Lx + x;
         const int rows = min(kRows, Ly - y0);
         float hi = 0.0f, lo = 0.0f;
         bool ok = in && !gap[o];
         float v = ok ? (float)(((double)z[o] - zmin) * scale) : 0.0f;
-#pragma unroll 2
+#pragma unroll 4
         for (int k = 0; k < rows; ++k) {
             const long long i = o + (long long)k * Lx;
-            // the pixel on the right (the next lane's own) and the one below
-            float right = __shfl_down_sync(0xffffffffu, v, 1);
-            bool ok_right = __shfl_down_sync(0xffffffffu, (int)ok, 1);
-            if ((threadIdx.x & 31) == 31) {
-                ok_right = in_right && !gap[i + 1];
-                if (ok_right) right = (float)(((double)z[i + 1] - zmin) * scale);
-            }
             const bool ok_below = in && y0 + k + 1 < Ly && !gap[i + Lx];
             const float below = ok_below ? (float)(((double)z[i + Lx] - zmin) * scale) : 0.0f;
-            if (ok && ok_right) {
+            const float right = __shfl_down_sync(0xffffffffu, v, 1);
+            const bool ok_right = __shfl_down_sync(0xffffffffu, (int)ok, 1);
+            if (own && ok && ok_right) {
                 two_sum(hi, lo, -(J * cosf(q * (v - right))));
                 ++cnt;
             }
-            if (ok && ok_below) {
+            if (own && ok && ok_below) {
                 two_sum(hi, lo, -(J * cosf(q * (v - below))));
                 ++cnt;
             }
@@ -261,7 +258,7 @@ extern "C" mpr_status mpr_sample_energy_noalloc(int n_img, const int* Lx, const 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     dim3 grid(kNoAllocBlocks, n_img);
     noalloc_extremes_kernel<<<grid, 256, 0, s>>>(S, z, gap, part);
-    noalloc_pairs_kernel<<<grid, kCols, 0, s>>>(S, z, gap, stat, (float)q, (float)J, part);
+    noalloc_pairs_kernel<<<grid, kPairThreads, 0, s>>>(S, z, gap, stat, (float)q, (float)J, part);
     noalloc_final_kernel<<<n_img, kNoAllocBlocks, 0, s>>>(part, stat, e_s, reinterpret_cast<long long*>(n_sp),
                                               z_min, z_max);
     const cudaError_t e = cudaGetLastError();

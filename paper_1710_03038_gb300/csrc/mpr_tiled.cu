@@ -186,14 +186,14 @@ __global__ void tile_const_kernel(const ImgDev* img, const TileDesc* tiles, int 
 
 }  // namespace
 
-size_t tiled_pass_smem(int tx, int ty, int gt, int chain_group, int flags) {
+size_t tiled_pass_smem(int tx, int ty, int gt, int n_cap, int chain_group, int flags) {
     using namespace tiled;
     const int P = pairs_for_group(chain_group);
-    if (flags & kGMRF) return Cfg<16, 16, 4, kModelGMRF>::smem_for(gt, P);
-    if (flags & kLiteralOR) return Cfg<16, 16, 4, kModelLIT>::smem_for(gt, P);
-    if (tx == 32 && ty == 16) return Cfg<32, 16, 8, kModelMPR>::smem_for(gt, P);
-    if (tx == 32 && ty == 32) return Cfg<32, 32, 8, kModelMPR>::smem_for(gt, P);
-    return Cfg<16, 16, 4, kModelMPR>::smem_for(gt, P);
+    if (flags & kGMRF) return Cfg<16, 16, 4, kModelGMRF>::smem_for(gt, n_cap, P);
+    if (flags & kLiteralOR) return Cfg<16, 16, 4, kModelLIT>::smem_for(gt, n_cap, P);
+    if (tx == 32 && ty == 16) return Cfg<32, 16, 8, kModelMPR>::smem_for(gt, n_cap, P);
+    if (tx == 32 && ty == 32) return Cfg<32, 32, 8, kModelMPR>::smem_for(gt, n_cap, P);
+    return Cfg<16, 16, 4, kModelMPR>::smem_for(gt, n_cap, P);
 }
 
 int tiled_pairs(int chain_group) { return tiled::pairs_for_group(chain_group); }

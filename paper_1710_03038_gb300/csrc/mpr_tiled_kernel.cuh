@@ -78,23 +78,22 @@ struct Cfg {
     static constexpr int HCAP = TX + TY;           // ring cells of one colour
     static constexpr int GT = NMAX + HCAP + 1;     // table entries (entry 0 = zeros)
     static constexpr size_t a16(size_t v) { return (v + 15) / 16 * 16; }
-    // per own site: byte offsets of the four neighbour entries
-    static constexpr size_t off_rows = 0;
-    // per own site: sample field (x, y), random-stream words
-    static constexpr size_t off_k = off_rows + sizeof(uint4) * NMAX;
-    // per own site (kModelLIT): the q = 1 sample field
-    static constexpr size_t off_f1 = off_k + sizeof(uint4) * NMAX;
-    static constexpr size_t off_red = off_f1 + (MODEL == kModelLIT ? sizeof(float4) * NMAX : 0);
-    // the table last, sized at launch for the largest tile of the pass
-    // the per-chain reduction area; sampling passes first keep the own sites'
-    // fixed-point realisation sums there (two words per site)
-    static constexpr size_t red_bytes =
-        sizeof(float4) * NW * 16 > 8 * NMAX ? sizeof(float4) * NW * 16 : 8 * NMAX;
-    static constexpr size_t off_tab = off_red + red_bytes;
-    static constexpr size_t smem_for(int gt, int P) {
-        return off_tab + (size_t)Cell<MODEL>::bytes * P * gt;
+    // Own sites' records, sized at launch for the tile with the most (n_cap sites): the
+    // byte offsets of the four neighbour entries, then the sample field (x, y) and the
+    // random-stream words, then (kModelLIT) the q = 1 sample field
+    static constexpr size_t own_bytes(int n_cap) {
+        return sizeof(uint4) * (MODEL == kModelLIT ? 3 : 2) * (size_t)n_cap;
     }
-    static constexpr size_t smem_max = smem_for(GT, 16);
+    // the per-chain reduction area and, in sampling passes, the own sites' fixed-point
+    // realisation sums (two words per site); apart, so that one barrier ends both (three
+    // before: 0.2880 -> 0.2818 ms per sampling sweep at 2048^2 x 32)
+    static constexpr size_t red_bytes = sizeof(float4) * NW * 16;
+    static constexpr size_t sum_bytes(int n_cap) { return a16(8 * (size_t)n_cap); }
+    // the table last, sized at launch for the largest tile of the pass
+    static constexpr size_t smem_for(int gt, int n_cap, int P) {
+        return red_bytes + sum_bytes(n_cap) + own_bytes(n_cap) + (size_t)Cell<MODEL>::bytes * P * gt;
+    }
+    static constexpr size_t smem_max = smem_for(GT, NMAX, 16);
 };
 
 __device__ __forceinline__ float4 tab_f4(const unsigned char* p) {
@@ -234,15 +233,15 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     constexpr int CB = Cell<MODEL>::bytes;
     static_assert(P >= 1 && P <= 16 && (P & (P - 1)) == 0, "pairs per site: power of two");
     extern __shared__ __align__(16) unsigned char smem[];
-    uint4* own_rows = reinterpret_cast<uint4*>(smem + Cf::off_rows);
-    uint4* own_k = reinterpret_cast<uint4*>(smem + Cf::off_k);
-    float4* own_f1 = reinterpret_cast<float4*>(smem + Cf::off_f1);
-    float4* red = reinterpret_cast<float4*>(smem + Cf::off_red);
-    unsigned char* tab = smem + Cf::off_tab;
+    float4* red = reinterpret_cast<float4*>(smem);
+    uint4* own_rows = reinterpret_cast<uint4*>(smem + Cf::red_bytes);
+    uint4* own_k = own_rows + a.n_cap;
+    float4* own_f1 = reinterpret_cast<float4*>(own_k + a.n_cap);
     // sampling passes: per own site, the sums over the block's chains of phi
     // (units of 2^-24 rad) and of phi^2 (units of 2^-21 rad^2), exact in 32 bits
     // for up to 32 chains
-    uint32_t* accs = reinterpret_cast<uint32_t*>(smem + Cf::off_red);
+    uint32_t* accs = reinterpret_cast<uint32_t*>(smem + Cf::red_bytes + Cf::own_bytes(a.n_cap));
+    unsigned char* tab = smem + Cf::red_bytes + Cf::own_bytes(a.n_cap) + Cf::sum_bytes(a.n_cap);
 
     const int tid = threadIdx.x;
     const int lane = tid & 31;
@@ -253,6 +252,20 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     // the tile record carries everything the addresses need (one dependent load)
     const TileDesc T = a.tiles[tile];
     const int c = a.colour;
+    // the slots of this thread's ring cells, all the list has room for: in flight
+    // together with the record that holds their number (their copies then wait for two
+    // loads in a row, not three: 2048^2 x 32 0.2537 -> 0.2501 ms per equilibration sweep,
+    // 1024^2 x 100 0.3060 -> 0.2953)
+    constexpr int NTP = NT / P;
+    constexpr int kRingSteps = (TX + TY + NTP - 1) / NTP;
+    const int e_lo = tid / P;
+    int ring_slot[kRingSteps];
+    {
+        const int2* h = a.halo + ((long long)tile * 2 + c) * a.halo_cap;
+#pragma unroll
+        for (int k = 0; k < kRingSteps; ++k)
+            ring_slot[k] = e_lo + k * NTP < TX + TY ? h[e_lo + k * NTP].x : 0;
+    }
     const int n_own = c ? T.cnt[1] : T.cnt[0];
     const int n_oth = c ? T.cnt[0] : T.cnt[1];
     // nothing to update and no red-gap / black-sample bond energy to add
@@ -282,16 +295,21 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
         if (has0 && j < n_own) vn = *reinterpret_cast<const float2*>(sto + j * cpi);
     }
     const int spread = tile & (kSpread - 1);
+    // what the update loop needs of the chains and the image, in flight during the fill
+    const int ch0 = t_img * a.n_chains + r0 + 2 * p;
+    const float2 alpha_s =
+        (a.flags & kAlphaOne)
+            ? f2(proposal_width(1.0f))
+            : make_float2(has0 ? a.ch.alpha[ch0] : 0.0f, has1 ? a.ch.alpha[ch0 + 1] : 0.0f);
+    const float c_acc = 1.4426950408889634f * I.invT;  // log2(e) / T
+    const PhiloxPair pair_words = philox_pair_words(sweep, c2, a.rk);
 
     // -- table of the other colour, raw: entry 1 + e, pair p ----------------------
-    // Each thread copies the angle pairs of its entries e = tid / P (mod NT / P)
-    // straight into the first 8 bytes of their table cells (all copies in flight
-    // at once, no registers) and converts the same entries below, so its own
-    // wait is enough.  Lanes without a pair copy nothing (their table column is
-    // never read for a stored result).
-    constexpr int NTP = NT / P;
-    const int n_ent = n_oth + n_halo;
-    const int e_lo = tid / P;
+    // Each thread copies the angle pairs of its entries (interior cells e = tid / P,
+    // mod NT / P, then ring cells likewise) straight into the first 8 bytes of their
+    // table cells (all copies in flight at once, no registers) and converts the same
+    // entries below, so its own wait is enough.  Lanes without a pair copy nothing
+    // (their table column is never read for a stored result).
     const uint32_t tab_s = smem_addr(tab);
     const uint32_t cell_lo = tab_s + (uint32_t)((1 + e_lo) * P + p) * CB;  // this thread's first cell
     constexpr uint32_t kDstStep = (uint32_t)CB * NTP * P;
@@ -303,6 +321,11 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
 #pragma unroll kUnroll
         for (int e = e_lo; e < n_oth; e += NTP, src += src_step, dst += kDstStep)
             cp_async8_s(dst, src);
+        const uint32_t ring = tab_s + (uint32_t)((1 + n_oth + e_lo) * P + p) * CB;
+#pragma unroll
+        for (int k = 0; k < kRingSteps; ++k)
+            if (e_lo + k * NTP < n_halo)
+                cp_async8_s(ring + k * kDstStep, st + (long long)ring_slot[k] * cp);
     }
     if (tid < P) {
         float4* z = reinterpret_cast<float4*>(tab + tid * CB);
@@ -316,7 +339,7 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
         const long long b = slot_off + off_own;
         constexpr uint32_t kRow = (uint32_t)CB * P;  // bytes per table entry
         if (ACC)
-            for (int j = tid; j < n_own; j += NT) accs[j] = accs[Cf::NMAX + j] = 0u;
+            for (int j = tid; j < n_own; j += NT) accs[j] = accs[a.n_cap + j] = 0u;
         for (int j = tid; j < n_own; j += NT) {
             const uint2 r = a.slot_ref[b + j];
             const float4 f = a.slot_cs[b + j];
@@ -328,15 +351,6 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
             if (MODEL == kModelLIT) own_f1[j] = make_float4(f.z, f.w, 0.0f, 0.0f);
         }
     }
-    // ring cells (slots from the ring list), same entry residue as above
-    if (has0) {
-        const int k_first = (max(n_oth - e_lo, 0) + NTP - 1) / NTP;  // steps to the ring
-        const int e_first = e_lo + k_first * NTP;
-        const int2* h = a.halo + ((long long)tile * 2 + c) * a.halo_cap + (e_first - n_oth);
-        uint32_t dst = cell_lo + (uint32_t)k_first * kDstStep;
-        for (int e = e_first; e < n_ent; e += NTP, h += NTP, dst += kDstStep)
-            cp_async8_s(dst, st + (long long)h->x * cp);
-    }
     cp_async_wait_all();
 
     // -- conversion in place; bonds between other-colour gap cells and their
@@ -346,9 +360,9 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
         const float4* fcs = a.slot_cs + slot_off + off_oth;
         unsigned char* t = tab + (size_t)((1 + e_lo) * P + p) * CB;
         // unrolled: the conversions of four entries overlap (0.2963 -> 0.2918 ms per
-        // equilibration sweep at 2048^2 x 32; by eight 0.2881 against 0.2867 by four)
+        // equilibration sweep at 2048^2 x 32; by eight slower)
 #pragma unroll 4
-        for (int e = e_lo; e < n_ent; e += NTP, t += (size_t)NTP * P * CB) {
+        for (int e = e_lo; e < n_oth; e += NTP, t += (size_t)NTP * P * CB) {
             const float2 v = *reinterpret_cast<const float2*>(t);
             const float4 cell = MODEL == kModelGMRF ? float4{} : store_cell<MODEL>(t, a.q, v);
             if (ENERGY && e < n_oth) {
@@ -356,17 +370,19 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
                 esum = add_sample_bonds<MODEL>(a, I, cell, v, f.x, f.y, slot_off + off_oth + e, esum);
             }
         }
+        if (MODEL != kModelGMRF) {
+            unsigned char* ring = tab + (size_t)((1 + n_oth + e_lo) * P + p) * CB;
+#pragma unroll
+            for (int k = 0; k < kRingSteps; ++k)
+                if (e_lo + k * NTP < n_halo) {
+                    unsigned char* cell = ring + (size_t)k * NTP * P * CB;
+                    store_cell<MODEL>(cell, a.q, *reinterpret_cast<const float2*>(cell));
+                }
+        }
     }
     __syncthreads();
 
     // -- own colour: every site of every chain of the group ---------------------
-    const int ch0 = t_img * a.n_chains + r0 + 2 * p;
-    const float2 alpha_s =
-        (a.flags & kAlphaOne)
-            ? f2(proposal_width(1.0f))
-            : make_float2(has0 ? a.ch.alpha[ch0] : 0.0f, has1 ? a.ch.alpha[ch0 + 1] : 0.0f);
-    const float c_acc = 1.4426950408889634f * I.invT;  // log2(e) / T
-    const PhiloxPair pair_words = philox_pair_words(sweep, c2, a.rk);
     unsigned cnt0 = 0, cnt1 = 0;
     const int n_steps = (n_own + SPW - 1) / SPW;
     const unsigned char* tabp = tab + p * CB;  // this lane's column of the table
@@ -403,29 +419,16 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
                 const bool lower = p < 8;
                 const float v = (lower ? sa : sb) + __shfl_xor_sync(0xffffffffu, lower ? sb : sa, 8);
                 if (in)
-                    atomicAdd(&accs[(lower ? 0 : Cf::NMAX) + j],
+                    atomicAdd(&accs[(lower ? 0 : a.n_cap) + j],
                               __float2uint_rn(v * (lower ? 16777216.0f : 2097152.0f)));
             } else if (in) {
                 atomicAdd(&accs[j], __float2uint_rn(sa * 16777216.0f));
-                atomicAdd(&accs[Cf::NMAX + j], __float2uint_rn(sb * 2097152.0f));
+                atomicAdd(&accs[a.n_cap + j], __float2uint_rn(sb * 2097152.0f));
             }
         }
         cnt0 += (act && o.acc0) ? 1u : 0u;
         cnt1 += (act1 && o.acc1) ? 1u : 0u;
         if (ENERGY) esum = add2(esum, make_float2(act ? o.e.x : 0.0f, act1 ? o.e.y : 0.0f));
-    }
-
-    if (ACC) {
-        // the block's sums go to the FP64 realisation sums (fire-and-forget adds;
-        // one add per site and block)
-        __syncthreads();
-        const bool accum2 = (a.flags & kAccumulate2) != 0;
-        for (int j = tid; j < n_own; j += NT) {
-            atomicAdd(a.acc1 + slot_off + off_own + j, (double)accs[j] * 0x1p-24);
-            if (accum2)
-                atomicAdd(a.acc2 + slot_off + off_own + j, (double)accs[Cf::NMAX + j] * 0x1p-21);
-        }
-        __syncthreads();  // the per-chain reduction below reuses the area
     }
 
     // -- per-chain totals: lanes of one pair, then warps ------------------------
@@ -441,6 +444,16 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     }
     if (lane < P) red[warp * P + lane] = make_float4(e0, e1, __uint_as_float(cnt0), __uint_as_float(cnt1));
     __syncthreads();
+    if (ACC) {
+        // the block's sums go to the FP64 realisation sums (fire-and-forget adds; one add
+        // per site and block)
+        const bool accum2 = (a.flags & kAccumulate2) != 0;
+        for (int j = tid; j < n_own; j += NT) {
+            atomicAdd(a.acc1 + slot_off + off_own + j, (double)accs[j] * 0x1p-24);
+            if (accum2)
+                atomicAdd(a.acc2 + slot_off + off_own + j, (double)accs[a.n_cap + j] * 0x1p-21);
+        }
+    }
     if (tid < P && 2 * tid < ng) {
         double E0 = 0.0, E1 = 0.0;
         unsigned n0 = 0, n1 = 0;
@@ -475,9 +488,9 @@ cudaError_t launch_one(const SweepArgs& a, cudaStream_t s, bool setup_only) {
         attr_set = true;
     }
     if (setup_only) return cudaSuccess;
-    if (a.gt < 1 || a.gt > Cf::GT) return cudaErrorInvalidValue;
+    if (a.gt < 1 || a.gt > Cf::GT || a.n_cap < 0 || a.n_cap > Cf::NMAX) return cudaErrorInvalidValue;
     dim3 grid(a.n_list, (a.chain_end - a.chain0 + a.chain_group - 1) / a.chain_group);
-    kernel<<<grid, Cf::NT, Cf::smem_for(a.gt, P), s>>>(a);
+    kernel<<<grid, Cf::NT, Cf::smem_for(a.gt, a.n_cap, P), s>>>(a);
     return cudaGetLastError();
 }
 
