@@ -434,7 +434,8 @@ def run_gpu(args):
     # two runs of the temperature lattices per Newton step (each one launch), the Newton
     # steps (and their set-up), the 16 initialisation kernels of the two contexts (map,
     # extremes, sample energy, tile tables, hot starts, chain set-up) and the prediction
-    line["gpu_launches"] = args.steps * (launches[0] * (ne + nm) + 2 * topts.iters
+    # (the sampling sweeps of a run share one bookkeeping launch)
+    line["gpu_launches"] = args.steps * (launches[0] * (ne + nm) - (nm - 1) + 2 * topts.iters
                                          + topts.iters + 1 + 16 + 1)
     if not args.no_plain:
         # the plain single-image path on the same job (one warm-up, one timed step)

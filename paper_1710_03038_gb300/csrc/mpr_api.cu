@@ -451,12 +451,12 @@ __global__ void set_alpha_kernel(ChainDev ch, int nc) {
     if (i < nc) ch.alpha[i] = proposal_width(ch.a[i]);
 }
 
-// Bookkeeping after every sweep: acceptance -> a (Alg. 2 step 4.2), energy
+// Bookkeeping after a sweep, or after n_sweeps sampling sweeps: acceptance -> a (Alg. 2 step 4.2), energy
 // record (step 4.3), counters.  One warp per chain sums the chain's kSpread
 // partial slots; the warps of all blocks share the chains.
 __global__ void end_sweep_kernel(const ImgDev* img, ChainDev ch, Control* ctl, int n_img,
                                  int n_chains, int equil, int record, int stats, int add_ess,
-                                 double A_targ, double k_a) {
+                                 double A_targ, double k_a, int n_sweeps) {
     static_assert(kSpread == 32, "one lane per spread slot");
     const uint32_t i = ctl->equil_index;
     const int nc = n_img * n_chains;
@@ -494,8 +494,8 @@ __global__ void end_sweep_kernel(const ImgDev* img, ChainDev ch, Control* ctl, i
         __threadfence();
         if (atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1) {
             ctl->ticket = 0;
-            ctl->sweep += 1;
-            if (equil) ctl->equil_index += 1;
+            ctl->sweep += (uint32_t)n_sweeps;
+            if (equil) ctl->equil_index += (uint32_t)n_sweeps;
         }
     }
 }
@@ -1240,10 +1240,16 @@ mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bo
     ChainRange cr[2];
     const int n_cr = chain_ranges(c, cr);
     const bool tiled = c->g.path == MPR_PATH_TILED;
+    // Equilibration adapts a after every sweep and recorded energies are per sweep;
+    // other sampling sweeps need no bookkeeping of their own: the launches carry their
+    // sweep number, the last one counts acceptances, and one bookkeeping launch ends the
+    // run (16 ragged images x 16, 25 sampling sweeps: 1835 -> 1710 us)
+    const bool once = tiled && !equil && !record;
     for (int k = 0; k < n; ++k) {
+        a.sweep_off = once ? (uint32_t)k : 0u;
         for (int colour = 0; colour < 2; ++colour) {
             a.colour = colour;
-            a.flags = base | ((record && colour == 1) ? kEnergy : 0);
+            a.flags = base | ((record && colour == 1) ? kEnergy : 0) | (once && k + 1 < n ? 0 : kCount);
             cudaError_t e = cudaSuccess;
             if (!tiled) {
                 e = launch_plain_pass(a, c->g.max_Lx, c->g.max_Ly, s);
@@ -1295,11 +1301,12 @@ mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bo
             }
             if (e != cudaSuccess) return fail(MPR_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(e));
         }
+        if (once && k + 1 < n) continue;
         // one warp per chain, 8 chains per block
         const int nc = c->g.n_img * c->g.n_chains;
         end_sweep_kernel<<<std::min((nc + 7) / 8, 1024), 256, 0, s>>>(
             c->d_img, c->ch, c->d_ctl, c->g.n_img, c->g.n_chains, equil ? 1 : 0, record ? 1 : 0,
-            stats ? 1 : 0, tiled ? 1 : 0, c->p.A_targ, c->p.k_a);
+            stats ? 1 : 0, tiled ? 1 : 0, c->p.A_targ, c->p.k_a, once ? n : 1);
         MPR_CUDA(cudaGetLastError());
     }
     return MPR_OK;

@@ -77,6 +77,7 @@ enum SweepFlags : int {
     kAlphaOne = 8,     // a = 1 (printed Alg. 2 step 5.2)
     kLiteralOR = 16,   // printed q = 1 over-relaxation formula (plain path only)
     kGMRF = 32,        // GMRF pair interaction of Sec. 4.3 (plain path only)
+    kCount = 64,       // count the accepted proposals (tiled launches)
 };
 
 struct SweepArgs {
@@ -111,6 +112,7 @@ struct SweepArgs {
     int tile_base;
     int n_list;                // tiled: tiles in the launch
     int n_img;
+    uint32_t sweep_off;        // sweeps of this run before the launch's (tiled launches)
     uint32_t img_tag;          // OR-ed into the image field of the counter (1 << 30: T lattices)
 };
 

@@ -279,7 +279,7 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
     const int ng = min(a.chain_group, a.chain_end - r0);
     const bool has0 = GROUPS != kRagged || 2 * p < ng;      // this lane's pair exists
     const bool has1 = GROUPS != kRagged || 2 * p + 1 < ng;  // and has a second chain
-    const uint32_t sweep = a.ctl->sweep;
+    const uint32_t sweep = a.ctl->sweep + a.sweep_off;
     const uint32_t c3 = (uint32_t)t_img | a.img_tag | ((uint32_t)c << 31);
     const uint32_t c2 = (uint32_t)(r0 >> 1) + (uint32_t)p;  // chain >> 1 of the pair
     const UpdateConst uk{a.q, a.inv_q, a.two_pi_q, a.J};
@@ -466,10 +466,11 @@ tiled_pass_kernel(const __grid_constant__ SweepArgs a) {
             n1 += __float_as_uint(r.w);
         }
         const long long b0 = (long long)(t_img * a.n_chains + r0 + 2 * tid) * kSpread + spread;
-        if (n0) atomicAdd(a.ch.acc_cnt + b0, n0);
+        const bool count = (a.flags & kCount) != 0;
+        if (count && n0) atomicAdd(a.ch.acc_cnt + b0, n0);
         if (ENERGY) atomicAdd(a.ch.e_cur + b0, E0);
         if (2 * tid + 1 < ng) {
-            if (n1) atomicAdd(a.ch.acc_cnt + b0 + kSpread, n1);
+            if (count && n1) atomicAdd(a.ch.acc_cnt + b0 + kSpread, n1);
             if (ENERGY) atomicAdd(a.ch.e_cur + b0 + kSpread, E1);
         }
     }
