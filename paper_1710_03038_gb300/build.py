@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libmpr.so")
-SOURCES = ["mpr_api.cu", "mpr_dense.cu", "mpr_tiled.cu", "mpr_tiled_32x16.cu", "mpr_tiled_16x16.cu",
+SOURCES = ["mpr_api.cu", "mpr_setup.cu", "mpr_dense.cu", "mpr_tiled.cu", "mpr_tiled_32x16.cu", "mpr_tiled_16x16.cu",
            "mpr_tiled_16x16_lit.cu", "mpr_tiled_16x16_gmrf.cu",
            "mpr_tiled_32x32.cu", "mpr_resident.cu", "mpr_resident_mpr.cu", "mpr_resident_gmrf.cu",
            "mpr_plain.cu", "mpr_lattice.cu", "mpr_noalloc.cu",

@@ -49,7 +49,7 @@ constexpr int kResidentBlocks = 2048;  // upper bound on the blocks that run at 
 // Byte offsets of the workspace regions of one context.
 struct Layout {
     size_t img, ctl, ch_a, ch_alpha, ch_cnt, ch_last, ch_ecur, ch_elast, ch_esum, ch_esum2;
-    size_t zst, gst, outst, eout, samp, slot_map, tiles, counts, halo, tile_list, scratch;
+    size_t zst, gst, outst, eout, samp, slot_map, tiles, counts, halo, tile_list, scratch, stats;
     size_t slot_pos, slot_ref, slot_cs, acc1, acc2, state, newton, hist, res_words, res_epoch, res_packets, res_e, res_end, sub;
     size_t total;
     long long n_slots;   // slot space over all images
@@ -139,6 +139,7 @@ Layout make_layout(const Geometry& g, const std::vector<long long>& slots_per_im
     L.halo = take(sizeof(int2) * (size_t)g.n_tiles * 2 * g.halo_cap);
     L.tile_list = take(sizeof(int) * 2 * (size_t)g.n_tiles);
     L.scratch = take(sizeof(double) * 4 * g.n_img);
+    L.stats = take(sizeof(TileStats) + sizeof(int) * 4 * kTileSizes);
     L.n_slots = 0;
     L.n_state = 0;
     for (int i = 0; i < g.n_img; ++i) {
@@ -199,6 +200,7 @@ struct mpr_ctx {
     int* d_slot_map = nullptr;
     TileDesc* d_tiles = nullptr;
     int2* d_halo = nullptr;
+    TileStats* d_stats = nullptr;  // then the tiles' size counts
     int* d_tile_list = nullptr;  // per colour: the tiles of the light launch, then the heavy ones
     uint32_t* d_slot_pos = nullptr;
     uint2* d_slot_ref = nullptr;
@@ -278,6 +280,7 @@ void bind_views(mpr_ctx* c) {
     c->d_slot_map = at<int>(w, L.slot_map);
     c->d_tiles = at<TileDesc>(w, L.tiles);
     c->d_halo = at<int2>(w, L.halo);
+    c->d_stats = at<TileStats>(w, L.stats);
     c->d_tile_list = at<int>(w, L.tile_list);
     c->d_slot_pos = at<uint32_t>(w, L.slot_pos);
     c->d_slot_ref = at<uint2>(w, L.slot_ref);
@@ -291,116 +294,6 @@ void bind_views(mpr_ctx* c) {
 }
 
 // ======================================================= init kernels
-
-__device__ __forceinline__ uint32_t ordered(float f) {
-    const uint32_t b = __float_as_uint(f);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-// Extremes over sample sites and gap counts, per image (blockIdx.y).
-__global__ void minmax_kernel(const ImgDev* img, const float* z, const uint8_t* gap,
-                              uint32_t* mm, unsigned long long* ngap) {
-    const ImgDev& I = img[blockIdx.y];
-    const long long n = (long long)I.Lx * I.Ly;
-    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-    unsigned long long cnt = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        if (gap[I.site_off + i]) { ++cnt; continue; }
-        const uint32_t o = ordered(z[I.site_off + i]);
-        lo = min(lo, o);
-        hi = max(hi, o);
-    }
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMin(mm + 2 * blockIdx.y, lo);
-        atomicMax(mm + 2 * blockIdx.y + 1, hi);
-        if (cnt) atomicAdd(ngap + blockIdx.y, cnt);
-    }
-}
-
-// Eq. map into the per-image sample plane (FP64 arithmetic, rounded once);
-// gap sites hold -1.
-__global__ void map_kernel(const ImgDev* img, const float* z, const uint8_t* gap, float* samp,
-                           int unconditional) {
-    const ImgDev& I = img[blockIdx.y];
-    const long long n = (long long)I.Lx * I.Ly;
-    const double zmin = I.zmin, scale = 2.0 * kPiD / ((double)I.zmax - (double)I.zmin);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long s = I.site_off + i;
-        samp[s] = (unconditional || gap[s]) ? -1.0f : (float)(((double)z[s] - zmin) * scale);
-    }
-}
-
-// Sample specific energy (Eq. mpr-sse) sums: -J sum cos(q dphi) over sample
-// pairs (right and down bonds), FP64.
-// One bond's energy in FP32 (summed in FP64 by the caller); the same
-// expression as the allocation-free entry point's.
-__device__ __forceinline__ float bond_energy(float d, float q, float J, int gmrf) {
-    return gmrf ? J * (d * d * (float)(0.5 / (kPiD * kPiD)) - 1.0f) : -J * cosf(q * d);
-}
-
-__global__ void sample_energy_kernel(const ImgDev* img, const float* samp, double q, double J,
-                                     int gmrf, double* sums, unsigned long long* npairs) {
-    const ImgDev& I = img[blockIdx.y];
-    const long long n = (long long)I.Lx * I.Ly;
-    double s = 0.0;
-    unsigned long long cnt = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const float v = samp[I.site_off + i];
-        if (v < 0.0f) continue;
-        const int x = (int)(i % I.Lx), y = (int)(i / I.Lx);
-        if (x + 1 < I.Lx) {
-            const float w = samp[I.site_off + i + 1];
-            if (w >= 0.0f) { s += (double)bond_energy(v - w, (float)q, (float)J, gmrf); ++cnt; }
-        }
-        if (y + 1 < I.Ly) {
-            const float w = samp[I.site_off + i + I.Lx];
-            if (w >= 0.0f) { s += (double)bond_energy(v - w, (float)q, (float)J, gmrf); ++cnt; }
-        }
-    }
-    s = warp_sum(s);
-    for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
-    if ((threadIdx.x & 31) == 0) {
-        if (s != 0.0) atomicAdd(sums + blockIdx.y, s);
-        if (cnt) atomicAdd(npairs + blockIdx.y, cnt);
-    }
-}
-
-// Start of the tiled state: hot (slot -> 2 pi u with the site's first uniform
-// at sweep 0xFFFFFFFF) or cold (every gap angle pi); padding slots and the
-// padding chain of an odd chain count hold 0.  One thread per (slot, chain
-// pair): the pair shares its Philox block (words 0 and 2) and one float2 store.
-__global__ void hot_start_tiled_kernel(const ImgDev* img, const uint32_t* slot_pos, float* state,
-                                       long long slots_img, int img_i, int n_chains, uint2 key,
-                                       uint32_t img_tag, int cold) {
-    const ImgDev& I = img[img_i];
-    const long long np = I.sstride / 2;  // chain pairs per slot
-    const long long total = slots_img * np;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-         t += (long long)gridDim.x * blockDim.x) {
-        const long long k = t / np;
-        const int c0 = 2 * (int)(t - k * np);
-        const uint32_t p = slot_pos[I.slot_off + k];
-        float2 v = make_float2(0.0f, 0.0f);
-        if (p != 0xFFFFFFFFu) {
-            if (cold) {
-                v = make_float2(kPi, c0 + 1 < n_chains ? kPi : 0.0f);
-            } else {
-                const int X = (int)(p & 0xFFFFu), Y = (int)(p >> 16);
-                const uint4 w = philox4x32_10(site_counter(X, Y, (X + Y) & 1, 0xFFFFFFFFu,
-                                                           (uint32_t)c0, (uint32_t)img_i | img_tag),
-                                              key);
-                v = make_float2(kTwoPi * u24(w.x), c0 + 1 < n_chains ? kTwoPi * u24(w.z) : 0.0f);
-            }
-        }
-        *reinterpret_cast<float2*>(state + state_index(I, c0, k)) = v;
-    }
-}
 
 // Dense planes of the plain path: fixed angle with the sign bit at samples,
 // hot start at gaps.
@@ -791,11 +684,13 @@ int chain_ranges(const mpr_ctx* c, ChainRange out[2]) {
     return 2;
 }
 
-// Sorts the tiles of each colour pass into a light launch, whose tables let
-// an SM hold as many blocks as its threads allow, and a heavy launch with the
-// rest (tiles inside large gap blocks, say), so that a few dense tiles do not
-// cut the occupancy of every block.  Without heavy tiles a pass is one launch.
-mpr_status split_tiles(mpr_ctx* c, const std::vector<TileDesc>& tiles, cudaStream_t s) {
+// Sorts the tiles of each colour pass into a light launch, whose blocks' shared memory
+// lets an SM hold as many as its threads allow, and a heavy launch with the rest (tiles
+// inside large gap blocks, say), so that a few dense tiles do not cut the occupancy of
+// every block.  Without heavy tiles a pass is one launch.  A block's shared memory
+// follows from the launch's largest table and its most own sites: of the pairs of
+// limits that fit, the one that leaves the fewest tiles out (by the sizes' counts).
+mpr_status split_tiles(mpr_ctx* c, const TileStats& st, cudaStream_t s) {
     const Geometry& g = c->g;
     const int cg = pick_chain_group(c), flags = model_flags(c->p);
     int dev = 0, sm_bytes = 0, reserved = 0;
@@ -803,68 +698,79 @@ mpr_status split_tiles(mpr_ctx* c, const std::vector<TileDesc>& tiles, cudaStrea
     MPR_CUDA(cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
     MPR_CUDA(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
     const size_t budget = (size_t)sm_bytes / tiled_blocks_per_sm(g.tx, g.ty) - (size_t)reserved;
-    const int n = g.n_tiles;
-    std::vector<int> list(2 * (size_t)n);
+    const auto bytes = [&](int e, int own) { return tiled_pass_smem(g.tx, g.ty, e, own, cg, flags); };
     bool split = false;
     for (int col = 0; col < 2; ++col) {
-        // light: the largest set of tiles, by table entries and own sites, whose common
-        // block size keeps the blocks per SM (the own sites' records are sized for the
-        // light tile with the most)
-        int gmax = 1, cmax = 1, glight = 1, clight = 1, nl = 0;
-        std::vector<int> heavy;
-        for (int t = 0; t < n; ++t) {
-            const int e = tiles[t].cnt[col ^ 1] + tiles[t].halo_cnt[col] + 1, own = tiles[t].cnt[col];
-            gmax = std::max(gmax, e);
-            cmax = std::max(cmax, own);
-            if (tiled_pass_smem(g.tx, g.ty, std::max(e, glight), std::max(own, clight), cg, flags) <= budget) {
-                list[(size_t)col * n + nl++] = t;
-                glight = std::max(glight, e);
-                clight = std::max(clight, own);
-            } else {
-                heavy.push_back(t);
+        c->gt[col] = c->gt_light[col] = std::max(1, st.gt[col]);
+        c->n_cap[col] = c->n_cap_light[col] = std::max(1, st.n_cap[col]);
+        c->n_light[col] = g.n_tiles;
+        split = split || bytes(c->gt[col], c->n_cap[col]) > budget;
+    }
+    if (!split) return MPR_OK;
+    std::vector<int> h(4 * kTileSizes);
+    int* d_hist = reinterpret_cast<int*>(c->d_stats + 1);
+    MPR_CUDA(cudaMemsetAsync(d_hist, 0, sizeof(int) * h.size(), s));
+    MPR_CUDA(launch_tile_hist(c->d_tiles, g.n_tiles, d_hist, s));
+    MPR_CUDA(cudaMemcpyAsync(h.data(), d_hist, sizeof(int) * h.size(), cudaMemcpyDeviceToHost, s));
+    MPR_CUDA(cudaStreamSynchronize(s));
+    for (int col = 0; col < 2; ++col) {
+        if (bytes(c->gt[col], c->n_cap[col]) <= budget) continue;
+        const int* he = &h[2 * col * kTileSizes];
+        const int* ho = he + kTileSizes;
+        int e = c->gt[col];
+        long long over_e = 0, over_own = 0, best = 1LL << 60;
+        c->gt_light[col] = c->n_cap_light[col] = 0;  // (no limits that fit: every tile is heavy)
+        for (int own = c->n_cap[col]; own >= 1; --own) {
+            // limits: own sites, and the most entries that fit beside them
+            while (e >= 1 && bytes(e, own) > budget) over_e += he[e--];
+            int most = e;
+            long long over = over_e;
+            while (most < c->gt[col] && bytes(most + 1, own) <= budget) over -= he[++most];
+            e = most;
+            over_e = over;
+            if (e >= 1 && over_e + over_own < best) {
+                best = over_e + over_own;
+                c->gt_light[col] = e;
+                c->n_cap_light[col] = own;
             }
+            over_own += ho[own];
         }
-        for (size_t k = 0; k < heavy.size(); ++k) list[(size_t)col * n + nl + k] = heavy[k];
-        c->gt[col] = gmax;
-        c->gt_light[col] = glight;
-        c->n_cap[col] = cmax;
-        c->n_cap_light[col] = clight;
-        c->n_light[col] = nl;
-        split = split || nl < n;
     }
-    if (split) {
-        MPR_CUDA(cudaMemcpyAsync(c->d_tile_list, list.data(), sizeof(int) * list.size(),
-                                 cudaMemcpyHostToDevice, s));
-        MPR_CUDA(cudaStreamSynchronize(s));
-    }
+    MPR_CUDA(launch_tile_split(c->d_tiles, g.n_tiles, c->gt_light, c->n_cap_light, c->d_tile_list,
+                               c->d_stats->n_light, s));
+    MPR_CUDA(cudaMemcpyAsync(c->n_light, c->d_stats->n_light, sizeof(c->n_light), cudaMemcpyDeviceToHost, s));
+    MPR_CUDA(cudaStreamSynchronize(s));
     return MPR_OK;
 }
 
-// Whether runs of sweeps go through the resident kernel: 16 x 16 tiles, the MPR bond
-// or the GMRF, and every (tile, chain group) block on the GPU at once.  The line lies
-// at the device's own limit: below it the resident run was the faster one at every
-// size measured.
-mpr_status choose_resident(mpr_ctx* c, const std::vector<TileDesc>& tiles, cudaStream_t s) {
+// Blocks of a resident run of the context (with those that record energies), or 0 where
+// runs of sweeps cannot go through the resident kernel: 16 x 16 tiles, the MPR bond or
+// the GMRF.
+long long resident_need(const mpr_ctx* c) {
     const Geometry& g = c->g;
-    const int flags = model_flags(c->p);
-    c->resident = false;
-    if (g.tx != 16 || g.ty != 16 || (flags & kLiteralOR)) return MPR_OK;
+    if (g.path != MPR_PATH_TILED || g.tx != 16 || g.ty != 16 || (model_flags(c->p) & kLiteralOR)) return 0;
     ChainRange cr[2];
     const int n_cr = chain_ranges(c, cr);
     const long long groups = (cr[0].chain_end + cr[0].group - 1) / cr[0].group + (n_cr - 1);
-    // (with the blocks that record energies)
     const long long need = (g.n_tiles + (long long)g.n_img * resident_recorders(cr[0].group)) * groups;
-    if (need > kResidentBlocks) return MPR_OK;
-    const int P = tiled_pairs(cr[0].group);
-    const bool gmrf = (flags & kGMRF) != 0;
-    size_t smem = 0;
-    for (const TileDesc& t : tiles) smem = std::max(smem, resident_smem(t, P, gmrf));
+    return need > kResidentBlocks ? 0 : need;
+}
+
+// Resident where every (tile, chain group) block fits the GPU at once.  The line lies
+// at the device's own limit: below it the resident run was the faster one at every
+// size measured.
+mpr_status choose_resident(mpr_ctx* c, const TileStats& st, cudaStream_t s) {
+    const long long need = resident_need(c);
+    c->resident = false;
+    if (need == 0) return MPR_OK;
     long long blocks = 0;
-    MPR_CUDA(resident_blocks(smem, gmrf, &blocks));
+    MPR_CUDA(resident_blocks(st.res_smem, &blocks));
     c->resident = need <= blocks;
-    c->res_smem = smem;
-    if (c->resident)
+    c->res_smem = st.res_smem;
+    if (c->resident) {
+        MPR_CUDA(resident_prepare(c->p.model == MPR_MODEL_GMRF));
         MPR_CUDA(cudaMemsetAsync(c->ws + c->L.res_words, 0, c->L.res_end - c->L.res_words, s));
+    }
     return MPR_OK;
 }
 
@@ -913,7 +819,23 @@ mpr_status validate_shapes(int n_img, const int* Lx, const int* Ly, int n_chains
     return MPR_OK;
 }
 
-// Builds a context over `ws`.  unconditional: every site free, no inputs.
+// Slots of an image without samples: every site a gap, each tile's colours padded to 4.
+long long full_slots(int Lx, int Ly, int tx, int ty) {
+    const auto tile = [](long long w, long long h) {
+        const long long red = (w * h + 1) / 2, black = w * h / 2;  // (origins are even)
+        return ((red + 3) & ~3LL) + ((black + 3) & ~3LL);
+    };
+    const long long nx = Lx / tx, ny = Ly / ty, rx = Lx % tx, ry = Ly % ty;
+    long long n = nx * ny * tile(tx, ty);
+    if (rx) n += ny * tile(rx, ty);
+    if (ry) n += nx * tile(tx, ry);
+    if (rx && ry) n += tile(rx, ry);
+    return n;
+}
+
+// Builds a context over `ws`: everything is enqueued on s except what the host must know
+// (the images' extremes, gaps and slots: one wait, none for the temperature lattices);
+// init_finish() reads the rest.  unconditional: every site free, no inputs.
 mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_chains,
                      const float* z, const uint8_t* gap, mpr_mem where, void* ws, size_t ws_bytes,
                      bool unconditional, cudaStream_t s) {
@@ -937,11 +859,12 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
     for (int i = 0; i < n_img; ++i) worst[i] = 0;
     c->ws = static_cast<unsigned char*>(ws);
     c->L = make_layout(g, worst, 0, staging);
-    if (c->L.scratch + align_up(sizeof(double) * 4 * n_img) > ws_bytes)
+    if (c->L.stats + align_up(sizeof(TileStats) + sizeof(int) * 4 * kTileSizes) > ws_bytes)
         return fail(MPR_ERR_WORKSPACE, "workspace too small");
     bind_views(c);
 
     c->h_img.assign(n_img, ImgDev{});
+    long long maxn = 0;
     for (int i = 0; i < n_img; ++i) {
         ImgDev& I = c->h_img[i];
         I.Lx = Lx[i];
@@ -952,9 +875,9 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
         I.n_bonds = (double)Lx[i] * (Ly[i] - 1) + (double)Ly[i] * (Lx[i] - 1);
         I.T = 1.0;
         I.invT = 1.0f;
+        maxn = std::max(maxn, (long long)Lx[i] * Ly[i]);
     }
-    MPR_CUDA(cudaMemcpyAsync(c->d_img, c->h_img.data(), sizeof(ImgDev) * n_img,
-                             cudaMemcpyHostToDevice, s));
+    MPR_CUDA(launch_put(c->d_img, c->h_img.data(), sizeof(ImgDev) * n_img, s));
     const size_t N = (size_t)g.n_sites;
     const float* d_z = nullptr;
     const uint8_t* d_gap = c->d_gst;
@@ -967,53 +890,19 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
         d_z = c->d_zst;
     }
 
-    // tile descriptors
-    std::vector<TileDesc> tiles;
-    if (tiled) {
-        tiles.reserve(g.n_tiles);
-        for (int i = 0; i < n_img; ++i)
-            for (int y0 = 0; y0 < Ly[i]; y0 += ty)
-                for (int x0 = 0; x0 < Lx[i]; x0 += tx) {
-                    TileDesc t{};
-                    t.img = i;
-                    t.x0 = x0;
-                    t.y0 = y0;
-                    tiles.push_back(t);
-                }
-        MPR_CUDA(cudaMemcpyAsync(c->d_tiles, tiles.data(), sizeof(TileDesc) * g.n_tiles,
-                                 cudaMemcpyHostToDevice, s));
-    }
-
-    // extremes and gap counts
+    // extremes and gap counts, tile records and slot segments
     double* scratch = at<double>(c->ws, c->L.scratch);
-    uint32_t* mm = reinterpret_cast<uint32_t*>(scratch);                         // [2 n_img]
-    unsigned long long* ngap = reinterpret_cast<unsigned long long*>(scratch + n_img);  // [n_img]
-    std::vector<uint32_t> h_mm(2 * n_img);
-    for (int i = 0; i < n_img; ++i) { h_mm[2 * i] = 0xFFFFFFFFu; h_mm[2 * i + 1] = 0u; }
-    MPR_CUDA(cudaMemcpyAsync(mm, h_mm.data(), sizeof(uint32_t) * 2 * n_img, cudaMemcpyHostToDevice, s));
-    MPR_CUDA(cudaMemsetAsync(ngap, 0, sizeof(unsigned long long) * n_img, s));
-    std::vector<unsigned long long> h_ngap(n_img, 0);
+    ImgScan* d_scan = reinterpret_cast<ImgScan*>(scratch);
+    std::vector<ImgScan> scan(n_img, ImgScan{0xFFFFFFFFu, 0u, 0ull, 0ull});
+    MPR_CUDA(launch_put(d_scan, scan.data(), sizeof(ImgScan) * n_img, s));
+    if (!unconditional) MPR_CUDA(launch_minmax(c->d_img, n_img, maxn, d_z, d_gap, d_scan, s));
+    if (tiled)
+        MPR_CUDA(launch_tile_count(c->d_img, n_img, c->d_tiles, g.n_tiles, d_gap, tx, ty,
+                                   at<int>(c->ws, c->L.counts), d_scan, s));
     if (!unconditional) {
-        long long maxn = 0;
-        for (int i = 0; i < n_img; ++i) maxn = std::max(maxn, (long long)Lx[i] * Ly[i]);
-        minmax_kernel<<<dim3(grid_for(maxn, 256, 1024), n_img), 256, 0, s>>>(c->d_img, d_z, d_gap, mm, ngap);
-        MPR_CUDA(cudaGetLastError());
+        MPR_CUDA(cudaMemcpyAsync(scan.data(), d_scan, sizeof(ImgScan) * n_img, cudaMemcpyDeviceToHost, s));
+        MPR_CUDA(cudaStreamSynchronize(s));
     }
-    std::vector<int> h_counts;
-    if (tiled) {
-        int* counts = at<int>(c->ws, c->L.counts);
-        MPR_CUDA(cudaMemsetAsync(counts, 0, sizeof(int) * 2 * g.n_tiles, s));
-        MPR_CUDA(launch_tile_count(c->d_img, c->d_tiles, g.n_tiles, d_gap, tx, ty, counts, s));
-        h_counts.resize(2 * g.n_tiles);
-        MPR_CUDA(cudaMemcpyAsync(h_counts.data(), counts, sizeof(int) * 2 * g.n_tiles,
-                                 cudaMemcpyDeviceToHost, s));
-    }
-    if (!unconditional) {
-        MPR_CUDA(cudaMemcpyAsync(h_mm.data(), mm, sizeof(uint32_t) * 2 * n_img, cudaMemcpyDeviceToHost, s));
-        MPR_CUDA(cudaMemcpyAsync(h_ngap.data(), ngap, sizeof(unsigned long long) * n_img,
-                                 cudaMemcpyDeviceToHost, s));
-    }
-    MPR_CUDA(cudaStreamSynchronize(s));
 
     // per image: range, gap count, slot space
     c->slots.assign(n_img, 0);
@@ -1030,33 +919,21 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
                 std::memcpy(&f, &b, 4);
                 return f;
             };
-            if (h_mm[2 * i] == 0xFFFFFFFFu)
+            if (scan[i].lo == 0xFFFFFFFFu)
                 return fail(MPR_ERR_DEGENERATE_RANGE, "image " + std::to_string(i) + " has no samples");
-            I.zmin = dec(h_mm[2 * i]);
-            I.zmax = dec(h_mm[2 * i + 1]);
+            I.zmin = dec(scan[i].lo);
+            I.zmax = dec(scan[i].hi);
             if (!(I.zmax > I.zmin))
                 return fail(MPR_ERR_DEGENERATE_RANGE,
                             "image " + std::to_string(i) + ": z_max == z_min over the samples");
             if (!std::isfinite(I.zmin) || !std::isfinite(I.zmax))
                 return fail(MPR_ERR_INVALID_ARG, "non-finite sample value in image " + std::to_string(i));
-            I.n_gap = (long long)h_ngap[i];
+            I.n_gap = (long long)scan[i].n_gap;
             if (I.n_gap == 0)
                 return fail(MPR_ERR_INVALID_ARG, "image " + std::to_string(i) + " has no gaps");
         }
-        if (tiled) {
-            long long off = 0;
-            for (int t = g.tile0[i]; t < g.tile0[i] + g.ntiles[i]; ++t) {
-                for (int col = 0; col < 2; ++col) {
-                    const int n = h_counts[2 * t + col];
-                    tiles[t].off[col] = (int)off;
-                    tiles[t].cnt[col] = n;
-                    off += (n + 3) & ~3;
-                }
-            }
-            c->slots[i] = off;
-        } else {
-            c->slots[i] = (long long)Lx[i] * Ly[i];
-        }
+        c->slots[i] = !tiled ? (long long)Lx[i] * Ly[i]
+                      : unconditional ? full_slots(Lx[i], Ly[i], tx, ty) : (long long)scan[i].slots;
     }
     c->L = make_layout(g, c->slots, sub_bytes, staging);
     if (c->L.total > ws_bytes)
@@ -1074,52 +951,23 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
         slot_off += c->slots[i];
         state_off += c->slots[i] * state_chains(g);
     }
-    MPR_CUDA(cudaMemcpyAsync(c->d_img, c->h_img.data(), sizeof(ImgDev) * n_img,
-                             cudaMemcpyHostToDevice, s));
+    MPR_CUDA(launch_put(c->d_img, c->h_img.data(), sizeof(ImgDev) * n_img, s));
+    MPR_CUDA(launch_map(c->d_img, n_img, maxn, d_z, d_gap, c->d_samp, unconditional, s));
     if (tiled) {
-        for (TileDesc& t : tiles) {
-            const ImgDev& I = c->h_img[t.img];
-            t.cp = (int)I.sstride;
-            t.state_off = I.state_off;
-            t.slot_off = I.slot_off;
-        }
-        MPR_CUDA(cudaMemcpyAsync(c->d_tiles, tiles.data(), sizeof(TileDesc) * g.n_tiles,
-                                 cudaMemcpyHostToDevice, s));
-        MPR_CUDA(cudaMemsetAsync(c->d_slot_pos, 0xFF, sizeof(uint32_t) * c->L.n_slots, s));
-        MPR_CUDA(launch_tile_fill(c->d_img, c->d_tiles, g.n_tiles, d_gap, tx, ty, c->d_slot_pos,
-                                  c->d_slot_map, c->d_halo, g.halo_cap, s));
-        // table entries of every tile and pass from the ring lists just built
-        MPR_CUDA(cudaMemcpyAsync(tiles.data(), c->d_tiles, sizeof(TileDesc) * g.n_tiles,
-                                 cudaMemcpyDeviceToHost, s));
-        MPR_CUDA(cudaStreamSynchronize(s));
-        MPR_TRY(split_tiles(c, tiles, s));
-        MPR_TRY(choose_resident(c, tiles, s));
         ChainRange cr[2];
-        const bool extra = c->n_light[0] < g.n_tiles || c->n_light[1] < g.n_tiles ||
-                           chain_ranges(c, cr) > 1;
-        if (extra && !c->side) {
-            MPR_CUDA(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
-            MPR_CUDA(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-            MPR_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
-        }
+        chain_ranges(c, cr);
+        MPR_CUDA(cudaMemsetAsync(c->d_stats, 0, sizeof(TileStats), s));
+        MPR_CUDA(launch_tile_tables(c->d_img, c->d_tiles, g.n_tiles, d_gap, tx, ty, c->d_slot_pos,
+                                    c->d_slot_map, c->d_halo, g.halo_cap, c->d_samp, (float)c->p.q,
+                                    c->p.model == MPR_MODEL_GMRF ? 1 : 0, c->p.literal_or ? 1 : 0,
+                                    c->d_slot_ref, c->d_slot_cs, tiled_pairs(cr[0].group), c->d_stats, s));
     }
-    long long maxn = 0;
-    for (int i = 0; i < n_img; ++i) maxn = std::max(maxn, (long long)Lx[i] * Ly[i]);
-    map_kernel<<<dim3(grid_for(maxn, 256, 2048), n_img), 256, 0, s>>>(c->d_img, d_z, d_gap, c->d_samp,
-                                                                      unconditional ? 1 : 0);
-    MPR_CUDA(cudaGetLastError());
-    if (tiled)
-        MPR_CUDA(launch_tile_const(c->d_img, c->d_tiles, g.n_tiles, tx, ty, c->d_slot_pos,
-                                   c->d_halo, g.halo_cap, c->d_samp, (float)c->p.q,
-                                   c->p.model == MPR_MODEL_GMRF ? 1 : 0, c->d_slot_ref,
-                                   c->d_slot_cs, s));
     const uint2 key = make_uint2((uint32_t)c->p.seed, (uint32_t)(c->p.seed >> 32));
     for (int i = 0; i < n_img; ++i) {
         if (tiled) {
             // the temperature lattices start cold (see mpr_estimate_T), images hot
-            hot_start_tiled_kernel<<<grid_for(c->slots[i] * state_chains(g) / 2), 256, 0, s>>>(
-                c->d_img, c->d_slot_pos, c->d_state, c->slots[i], i, n_chains, key, c->img_tag,
-                unconditional ? 1 : 0);
+            MPR_CUDA(launch_hot_start(c->d_img, c->d_slot_pos, c->d_state, c->slots[i], i, n_chains, key,
+                                      c->img_tag, unconditional, s));
         } else {
             init_plain_kernel<<<grid_for((long long)Lx[i] * Ly[i] * n_chains), 256, 0, s>>>(
                 c->d_img, c->d_samp, c->d_state, i, n_chains, key, c->img_tag);
@@ -1132,33 +980,39 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
     MPR_CUDA(cudaMemsetAsync(c->d_ctl, 0, sizeof(Control), s));
     MPR_CUDA(cudaMemsetAsync(c->d_acc1, 0, sizeof(double) * c->L.n_slots, s));
     MPR_CUDA(cudaMemsetAsync(c->d_acc2, 0, sizeof(double) * c->L.n_slots, s));
-
-    // sample specific energy
     if (!unconditional) {
         double* sums = scratch + 2 * n_img;
         unsigned long long* npairs = reinterpret_cast<unsigned long long*>(scratch + 3 * n_img);
         MPR_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * 2 * n_img, s));
-        sample_energy_kernel<<<dim3(grid_for(maxn, 256, 1024), n_img), 256, 0, s>>>(
-            c->d_img, c->d_samp, c->p.q, c->p.J, c->p.model == MPR_MODEL_GMRF ? 1 : 0, sums, npairs);
-        MPR_CUDA(cudaGetLastError());
-        std::vector<double> h_sums(n_img);
-        std::vector<unsigned long long> h_np(n_img);
-        MPR_CUDA(cudaMemcpyAsync(h_sums.data(), sums, sizeof(double) * n_img, cudaMemcpyDeviceToHost, s));
-        MPR_CUDA(cudaMemcpyAsync(h_np.data(), npairs, sizeof(unsigned long long) * n_img,
-                                 cudaMemcpyDeviceToHost, s));
-        MPR_CUDA(cudaStreamSynchronize(s));
-        for (int i = 0; i < n_img; ++i) {
-            ImgDev& I = c->h_img[i];
-            I.n_sp = (long long)h_np[i];
-            I.E_ss = h_sums[i];
-            I.e_s = I.n_sp > 0 ? h_sums[i] / (double)I.n_sp : std::nan("");
-        }
-        MPR_CUDA(cudaMemcpyAsync(c->d_img, c->h_img.data(), sizeof(ImgDev) * n_img,
-                                 cudaMemcpyHostToDevice, s));
+        MPR_CUDA(launch_sample_energy(c->d_img, n_img, maxn, c->d_samp, (float)c->p.q, (float)c->p.J,
+                                      c->p.model == MPR_MODEL_GMRF ? 1 : 0, sums, npairs, s));
     }
     c->sweep = 0;
     c->equil_index = 0;
     c->n_meas_done = 0;
+    return MPR_OK;
+}
+
+// What init_impl left on the device: the images' sample energies, the largest tiles and
+// with them the launches of a sweep.  Blocking.
+mpr_status init_finish(mpr_ctx* c, cudaStream_t s) {
+    const Geometry& g = c->g;
+    const bool tiled = g.path == MPR_PATH_TILED;
+    TileStats st{};
+    if (!c->unconditional)
+        MPR_CUDA(cudaMemcpyAsync(c->h_img.data(), c->d_img, sizeof(ImgDev) * g.n_img, cudaMemcpyDeviceToHost, s));
+    if (tiled) MPR_CUDA(cudaMemcpyAsync(&st, c->d_stats, sizeof(st), cudaMemcpyDeviceToHost, s));
+    MPR_CUDA(cudaStreamSynchronize(s));
+    if (!tiled) return MPR_OK;
+    MPR_TRY(split_tiles(c, st, s));
+    MPR_TRY(choose_resident(c, st, s));
+    ChainRange cr[2];
+    const bool extra = c->n_light[0] < g.n_tiles || c->n_light[1] < g.n_tiles || chain_ranges(c, cr) > 1;
+    if (extra && !c->side) {
+        MPR_CUDA(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+        MPR_CUDA(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+        MPR_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+    }
     return MPR_OK;
 }
 
@@ -1504,7 +1358,11 @@ mpr_status mpr_init_grid(mpr_ctx** out, int n_img, const int* Lx, const int* Ly,
     }
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     mpr_status st = init_impl(c, n_img, Lx, Ly, n_chains, z, gap, where, workspace, ws_bytes, false, s);
-    if (st != MPR_OK) { delete c; return st; }
+    if (st != MPR_OK) {
+        cudaStreamSynchronize(s);  // (what is enqueued reads the caller's buffers)
+        delete c;
+        return st;
+    }
     // unconditional lattices of the temperature estimate
     c->sub = new (std::nothrow) mpr_ctx();
     if (!c->sub) { delete c; return fail(MPR_ERR_INVALID_ARG, "out of host memory"); }
@@ -1521,11 +1379,18 @@ mpr_status mpr_init_grid(mpr_ctx** out, int n_img, const int* Lx, const int* Ly,
     if (st == MPR_OK)
         st = init_impl(c->sub, n_img, LT.data(), LT.data(), c->topt.chains, nullptr, nullptr,
                        MPR_DEVICE, c->ws + c->L.sub, sub_bytes, true, s);
+    // (everything is enqueued before the host waits)
+    if (st == MPR_OK) st = init_finish(c, s);
+    if (st == MPR_OK) st = init_finish(c->sub, s);
     if (st == MPR_OK) {
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = fail(MPR_ERR_CUDA, cudaGetErrorString(e));
     }
-    if (st != MPR_OK) { delete c; return st; }
+    if (st != MPR_OK) {
+        cudaStreamSynchronize(s);
+        delete c;
+        return st;
+    }
     *out = c;
     return MPR_OK;
 }
@@ -1640,7 +1505,7 @@ mpr_status mpr_autotune(int n_img, const int* Lx, const int* Ly, int n_chains, m
             mpr_default_T_opts(&c.topt);
             // the candidate must fit the workspace and the tile's per-lane limit
             if (init_impl(&c, n_img, Lx, Ly, n_chains, z, gap, where, workspace, ws_bytes, false,
-                          s) != MPR_OK)
+                          s) != MPR_OK || init_finish(&c, s) != MPR_OK)
                 continue;
             std::vector<double> T(n_img);
             for (int i = 0; i < n_img; ++i) {
@@ -1707,6 +1572,7 @@ mpr_status mpr_eT_table(int L, int n_T, const double* T, int chains, int n_equil
     std::vector<int> Ls(n_T, L);
     MPR_TRY(init_impl(&u, n_T, Ls.data(), Ls.data(), chains, nullptr, nullptr, MPR_DEVICE, workspace,
                       ws_bytes, true, s));
+    MPR_TRY(init_finish(&u, s));
     u.img_tag = 1u << 29;  // a stream of its own
     MPR_CUDA(cudaMemcpyAsync(u.d_newton, T, sizeof(double) * n_T, cudaMemcpyHostToDevice, s));
     set_T_kernel<<<grid_for(n_T), 256, 0, s>>>(u.d_img, u.d_newton, n_T);

@@ -129,19 +129,52 @@ bool tiled_config_supported(int tile_x, int tile_y);
 // the printed over-relaxation and the GMRF model run with 16 x 16 tiles
 bool tiled_model_supported(int tile_x, int tile_y, int flags);
 
-// tile-table construction (tiled path)
-cudaError_t launch_tile_count(const ImgDev* img, const TileDesc* tiles, int n_tiles,
-                              const uint8_t* gap, int tile_x, int tile_y, int* counts,
+// What the host reads back of an image before the slot space is laid out: sample
+// extremes (order-preserving encodings; lo starts at 0xFFFFFFFF), gaps, slots.
+struct ImgScan {
+    uint32_t lo, hi;
+    unsigned long long n_gap, slots;
+};
+static_assert(sizeof(ImgScan) <= 4 * sizeof(double), "the scratch holds one per image");
+
+// The batch's largest tiles, by the colour of the pass: table entries, own sites; shared
+// memory of a resident block; tiles of the light launch.
+struct TileStats {
+    int gt[2], n_cap[2];
+    unsigned res_smem;
+    int n_light[2], pad;
+};
+constexpr int kTileSizes = 640;  // sizes of a tile: at most 512 + 64 + 1 table entries
+
+// initialisation (mpr_setup.cu)
+// bytes (a multiple of 4) of a host record to device memory, by value in launches
+cudaError_t launch_put(void* dst, const void* src, size_t bytes, cudaStream_t s);
+cudaError_t launch_minmax(const ImgDev* img, int n_img, long long max_sites, const float* z,
+                          const uint8_t* gap, ImgScan* scan, cudaStream_t s);
+// tile records and slot segments (scan[i].slots: their total)
+cudaError_t launch_tile_count(const ImgDev* img, int n_img, TileDesc* tiles, int n_tiles,
+                              const uint8_t* gap, int tile_x, int tile_y, int* counts, ImgScan* scan,
                               cudaStream_t s);
-cudaError_t launch_tile_fill(const ImgDev* img, const TileDesc* tiles, int n_tiles,
-                             const uint8_t* gap, int tile_x, int tile_y, uint32_t* slot_pos,
-                             int* slot_map, int2* halo, int halo_cap, cudaStream_t s);
-// per slot: the table entries of its gap neighbours in the pass of its own
-// colour (up, down, left, right; 0 = not a gap) and its sample field
-cudaError_t launch_tile_const(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tile_x,
-                              int tile_y, const uint32_t* slot_pos, const int2* halo, int halo_cap,
-                              const float* samp, float q, int gmrf, uint2* slot_ref,
-                              float4* slot_cs, cudaStream_t s);
+cudaError_t launch_map(const ImgDev* img, int n_img, long long max_sites, const float* z,
+                       const uint8_t* gap, float* samp, bool unconditional, cudaStream_t s);
+// slots, ring lists and per-slot constants; res_P: chain pairs per site of a resident block
+cudaError_t launch_tile_tables(const ImgDev* img, TileDesc* tiles, int n_tiles, const uint8_t* gap,
+                               int tile_x, int tile_y, uint32_t* slot_pos, int* slot_map, int2* halo,
+                               int halo_cap, const float* samp, float q, int gmrf, int literal,
+                               uint2* slot_ref, float4* slot_cs, int res_P, TileStats* stats,
+                               cudaStream_t s);
+// tiles by size: [colour][table entries, own sites][kTileSizes], added to hist
+cudaError_t launch_tile_hist(const TileDesc* tiles, int n_tiles, int* hist, cudaStream_t s);
+// per colour the list of the light tiles (at most e_max entries and own_max sites), then the others
+cudaError_t launch_tile_split(const TileDesc* tiles, int n_tiles, const int e_max[2], const int own_max[2],
+                              int* list, int* n_light, cudaStream_t s);
+cudaError_t launch_hot_start(const ImgDev* img, const uint32_t* slot_pos, float* state, long long slots,
+                             int img_i, int n_chains, uint2 key, uint32_t img_tag, bool cold,
+                             cudaStream_t s);
+// e_s, E_ss and n_sp of every image (sums, npairs: zeroed scratch)
+cudaError_t launch_sample_energy(ImgDev* img, int n_img, long long max_sites, const float* samp, float q,
+                                 float J, int gmrf, double* sums, unsigned long long* npairs,
+                                 cudaStream_t s);
 // Dynamic shared memory of a colour-pass block of tile shape tx x ty for a
 // launch whose largest tiles have gt table entries and n_cap own sites; flags: the model bits of
 // SweepFlags (kLiteralOR, kGMRF).

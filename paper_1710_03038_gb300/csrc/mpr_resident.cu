@@ -13,36 +13,38 @@ Kernel pick(bool acc, bool energy, bool gmrf) {
 
 }  // namespace resident
 
-size_t resident_smem(const TileDesc& t, int P, bool gmrf) {
-    using namespace resident;
-    const size_t n = (size_t)t.cnt[0] + t.cnt[1];
-    const size_t cells = n + t.halo_cnt[0] + t.halo_cnt[1] + 2;
-    return kFixed + 32 * n + sum_bytes(std::max(t.cnt[0], t.cnt[1])) +
-           std::max(cells * P * (gmrf ? 8 : 16) + 2 * n, sizeof(double) * kNT);  // (a recorder: one each)
-}
-
 int resident_recorders(int group) { return (group + resident::kRecorderChains - 1) / resident::kRecorderChains; }
 
-cudaError_t resident_blocks(size_t smem, bool gmrf, long long* blocks) {
-    using namespace resident;
+cudaError_t resident_blocks(size_t smem, long long* blocks) {
     *blocks = 0;
-    int dev = 0, sms = 0, coop = 0, most = 0;
+    int dev = 0, sms = 0, coop = 0, most = 0, sm_bytes = 0, reserved = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const auto get = [&](int* v, cudaDeviceAttr a) {
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(v, a, dev);
+    };
+    get(&sms, cudaDevAttrMultiProcessorCount);
+    get(&coop, cudaDevAttrCooperativeLaunch);
+    get(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin);
+    get(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor);
+    get(&reserved, cudaDevAttrReservedSharedMemoryPerBlock);
     if (e != cudaSuccess || !coop || smem > (size_t)most) return e;
-    int least = 1 << 30;
-    for (int v = 0; v < 4; ++v) {
-        const void* f = reinterpret_cast<const void*>(pick(v & 1, v & 2, gmrf));
-        int per = 0;
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, kNT, smem);
-        if (e != cudaSuccess) return e;
-        least = std::min(least, per);
-    }
-    *blocks = (long long)least * sms;
+    // (shared memory is given out in units of 128 bytes)
+    const size_t block = (smem + 127) / 128 * 128 + (size_t)reserved;
+    *blocks = (long long)std::min((size_t)resident::kBlocksPerSM, (size_t)sm_bytes / block) * sms;
     return cudaSuccess;
+}
+
+cudaError_t resident_prepare(bool gmrf) {
+    static bool done[2] = {false, false};
+    if (done[gmrf]) return cudaSuccess;
+    int dev = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    for (int v = 0; v < 4 && e == cudaSuccess; ++v)
+        e = cudaFuncSetAttribute(reinterpret_cast<const void*>(resident::pick(v & 1, v & 2, gmrf)),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    done[gmrf] = e == cudaSuccess;
+    return e;
 }
 
 cudaError_t launch_resident(const ResidentArgs& ra, int n_groups, size_t smem, cudaStream_t s) {

@@ -24,13 +24,27 @@ struct ResidentArgs {
     uint32_t* epoch;       // epoch of the last launch's last pass
 };
 
-// Shared memory of a block of tile t with P chain pairs per site.
-size_t resident_smem(const TileDesc& t, int P, bool gmrf);
+// Shared memory of a block: the fixed part, the own sites' records and sums, the two
+// tables and the sites' packet places, for a tile of n0 red and n1 black sites with h0
+// and h1 ring cells and P chain pairs per site.
+constexpr int kResidentFixed = 2304;
+__host__ __device__ inline unsigned resident_sum_bytes(int n_max) {
+    return (40u * (unsigned)n_max + 15u) / 16u * 16u;
+}
+__host__ __device__ inline unsigned resident_smem(int n0, int n1, int h0, int h1, int P, bool gmrf) {
+    const unsigned n = (unsigned)(n0 + n1);
+    const unsigned tables = (n + (unsigned)(h0 + h1) + 2u) * (unsigned)P * (gmrf ? 8u : 16u) + 2u * n;
+    // (a block that records energies: a double per thread)
+    return (unsigned)kResidentFixed + 32u * n + resident_sum_bytes(n0 > n1 ? n0 : n1) +
+           (tables > 1024u ? tables : 1024u);
+}
 // Blocks that record the energies of a group of that many chains.
 int resident_recorders(int group);
 // Blocks of that size that the device holds at once (0: no cooperative launches, or
-// one block does not fit); sets the kernels' shared-memory limit.
-cudaError_t resident_blocks(size_t smem, bool gmrf, long long* blocks);
+// one block does not fit).
+cudaError_t resident_blocks(size_t smem, long long* blocks);
+// Sets the kernels' shared-memory limit (not during a capture).
+cudaError_t resident_prepare(bool gmrf);
 cudaError_t launch_resident(const ResidentArgs& ra, int n_groups, size_t smem, cudaStream_t s);
 
 namespace resident {

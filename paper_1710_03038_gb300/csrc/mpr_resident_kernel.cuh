@@ -77,9 +77,8 @@ struct Fixed {
     int ring[2][kRing];  // ring cells: packet index (tile, place) of the cell's site
     int slot[kRing];     // ring cells of the first red pass: their slots
 };
-constexpr size_t kFixed = (sizeof(Fixed) + 15) / 16 * 16;
-
-__host__ __device__ inline unsigned sum_bytes(int nmax) { return (40u * (unsigned)nmax + 15u) / 16u * 16u; }
+constexpr size_t kFixed = kResidentFixed;
+static_assert(sizeof(Fixed) <= kFixed && kFixed % 16 == 0, "fixed part of the shared memory");
 
 // A tile's packets: top row 0-15, bottom row 16-31, left column 32-47, right column
 // 48-63 (a corner site has two).
@@ -210,7 +209,7 @@ __device__ __forceinline__ bool run_tile(const ResidentArgs& ra, unsigned char* 
         const int n0 = T.cnt[0], n1 = T.cnt[1], nmax = max(n0, n1);
         uint4* cons = rows + n0 + n1;
         const unsigned acc0 = (unsigned)(kFixed + 32 * (n0 + n1));
-        const unsigned tab0 = acc0 + (ACC ? sum_bytes(nmax) : 0u);
+        const unsigned tab0 = acc0 + (ACC ? resident_sum_bytes(nmax) : 0u);
         const unsigned tab1 = tab0 + (unsigned)(1 + n1 + T.halo_cnt[0]) * kRow;
         const unsigned edge0 = tab1 + (unsigned)(1 + n0 + T.halo_cnt[1]) * kRow;
         uint16_t* edge = reinterpret_cast<uint16_t*>(smem + edge0);
@@ -264,7 +263,7 @@ __device__ __forceinline__ bool run_tile(const ResidentArgs& ra, unsigned char* 
             else *reinterpret_cast<float4*>(z) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
         if (ACC)
-            for (unsigned j = tid; j < sum_bytes(nmax) / 4; j += kNT)
+            for (unsigned j = tid; j < resident_sum_bytes(nmax) / 4; j += kNT)
                 reinterpret_cast<uint32_t*>(smem + acc0)[j] = 0u;
         const long long chain0 = (long long)T.img * a.n_chains + r0;
         if (tid < 32) {
