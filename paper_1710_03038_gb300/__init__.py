@@ -136,8 +136,13 @@ class Context:
         self.chains = int(chains)
         on_dev = isinstance(zs[0], torch.Tensor) and zs[0].is_cuda
         if on_dev:
-            zf = torch.cat([t.reshape(-1).to(torch.float32) for t in zs]).contiguous()
-            gf = torch.cat([(t.reshape(-1) != 0).to(torch.uint8) for t in gs]).contiguous()
+            # (one image of the library's types is read in place: any nonzero mask byte is a gap)
+            zf = [t.reshape(-1).to(torch.float32) for t in zs]
+            gf = [t.reshape(-1) for t in gs]
+            gf = [t.view(torch.uint8) if t.dtype in (torch.uint8, torch.bool) else (t != 0).to(torch.uint8)
+                  for t in gf]
+            zf = torch.cat(zf) if len(zf) > 1 else zf[0].contiguous()
+            gf = torch.cat(gf) if len(gf) > 1 else gf[0].contiguous()
             where = _lib.MPR_DEVICE
             ng = [int(g.count_nonzero()) for g in gs]
         elif (len(zs) == 1 and isinstance(zs[0], torch.Tensor) and isinstance(gs[0], torch.Tensor)

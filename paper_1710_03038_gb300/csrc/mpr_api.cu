@@ -1832,7 +1832,8 @@ static mpr_status state_copy(mpr_ctx* c, float* phi, mpr_mem where, int dir, cud
         long long maxn = 0;
         for (int i = 0; i < c->g.n_img; ++i) maxn = std::max(maxn, (long long)c->g.Lx[i] * c->g.Ly[i]);
         if (tiled) {
-            MPR_CUDA(launch_state_tiles(c->d_img, c->d_tiles, c->g.n_tiles, c->g.tx, c->g.ty, c->d_slot_pos,
+            MPR_CUDA(launch_state_tiles(c->d_img, c->d_tiles, c->g.n_tiles, c->g.tx, c->g.ty,
+                                        std::min(c->g.tx * c->g.ty, c->n_cap[0] + c->n_cap[1]), c->d_slot_pos,
                                         c->d_samp, c->d_state, c->g.n_chains, phi, dir == 1, s));
             return MPR_OK;
         }

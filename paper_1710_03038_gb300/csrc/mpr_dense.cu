@@ -61,15 +61,16 @@ predict_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int np
 }
 
 // States of 32 chains of a tile <-> dense planes (SET: the gap sites only), through
-// shared memory: rows of 32 chains on one side, rows of the tile on the other
-// (2048^2 x 32 chains out: 1020 us before, a chain at a time).
+// shared memory: rows of 32 chains on one side, rows of the tile on the other.  Bound by
+// the plane rows (64 bytes each); shared memory is sized by the batch's fullest tile, so
+// that eight blocks share an SM.
 template <bool SET>
 __global__ void __launch_bounds__(256)
 state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix,
-                  const uint32_t* __restrict__ slot_pos, const float* __restrict__ samp,
+                  int n_max, const uint32_t* __restrict__ slot_pos, const float* __restrict__ samp,
                   float* __restrict__ state, int n_chains, float* __restrict__ dense) {
-    extern __shared__ float rows[];  // [sites of the tile][33], then the tile's map
-    uint16_t* map = reinterpret_cast<uint16_t*>(rows + npix * 33);  // pixel -> site, 0xFFFF: a sample
+    extern __shared__ float rows[];  // [sites of the tile, at most n_max][33], then the tile's map
+    uint16_t* map = reinterpret_cast<uint16_t*>(rows + n_max * 33);  // pixel -> site, 0xFFFF: a sample
     const TileDesc T = tiles[blockIdx.x];
     const ImgDev& I = img[T.img];
     const int Lx = I.Lx, Ly = I.Ly, n = T.cnt[0] + T.cnt[1];
@@ -84,7 +85,7 @@ state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix
     }
     float* st = state + T.state_off + r0 + lane;
     if (!SET && lane < nr) {
-#pragma unroll 4
+#pragma unroll 8
         for (int j = warp; j < n; j += 8) rows[j * 33 + lane] = st[(long long)slot_of(j) * T.cp];
     }
     __syncthreads();
@@ -100,14 +101,14 @@ state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix
             if (m == 0xFFFF) continue;
             float* row = rows + m * 33;
 #pragma unroll 8
-            for (int r = 0; r < nr; ++r, d += plane) row[r] = *d;
+            for (int r = 0; r < nr; ++r, d += plane) row[r] = __ldcs(d);
         } else if (m == 0xFFFF) {
             const float v = samp[I.site_off + site];
-            for (int r = 0; r < nr; ++r, d += plane) *d = v;
+            for (int r = 0; r < nr; ++r, d += plane) __stcs(d, v);
         } else {
             const float* row = rows + m * 33;
 #pragma unroll 8
-            for (int r = 0; r < nr; ++r, d += plane) *d = row[r];
+            for (int r = 0; r < nr; ++r, d += plane) __stcs(d, row[r]);
         }
     }
     if (SET) {
@@ -198,17 +199,17 @@ cudaError_t launch_predict_tiles(const ImgDev* img, const TileDesc* tiles, int n
 }
 
 cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tx, int ty,
-                               const uint32_t* slot_pos, const float* samp, float* state, int n_chains,
-                               float* dense, bool set, cudaStream_t s) {
-    const size_t smem = (size_t)tx * ty * (33 * sizeof(float) + sizeof(uint16_t));
+                               int n_max, const uint32_t* slot_pos, const float* samp, float* state,
+                               int n_chains, float* dense, bool set, cudaStream_t s) {
+    const size_t smem = (size_t)n_max * 33 * sizeof(float) + (size_t)tx * ty * sizeof(uint16_t);
     const auto kernel = set ? state_tile_kernel<true> : state_tile_kernel<false>;
-    if (smem > 48 * 1024) {  // 32 x 16 and 32 x 32 tiles
+    if (smem > 48 * 1024) {  // (32 x 16 and 32 x 32 tiles)
         const cudaError_t e =
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kernel<<<dim3(n_tiles, (n_chains + 31) / 32), 256, smem, s>>>(img, tiles, log2_of(tx), tx * ty, slot_pos,
-                                                                  samp, state, n_chains, dense);
+    kernel<<<dim3(n_tiles, (n_chains + 31) / 32), 256, smem, s>>>(img, tiles, log2_of(tx), tx * ty, n_max,
+                                                                  slot_pos, samp, state, n_chains, dense);
     return cudaGetLastError();
 }
 

@@ -190,8 +190,8 @@ cudaError_t launch_predict_tiles(const ImgDev* img, const TileDesc* tiles, int n
                                  const double* acc2, const float* z, const uint8_t* gap,
                                  double n_samples, float* zhat, float* zstd, cudaStream_t s);
 cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tile_x,
-                               int tile_y, const uint32_t* slot_pos, const float* samp, float* state,
-                               int n_chains, float* dense, bool set, cudaStream_t s);
+                               int tile_y, int n_max, const uint32_t* slot_pos, const float* samp,
+                               float* state, int n_chains, float* dense, bool set, cudaStream_t s);
 cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles,
                                 int tile_x, int tile_y, const float* state, const float* samp,
                                 const int* slot_map, int n_chains, float q, float J, int gmrf,

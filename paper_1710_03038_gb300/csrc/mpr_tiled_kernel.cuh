@@ -44,8 +44,7 @@
 // (some pairs of a group may be missing), kWhole (every group has 2P chains: no test
 // of a pair's existence) and kOnly (the 2P chains of the one group are all there are:
 // slots lie 2P floats apart, a constant).  2048^2 x 32, ms per equilibration sweep: all
-// three read at run time 0.2867, ENERGY compiled in 0.2655, kOnly 0.2556.  Passes
-// that record energies run as kRagged: one variant less for rare passes.
+// three read at run time 0.2867, ENERGY compiled in 0.2655, kOnly 0.2556.
 //
 // Models.  kModelMPR: the MPR bond with the q-consistent over-relaxation;
 // kModelLIT: the over-relaxation as printed (q = 1 field; the table cell
@@ -495,26 +494,34 @@ cudaError_t launch_one(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     return cudaGetLastError();
 }
 
-template <int TX, int TY, int NW, int P, bool ACC, int MODEL>
-cudaError_t launch_acc(const SweepArgs& a, cudaStream_t s, bool setup_only) {
+template <int TX, int TY, int NW, int P, bool ACC, int MODEL, bool ENERGY>
+cudaError_t launch_groups(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     // the variants for whole groups exist for 16 x 16 tiles, the shape of every
     // automatic choice
     constexpr bool kVariants = TX == 16 && TY == 16 && MODEL != kModelLIT;
     constexpr int kW = kVariants ? kWhole : kRagged, kO = kVariants ? kOnly : kRagged;
     if (setup_only) {
-        cudaError_t e = launch_one<TX, TY, NW, P, ACC, MODEL, true, kRagged>(a, s, true);
-        if (e == cudaSuccess) e = launch_one<TX, TY, NW, P, ACC, MODEL, false, kRagged>(a, s, true);
-        if (e == cudaSuccess) e = launch_one<TX, TY, NW, P, ACC, MODEL, false, kW>(a, s, true);
-        if (e == cudaSuccess) e = launch_one<TX, TY, NW, P, ACC, MODEL, false, kO>(a, s, true);
+        cudaError_t e = launch_one<TX, TY, NW, P, ACC, MODEL, ENERGY, kRagged>(a, s, true);
+        if (e == cudaSuccess) e = launch_one<TX, TY, NW, P, ACC, MODEL, ENERGY, kW>(a, s, true);
+        if (e == cudaSuccess) e = launch_one<TX, TY, NW, P, ACC, MODEL, ENERGY, kO>(a, s, true);
         return e;
     }
-    if (a.flags & kEnergy) return launch_one<TX, TY, NW, P, ACC, MODEL, true, kRagged>(a, s, false);
     const bool whole = a.chain_group == 2 * P && (a.chain_end - a.chain0) % (2 * P) == 0;
     // (slots are a multiple of 4 floats apart)
     if (whole && a.n_chains == 2 * P && P % 2 == 0)
-        return launch_one<TX, TY, NW, P, ACC, MODEL, false, kO>(a, s, false);
-    if (whole) return launch_one<TX, TY, NW, P, ACC, MODEL, false, kW>(a, s, false);
-    return launch_one<TX, TY, NW, P, ACC, MODEL, false, kRagged>(a, s, false);
+        return launch_one<TX, TY, NW, P, ACC, MODEL, ENERGY, kO>(a, s, false);
+    if (whole) return launch_one<TX, TY, NW, P, ACC, MODEL, ENERGY, kW>(a, s, false);
+    return launch_one<TX, TY, NW, P, ACC, MODEL, ENERGY, kRagged>(a, s, false);
+}
+
+template <int TX, int TY, int NW, int P, bool ACC, int MODEL>
+cudaError_t launch_acc(const SweepArgs& a, cudaStream_t s, bool setup_only) {
+    if (setup_only) {
+        cudaError_t e = launch_groups<TX, TY, NW, P, ACC, MODEL, false>(a, s, true);
+        return e != cudaSuccess ? e : launch_groups<TX, TY, NW, P, ACC, MODEL, true>(a, s, true);
+    }
+    if (a.flags & kEnergy) return launch_groups<TX, TY, NW, P, ACC, MODEL, true>(a, s, false);
+    return launch_groups<TX, TY, NW, P, ACC, MODEL, false>(a, s, false);
 }
 
 template <int TX, int TY, int NW, int P, int MODEL>

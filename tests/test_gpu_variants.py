@@ -67,9 +67,10 @@ def big_run(path, R, cg, model="mpr", n=2):
     ctx.set_T([0.1])
     ctx.sweep(n, "equil")
     ctx.sweep(1, "equil", record_energy=True)
+    e = ctx.chain_info()["e_last"]
     ctx.sweep(n, "measure")
     info = ctx.chain_info()
-    return ctx.get_state()[0], info, ctx.predict()[0]
+    return ctx.get_state()[0], dict(info, e_last=e), ctx.predict()[0]
 
 
 @pytest.mark.parametrize("R,cg,model", [(4, 4, "mpr"), (8, 8, "mpr"), (16, 16, "mpr"), (32, 32, "mpr"),
@@ -80,6 +81,7 @@ def test_launches_per_colour_equal_the_plain_path(R, cg, model):
     assert torch.equal(got[0], want[0])
     for k in ("a", "accepted"):
         assert np.array_equal(got[1][k], want[1][k])
+    assert np.allclose(got[1]["e_last"], want[1]["e_last"], rtol=0, atol=1e-6)
     assert torch.allclose(got[2], want[2], rtol=1e-6, atol=1e-5)
 
 
@@ -134,3 +136,45 @@ def test_resident_runs_in_a_caller_capture_and_on_two_streams():
     for ctx, w in zip(ctxs, want):
         for a, b in zip(ctx.get_state(), w):
             assert np.array_equal(a.cpu().numpy(), b)
+
+
+# ------------------------------------------------------------------- dense views
+
+@pytest.mark.parametrize("tile", [(16, 16), (32, 16), (32, 32)])
+@pytest.mark.parametrize("R", [1, 33])
+def test_dense_views_of_every_tile_shape(tile, R):
+    """States, energies and predictions, one tile per block, against torch in FP64: ragged
+    images, a tile that is all gap, one chain and a second group of chains."""
+    zs, gs = images()
+    ctx = mpr.Context(zs, gs, chains=R, params=mpr.Params(seed=9, tile=tile))
+    ctx.set_T([0.2, 0.05, 0.4])
+    start = ctx.get_state()
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    new = [torch.rand(s.shape, device="cuda", generator=gen) * 6.28 for s in start]
+    ctx.set_state(new)
+    H = ctx.energy()
+    for i, (s, n, g) in enumerate(zip(ctx.get_state(), new, gs)):
+        gap = torch.from_numpy(g).cuda() != 0
+        assert torch.equal(s[:, gap], n[:, gap])                   # gaps as set
+        assert torch.equal(s[:, ~gap], start[i][:, ~gap])          # samples as mapped
+        d = s.double()
+        want = -(torch.cos(0.5 * (d[:, 1:] - d[:, :-1])).sum((1, 2)) +
+                 torch.cos(0.5 * (d[:, :, 1:] - d[:, :, :-1])).sum((1, 2)))
+        h, w = g.shape
+        want /= h * (w - 1) + w * (h - 1)
+        # FP32 differences and cosines of angles below 2 pi: 5e-7 a bond
+        assert np.max(np.abs(H[i] - want.cpu().numpy())) < 5e-7
+    ctx.sweep(5, "measure")
+    s1, s2, n = ctx.accumulators()
+    zh, sd = ctx.predict(std=True)
+    info = ctx.image_info()
+    for i, g in enumerate(gs):
+        gap = torch.from_numpy(g).cuda() != 0
+        scale = (float(info["zmax"][i]) - float(info["zmin"][i])) / (2 * np.pi)
+        m = s1[i] / n
+        want = torch.where(gap, float(info["zmin"][i]) + scale * m, torch.from_numpy(zs[i]).cuda().double())
+        assert torch.equal(zh[i], want.float()) or (zh[i] - want.float()).abs().max() <= 4e-6 * want.abs().max()
+        v = torch.sqrt((s2[i] / n - m * m).clamp(min=0)) * scale
+        v = torch.where(gap, v, torch.zeros_like(v))
+        # the variance is a difference of sums of up to 40 rad^2 in FP64 (1e-14): 1e-7 rad
+        assert (sd[i].double() - v).abs().max() < 1e-6 * scale + 2e-7 * float(v.max())
