@@ -91,7 +91,29 @@ state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix
     __syncthreads();
     const long long plane = (long long)Lx * Ly;
     float* d0 = dense + I.site_off * n_chains + r0 * plane;
-    for (int i = threadIdx.x; i < npix; i += 256) {
+    // out, four pixels of a row at a time, where every plane's rows start on 16 bytes and the
+    // tile is whole in x (2048^2 x 32: 256 -> 160 us)
+    const bool quads = !SET && T.x0 + (1 << tx_log) <= Lx && Lx % 4 == 0 && I.site_off % 4 == 0 &&
+                       (reinterpret_cast<uintptr_t>(dense) & 15) == 0;
+    for (int i = 4 * (threadIdx.x & 63); quads && i < npix; i += 256) {
+        const int x = T.x0 + (i & ((1 << tx_log) - 1)), y = T.y0 + (i >> tx_log);
+        if (y >= Ly) continue;
+        const long long site = (long long)y * Lx + x;
+        const ushort4 m = *reinterpret_cast<const ushort4*>(map + i);
+        const float4 sample = *reinterpret_cast<const float4*>(samp + I.site_off + site);
+        const auto row = [&](unsigned j) { return rows + (j == 0xFFFFu ? 0u : j * 33u); };
+        const float *a = row(m.x), *b = row(m.y), *c = row(m.z), *d = row(m.w);
+#pragma unroll 4
+        for (int r = threadIdx.x >> 6; r < nr; r += 4) {
+            float4 v = sample;
+            if (m.x != 0xFFFFu) v.x = a[r];
+            if (m.y != 0xFFFFu) v.y = b[r];
+            if (m.z != 0xFFFFu) v.z = c[r];
+            if (m.w != 0xFFFFu) v.w = d[r];
+            *reinterpret_cast<float4*>(d0 + r * plane + site) = v;
+        }
+    }
+    for (int i = threadIdx.x; !quads && i < npix; i += 256) {
         const int x = T.x0 + (i & ((1 << tx_log) - 1)), y = T.y0 + (i >> tx_log);
         if (x >= Lx || y >= Ly) continue;
         const long long site = (long long)y * Lx + x;
@@ -101,14 +123,14 @@ state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix
             if (m == 0xFFFF) continue;
             float* row = rows + m * 33;
 #pragma unroll 8
-            for (int r = 0; r < nr; ++r, d += plane) row[r] = __ldcs(d);
+            for (int r = 0; r < nr; ++r, d += plane) row[r] = *d;
         } else if (m == 0xFFFF) {
             const float v = samp[I.site_off + site];
-            for (int r = 0; r < nr; ++r, d += plane) __stcs(d, v);
+            for (int r = 0; r < nr; ++r, d += plane) *d = v;
         } else {
             const float* row = rows + m * 33;
 #pragma unroll 8
-            for (int r = 0; r < nr; ++r, d += plane) __stcs(d, row[r]);
+            for (int r = 0; r < nr; ++r, d += plane) *d = row[r];
         }
     }
     if (SET) {
@@ -118,43 +140,58 @@ state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix
     }
 }
 
-// H of 32 chains of an image (blockIdx.y, z): a lane is a chain, a block walks tiles.
-// The tile's angles and those right of and below it lie in shared memory, a row of 32
-// chains per pixel.  FP32 bond terms as before; their sum in two FP32 words (TwoSum,
-// Knuth: the rounding error of every addition is kept), FP64 from there: an FP64
-// addition per pixel and chain ran at 1/32 of the rate (1000 x 777 x 24: 177 us before).
-__global__ void __launch_bounds__(256)
+// H of 32 chains of an image (blockIdx.y, z): a lane is a chain, a block walks strips of
+// STRIP rows of a tile.  The strip's angles and those right of and below it lie in
+// shared memory, a row of 32 chains per pixel.  FP32 bond terms as before; their sum in
+// two FP32 words (TwoSum: the rounding error of every addition is kept), FP64 from
+// there: an FP64 addition per pixel and chain ran at 1/32 of the rate.  Bound by the
+// two cosines per pixel and chain; small batches by the chain of a warp's pixels: they
+// take strips of two rows, four warps to a row (64^2 x 32: 23 us with whole tiles).
+template <int STRIP, int NW>
+__global__ void __launch_bounds__(NW * 32)
 energy_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int ty, const float* state,
                    const float* samp, const int* slot_map, int n_chains, float q, float J, int gmrf,
                    double* out) {
-    extern __shared__ float ang[];  // [(ty + 1) x (tx + 1)][32]
-    __shared__ double part[8][32];
+    extern __shared__ float ang[];  // [(STRIP + 1) x (tx + 1)][32]
+    __shared__ double part[NW][32];
+    constexpr int kParts = NW > STRIP ? NW / STRIP : 1;  // warps to a row
     const ImgDev& I = img[blockIdx.z];
-    const int Lx = I.Lx, Ly = I.Ly, tx = 1 << tx_log, ew = tx + 1;
+    const int Lx = I.Lx, Ly = I.Ly, tx = 1 << tx_log, ew = tx + 1, strips = ty / STRIP;
     const int r0 = blockIdx.y * 32, nr = min(32, n_chains - r0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = min(lane, nr - 1);  // idle lanes repeat the last chain
     double sum = 0.0;
-    for (int t = blockIdx.x; t < I.ntiles; t += gridDim.x) {
-        const TileDesc& T = tiles[I.tile0 + t];
-        const int w = min(ew, Lx - T.x0), h = min(ty + 1, Ly - T.y0);  // with the neighbours that exist
+    for (int t = blockIdx.x; t < I.ntiles * strips; t += gridDim.x) {
+        const TileDesc& T = tiles[I.tile0 + t / strips];
+        const int x00 = T.x0, y00 = T.y0 + t % strips * STRIP;
+        // with the neighbours that exist (rows below the image: nothing to do)
+        const int w = min(ew, Lx - x00), h = min(STRIP + 1, Ly - y00);
         __syncthreads();
-        for (int y = warp; y < h; y += 8) {
-            const long long s0 = I.site_off + (long long)(T.y0 + y) * Lx + T.x0;
-#pragma unroll 4
-            for (int x = 0; x < w; ++x) {
-                const int s = slot_map[s0 + x];
-                ang[(y * ew + x) * 32 + lane] = s >= 0 ? state[I.state_off + (long long)s * I.sstride + r0 + r]
-                                                       : samp[s0 + x];
+        for (int y = warp; y < h; y += NW) {
+            // a row's slots and samples by lane, then its cells' rows of chains, all in flight
+            const long long s0 = I.site_off + (long long)(y00 + y) * Lx + x00;
+            for (int x0 = 0; x0 < w; x0 += 32) {
+                const bool in = x0 + lane < w;
+                const int slot = in ? slot_map[s0 + x0 + lane] : -1;
+                const float sample = in ? samp[s0 + x0 + lane] : 0.0f;
+#pragma unroll 8
+                for (int x = 0; x < min(32, w - x0); ++x) {
+                    const int s = __shfl_sync(0xffffffffu, slot, x);
+                    const float v = __shfl_sync(0xffffffffu, sample, x);
+                    ang[(y * ew + x0 + x) * 32 + lane] =
+                        s >= 0 ? state[I.state_off + (long long)s * I.sstride + r0 + r] : v;
+                }
             }
         }
         __syncthreads();
-        const int wi = min(tx, Lx - T.x0), hn = min(ty, Ly - T.y0);
+        const int hn = min(STRIP, Ly - y00), x_lo = warp % kParts * (tx / kParts);
+        const int x_hi = min(x_lo + tx / kParts, Lx - x00);
         float hi = 0.0f, lo = 0.0f;
-        for (int y = warp; y < hn; y += 8) {
+        for (int y = warp / kParts; y < hn; y += NW / kParts) {
             const float* a = ang + y * ew * 32 + lane;
-            float v = a[0];
-            for (int x = 0; x < wi; ++x) {
+            float v = x_lo < x_hi ? a[x_lo * 32] : 0.0f;
+#pragma unroll 4
+            for (int x = x_lo; x < x_hi; ++x) {
                 float e = 0.0f, right = 0.0f;
                 if (x + 1 < w) {
                     right = a[(x + 1) * 32];
@@ -176,7 +213,7 @@ energy_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int ty,
     if (warp == 0 && lane < nr) {
         double s = 0.0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) s += part[k][lane];
+        for (int k = 0; k < NW; ++k) s += part[k][lane];
         atomicAdd(out + (long long)blockIdx.z * n_chains + r0 + lane, s);
     }
 }
@@ -201,6 +238,7 @@ cudaError_t launch_predict_tiles(const ImgDev* img, const TileDesc* tiles, int n
 cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tx, int ty,
                                int n_max, const uint32_t* slot_pos, const float* samp, float* state,
                                int n_chains, float* dense, bool set, cudaStream_t s) {
+    n_max = (n_max + 3) & ~3;  // (the map after the rows starts on 16 bytes)
     const size_t smem = (size_t)n_max * 33 * sizeof(float) + (size_t)tx * ty * sizeof(uint16_t);
     const auto kernel = set ? state_tile_kernel<true> : state_tile_kernel<false>;
     if (smem > 48 * 1024) {  // (32 x 16 and 32 x 32 tiles)
@@ -216,18 +254,23 @@ cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_t
 cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles, int tx,
                                 int ty, const float* state, const float* samp, const int* slot_map,
                                 int n_chains, float q, float J, int gmrf, double* out, cudaStream_t s) {
-    const size_t smem = (size_t)(tx + 1) * (ty + 1) * 32 * sizeof(float);
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(
-            energy_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    // about eight blocks per SM over all images and chain groups
     const int groups = (n_chains + 31) / 32;
-    const int blocks = std::max(1, std::min(max_tiles, 152 * 8 / std::max(1, groups * n_img) + 1));
-    energy_tile_kernel<<<dim3(blocks, groups, n_img), 256, smem, s>>>(
-        img, tiles, log2_of(tx), ty, state, samp, slot_map, n_chains, q, J, gmrf, out);
-    return cudaGetLastError();
+    const auto launch = [&](auto kernel, int strip, int nw, int per_sm) {
+        const size_t smem = (size_t)(tx + 1) * (strip + 1) * 32 * sizeof(float);
+        if (smem > 48 * 1024) {  // (32 x 32 tiles)
+            const cudaError_t e =
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        const long long most = 152LL * per_sm / std::max(1, groups * n_img) + 1;
+        const int blocks = (int)std::max(1LL, std::min((long long)max_tiles * (ty / strip), most));
+        kernel<<<dim3(blocks, groups, n_img), nw * 32, smem, s>>>(img, tiles, log2_of(tx), ty, state, samp,
+                                                                  slot_map, n_chains, q, J, gmrf, out);
+        return cudaGetLastError();
+    };
+    // the line: below four blocks per SM of whole tiles the strips are the shorter chain
+    if ((long long)max_tiles * groups * n_img < 152 * 4) return launch(energy_tile_kernel<2, 8>, 2, 8, 8);
+    return launch(energy_tile_kernel<16, 8>, 16, 8, 8);
 }
 
 }  // namespace mpr

@@ -178,3 +178,24 @@ def test_dense_views_of_every_tile_shape(tile, R):
         v = torch.where(gap, v, torch.zeros_like(v))
         # the variance is a difference of sums of up to 40 rad^2 in FP64 (1e-14): 1e-7 rad
         assert (sd[i].double() - v).abs().max() < 1e-6 * scale + 2e-7 * float(v.max())
+
+
+@pytest.mark.parametrize("shape,R", [((128, 192), 32), ((131, 192), 33), ((100, 190), 32), ((97, 129), 40)])
+def test_states_out_by_quads_and_by_pixels(shape, R):
+    """States of more than 2^18 values: rows of whole quads (sides a multiple of four, whole
+    and cut tiles) and of pixels; an output that starts off a 16-byte boundary."""
+    h, w = shape
+    z = synthetic.grf(shape, nu=0.5, ell=6.0, mean=50, std=10, seed=3).astype(np.float32)
+    g = synthetic.uniform_gaps(shape, 0.4, 5).astype(np.uint8)
+    g[16:32, 16:32] = 1
+    out = []
+    for path in ("plain", "tiled"):
+        ctx = mpr.Context([z], [g], chains=R, params=mpr.Params(seed=5, path=path))
+        out.append((ctx, ctx.get_state()[0]))
+    assert torch.equal(out[0][1], out[1][1])
+    from paper_1710_03038_gb300 import _lib
+    flat = torch.full((R * h * w + 1,), -7.0, device="cuda")
+    _lib.call("mpr_get_state", out[1][0]._ctx, mpr._ptr(flat[1:]), _lib.MPR_DEVICE, mpr._stream_ptr())
+    torch.cuda.synchronize()
+    assert float(flat[0]) == -7.0
+    assert torch.equal(flat[1:].view(R, h, w), out[0][1])
