@@ -20,7 +20,7 @@ namespace mpr {
 struct TileDesc {
     int img;
     int x0, y0;
-    int cp;           // floats per slot of the image's state (chains rounded up to 4)
+    int cp;           // floats per slot of the image's state (chains rounded up)
     int off[2];       // slot offset of the colour-c gap segment inside the image's slot space
     int cnt[2];       // gap sites of colour c in the tile
     int halo_cnt[2];  // other-colour gap sites in the 1-ring seen by the colour-c pass
@@ -36,7 +36,7 @@ struct ImgDev {
     long long site_off;   // offset in concatenated [sum Lx*Ly] arrays
     long long state_off;  // float offset of chain 0, slot 0 in the state buffer
     long long stride;     // floats between consecutive chains (tiled: 1)
-    long long sstride;    // floats between consecutive slots (tiled: chains rounded up to even)
+    long long sstride;    // floats between consecutive slots (tiled: chains rounded up)
     long long slot_off;   // tiled: offset in the slot arrays (acc, slot_pos); plain: site_off
     int tile0, ntiles;
     float zmin, zmax;

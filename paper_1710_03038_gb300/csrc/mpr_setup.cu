@@ -394,7 +394,8 @@ __global__ void __launch_bounds__(256)
 hot_start_kernel(const ImgDev* img, const uint32_t* __restrict__ slot_pos, float* __restrict__ state,
                  long long slots, int img_i, int n_chains, uint2 key, uint32_t img_tag, int cold) {
     const ImgDev& I = img[img_i];
-    const uint32_t nq = (uint32_t)(I.sstride / 4);  // chains in fours per slot
+    const uint32_t nq = (uint32_t)((n_chains + 3) / 4);  // chains in fours per slot
+    const long long row = I.sstride / 4;
     float4* st = reinterpret_cast<float4*>(state + I.state_off);
     const long long total = slots * nq;
     for (long long t = blockIdx.x * 256LL + threadIdx.x; t < total; t += gridDim.x * 256LL) {
@@ -417,7 +418,7 @@ hot_start_kernel(const ImgDev* img, const uint32_t* __restrict__ slot_pos, float
             if (c0 + 2 >= n_chains) v.z = 0.0f;
             if (c0 + 3 >= n_chains) v.w = 0.0f;
         }
-        st[t] = v;
+        st[k * row + c0 / 4] = v;
     }
 }
 

@@ -6,7 +6,7 @@
 // colour form a contiguous segment of the image's slot space (row-major
 // inside the tile, padded to 4 slots).  The state is slot-major with the
 // realisations interleaved: slot k of chain r sits at k * CP + r, CP being the
-// chain count rounded up to a multiple of 4, so the pair (2m, 2m + 1) of one
+// chain count rounded up (see state_chains), so the pair (2m, 2m + 1) of one
 // slot is one aligned float2 and the pairs of a chain group are contiguous.
 //
 // Work.  One thread block takes one tile and a group of 2P chains (P pairs).
@@ -514,13 +514,34 @@ cudaError_t launch_groups(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     return launch_one<TX, TY, NW, P, ACC, MODEL, ENERGY, kRagged>(a, s, false);
 }
 
+// Warps of a block where the chain groups are small.  With few pairs a block of four
+// warps has one or two steps per warp between its waits; fewer warps per block and more
+// blocks per SM overlap the waits better, as long as the blocks' tables leave room for
+// nearly as many warps.  us per equilibration / sampling sweep, four warps -> fewer:
+// 2048^2 at 40 % x 4 chains 83 / 99 -> 61 / 61 (one warp), x 16 159 / 173 -> 143 / 156
+// (two); x 8 sampling 128 -> 102, but equilibration 57 -> 62 at 1500^2 x 7: two warps for
+// sampling only; 1024^2 at 50 % x 16 sampling 51 -> 53 with 24 warps per SM: 26 asked for.
+// Passes that record energies keep the four warps, which fix the order of their sums,
+// and so do launches beside another (1024^2 x 100: 276 -> 285).
+constexpr int small_group_warps(int P, bool acc) {
+    return P == 2 ? 1 : P == 4 && acc ? 2 : P == 8 ? 2 : 4;
+}
+constexpr int kSmallGroupSmWarps = 26;
+
 template <int TX, int TY, int NW, int P, bool ACC, int MODEL>
 cudaError_t launch_acc(const SweepArgs& a, cudaStream_t s, bool setup_only) {
+    constexpr int kFew = TX == 16 && TY == 16 && MODEL != kModelLIT ? small_group_warps(P, ACC) : NW;
     if (setup_only) {
         cudaError_t e = launch_groups<TX, TY, NW, P, ACC, MODEL, false>(a, s, true);
+        if (e == cudaSuccess && kFew != NW) e = launch_groups<TX, TY, kFew, P, ACC, MODEL, false>(a, s, true);
         return e != cudaSuccess ? e : launch_groups<TX, TY, NW, P, ACC, MODEL, true>(a, s, true);
     }
     if (a.flags & kEnergy) return launch_groups<TX, TY, NW, P, ACC, MODEL, true>(a, s, false);
+    constexpr size_t kSmBytes = 228 * 1024, kReserved = 1024;  // of an SM, per block
+    if (kFew != NW && a.chain_end - a.chain0 == a.n_chains &&
+        (Cfg<TX, TY, kFew, MODEL>::smem_for(a.gt, a.n_cap, P) + kReserved) *
+                ((kSmallGroupSmWarps + kFew - 1) / kFew) <= kSmBytes)
+        return launch_groups<TX, TY, kFew, P, ACC, MODEL, false>(a, s, false);
     return launch_groups<TX, TY, NW, P, ACC, MODEL, false>(a, s, false);
 }
 

@@ -59,10 +59,11 @@ def test_variants_equal_the_plain_path(R, cg, model):
 # Batches whose tiles and chain groups fit the GPU at once run their sweeps in one
 # launch (the tests above); more than about a thousand blocks take a launch per colour.
 
-def big_run(path, R, cg, model="mpr", n=2):
+def big_run(path, R, cg, model="mpr", n=2, hole=True):
     z = synthetic.grf((530, 545), nu=0.5, ell=9.0, mean=50, std=10, seed=61).astype(np.float32)
     g = synthetic.uniform_gaps((530, 545), 0.35, 62).astype(np.uint8)
-    g[100:150, 200:260] = 1  # tiles that are all gap
+    if hole:
+        g[100:150, 200:260] = 1  # tiles that are all gap
     ctx = mpr.Context([z], [g], chains=R, params=mpr.Params(seed=78, path=path, chain_group=cg, model=model))
     ctx.set_T([0.1])
     ctx.sweep(n, "equil")
@@ -82,6 +83,18 @@ def test_launches_per_colour_equal_the_plain_path(R, cg, model):
     for k in ("a", "accepted"):
         assert np.array_equal(got[1][k], want[1][k])
     assert np.allclose(got[1]["e_last"], want[1]["e_last"], rtol=0, atol=1e-6)
+    assert torch.allclose(got[2], want[2], rtol=1e-6, atol=1e-5)
+
+
+@pytest.mark.parametrize("R,model", [(4, "mpr"), (3, "mpr"), (8, "mpr"), (7, "gmrf"), (16, "mpr"), (13, "gmrf"),
+                                     (32, "mpr"), (2, "mpr"), (20, "mpr"), (33, "gmrf")])
+def test_small_groups_and_padded_rows_equal_the_plain_path(R, model):
+    """Blocks of fewer warps (no tile is dense) and rows of 4, 8, 16 and 32 chains with up
+    to half of them padding."""
+    want, got = (big_run(p, R, 0, model, hole=False) for p in ("plain", "tiled"))
+    assert torch.equal(got[0], want[0])
+    for k in ("a", "accepted"):
+        assert np.array_equal(got[1][k], want[1][k])
     assert torch.allclose(got[2], want[2], rtol=1e-6, atol=1e-5)
 
 
