@@ -69,14 +69,15 @@ struct Geometry {
 // Floats per slot of the state buffer: the tiled layout interleaves the chains, rounded
 // up to 4, 8, 16 or a multiple of 32, so that a chain group's row of a slot starts on
 // its own size and never straddles a 128-byte line (1024^2 at 50 % gaps: 100 chains in
-// rows of 400 bytes 296 us an equilibration sweep, in rows of 512 bytes 245; 96 chains,
-// 384 bytes, 236).  Batches whose states would pass 48 GB that way keep to a multiple
-// of 4 (by the pixels alone: the choice must not depend on the gaps or the tile shape).
+// rows of 400 bytes 296 us an equilibration and 316 a sampling sweep, in rows of 512
+// bytes 276 and 299).  Batches whose states would pass 16 GB that way keep to a multiple
+// of 4, so that the rounding costs 8 GB at most (by the pixels alone: the choice must
+// not depend on the gaps or the tile shape).
 long long state_chains(const Geometry& g) {
     const long long n = g.n_chains;
     if (g.path != MPR_PATH_TILED) return n;
     const long long wide = n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : (n + 31) & ~31LL;
-    return g.n_sites * wide * 4 <= 48LL << 30 ? wide : (n + 3) & ~3LL;
+    return g.n_sites * wide * 4 <= 16LL << 30 ? wide : (n + 3) & ~3LL;
 }
 
 void make_geometry(Geometry& g, int n_img, const int* Lx, const int* Ly, int n_chains, int path,
