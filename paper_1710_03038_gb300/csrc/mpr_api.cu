@@ -238,6 +238,7 @@ struct mpr_ctx {
     // tiled: every tile and chain group fits the GPU at once, so a run of sweeps is one
     // launch (resident sweeps) with this much shared memory per block
     bool resident = false;
+    int steps = 1;  // warp steps of a block in a colour pass, at the tile with the most sites
     size_t res_smem = 0;
     mpr_ctx* sub = nullptr;   // unconditional lattices of the temperature estimate
     // instantiated CUDA graphs of sweep sequences, keyed by (n, phase, flags, stats, accumulate)
@@ -764,8 +765,7 @@ long long resident_need(const mpr_ctx* c) {
 }
 
 // Resident where every (tile, chain group) block fits the GPU at once.  The line lies
-// at the device's own limit: below it the resident run was the faster one at every
-// size measured.
+// at the device's own limit; which of such a batch's runs go there: resident_runs.
 mpr_status choose_resident(mpr_ctx* c, const TileStats& st, cudaStream_t s) {
     const long long need = resident_need(c);
     c->resident = false;
@@ -773,12 +773,32 @@ mpr_status choose_resident(mpr_ctx* c, const TileStats& st, cudaStream_t s) {
     long long blocks = 0;
     MPR_CUDA(resident_blocks(st.res_smem, &blocks));
     c->resident = need <= blocks;
+    ChainRange cr[2];
+    chain_ranges(c, cr);
+    // (four warps, 32 (site, pair) lanes each)
+    c->steps = (std::max(st.n_cap[0], st.n_cap[1]) * tiled_pairs(cr[0].group) + 127) / 128;
     c->res_smem = st.res_smem;
     if (c->resident) {
         MPR_CUDA(resident_prepare(c->p.model == MPR_MODEL_GMRF));
         MPR_CUDA(cudaMemsetAsync(c->ws + c->L.res_words, 0, c->L.res_end - c->L.res_words, s));
     }
     return MPR_OK;
+}
+
+// Whether a run of sweeps goes to the resident kernel.  What it saves is the launches;
+// against it stand that its blocks hold their places on the SMs from the first sweep to
+// the last, which keeps other streams' work out, and that a sweep that adapts a or
+// records energies ends in a wait of every tile for the slowest one.  The more warp
+// steps a block has in a pass, the less the launches matter.  us per sweep, launches ->
+// resident, at up to two steps: 256^2 x 16 chains 15.0 -> 9.0 equilibrating, 12.7 -> 8.2
+// sampling; three: 400^2 x 8 at 60 % gaps 14.1 -> 11.3, 13.0 -> 9.5; four: 600 x 400 x 8
+// does not fit, 462 x 367 x 7 with a block of gaps 12.6 -> 12.8, 12.5 -> 9.2, and two
+// such contexts in turn on two streams took 8.6 a sweep launched, 11.2 resident; six and
+// eight: GMRF 462 x 367 x 10 with recorded energies 21.6 -> 24.9, 20.6 -> 29.0, sampling
+// 16.1 -> 13.6, 16.6 -> 13.7; twelve (x 32) sampling 19.6 -> 20.8.
+bool resident_runs(const mpr_ctx* c, int phase, int flags) {
+    const bool waits = phase == MPR_EQUIL || (flags & MPR_RECORD_ENERGY);
+    return c->resident && c->steps <= (waits ? 3 : 8);
 }
 
 mpr_status sub_workspace_size(const mpr_params& p, const mpr_T_opts& o, int n_img, const int* Lx,
@@ -1223,7 +1243,7 @@ mpr_status run_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool 
                       cudaStream_t s) {
     // (a caller that is capturing gets the launches in its own capture)
     const bool graph = n >= 4 && graphs_usable(c, s);
-    if (c->resident && n > 0) {
+    if (n > 0 && resident_runs(c, phase, flags)) {
         // (a chain's word holds 2^40 accepted proposals: 2^20 sweeps of 2048 tiles)
         constexpr int kMost = 1 << 20;
         for (int k = 0; k < n; k += kMost)

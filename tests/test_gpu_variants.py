@@ -126,6 +126,25 @@ def test_resident_runs_join_without_a_seam(lengths, phase):
     assert out[0][2] == out[1][2]
 
 
+@pytest.mark.parametrize("R,cg,model", [(8, 8, "mpr"), (7, 7, "gmrf"), (16, 16, "mpr"), (20, 16, "gmrf"), (32, 32, "mpr")])
+def test_resident_and_launched_runs_alternate(R, cg, model):
+    """A tile that is all gap: four warp steps and more, so that equilibration and recorded
+    runs are launched per colour and sampling runs are resident (up to eight steps)."""
+    out = []
+    for path in ("plain", "tiled"):
+        zs, gs = images()
+        ctx = mpr.Context(zs, gs, chains=R, params=mpr.Params(seed=79, path=path, chain_group=cg, model=model))
+        ctx.set_T([0.2, 0.05, 0.4])
+        for n, phase, record in ((2, "equil", False), (3, "measure", False), (1, "measure", True),
+                                 (2, "measure", False), (1, "equil", False), (2, "equil", True), (1, "measure", False)):
+            ctx.sweep(n, phase, record_energy=record)
+        out.append(([s.cpu().numpy() for s in ctx.get_state()], ctx.chain_info()))
+    for a, b in zip(out[0][0], out[1][0]):
+        assert np.array_equal(a, b)
+    for k in ("a", "accepted"):
+        assert np.array_equal(out[0][1][k], out[1][1][k])
+
+
 def test_resident_runs_in_a_caller_capture_and_on_two_streams():
     """A captured run replays like a direct one, and contexts on two streams do not
     disturb each other."""
