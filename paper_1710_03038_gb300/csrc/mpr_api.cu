@@ -790,9 +790,9 @@ mpr_status choose_resident(mpr_ctx* c, const TileStats& st, cudaStream_t s) {
 // the last, which keeps other streams' work out, and that a sweep that adapts a or
 // records energies ends in a wait of every tile for the slowest one.  The more warp
 // steps a block has in a pass, the less the launches matter.  us per sweep, launches ->
-// resident, at up to two steps: 256^2 x 16 chains 15.0 -> 9.0 equilibrating, 12.7 -> 8.2
-// sampling; three: 400^2 x 8 at 60 % gaps 14.1 -> 11.3, 13.0 -> 9.5; four: 600 x 400 x 8
-// does not fit, 462 x 367 x 7 with a block of gaps 12.6 -> 12.8, 12.5 -> 9.2, and two
+// resident, at up to two steps: 256^2 x 16 chains 15.9 -> 9.0 equilibrating, 12.7 -> 8.2
+// sampling; three: 400^2 x 8 at 60 % gaps 14.1 -> 11.3, 13.0 -> 9.5; four: 462 x 367 x 7
+// with a block of gaps at 23 % 12.6 -> 12.8 equilibrating, 12.5 -> 9.2 sampling, and two
 // such contexts in turn on two streams took 8.6 a sweep launched, 11.2 resident; six and
 // eight: GMRF 462 x 367 x 10 with recorded energies 21.6 -> 24.9, 20.6 -> 29.0, sampling
 // 16.1 -> 13.6, 16.6 -> 13.7; twelve (x 32) sampling 19.6 -> 20.8.

@@ -11,7 +11,9 @@
 // Equilibration / sampling sweeps, us, launches per colour -> resident: 64^2 x 7
 // chains at 30 % gaps 11.3 / 11.4 -> 4.2 / 4.4; 256^2 x 16 12.4 / 12.8 -> 7.4 / 5.7;
 // 330^2 x 32 at 40 % 18.0 / 19.1 -> 12.4 / 12.2; 500^2 x 32 at 20 % 18.8 / 19.9 ->
-// 17.8 / 15.3 (close to one wave of blocks: the line where it ends).  What is left of a
+// 17.8 / 15.3 (close to one wave of blocks, the most there is room for; which runs of a
+// batch come here is decided by their warp steps, at the last two sizes the sampling
+// runs only: resident_runs).  What is left of a
 // 64^2 pass (2 us) is latency: about 1 us of dependent instructions of one warp step,
 // the rest the trip of the packets through L2.
 //
