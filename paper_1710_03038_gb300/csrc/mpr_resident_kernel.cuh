@@ -509,15 +509,20 @@ __device__ __forceinline__ bool run_tile(const ResidentArgs& ra, unsigned char* 
         }
     }
     if (ACC) {
-        // one add per site and run: the sums of a run are exact in 64 bits
+        // one add per site and run: the sums of a run are exact in 64 bits.  Thread t takes
+        // the red and the black site t, as in the passes, so that it reads what it wrote itself
+        // (a walk over the records in order would cross threads, with no barrier since the last
+        // pass's sums)
         const bool accum2 = (a.flags & kAccumulate2) != 0;
-        const int n = fx->n[0] + fx->n[1];
         const unsigned long long* run = reinterpret_cast<const unsigned long long*>(
-            smem + kFixed + 32 * n + 8 * max(fx->n[0], fx->n[1]));
-        for (int j = tid; j < n; j += kNT) {
-            const long long slot = slot_off + (j < fx->n[0] ? fx->off[0] + j : fx->off[1] + j - fx->n[0]);
-            atomicAdd(a.acc1 + slot, (double)run[2 * j] * 0x1p-24);
-            if (accum2) atomicAdd(a.acc2 + slot, (double)run[2 * j + 1] * 0x1p-21);
+            smem + kFixed + 32 * (fx->n[0] + fx->n[1]) + 8 * max(fx->n[0], fx->n[1]));
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            if (tid >= fx->n[c]) continue;
+            const long long slot = slot_off + fx->off[c] + tid;
+            const unsigned long long* sums = run + 2 * (fx->first[c] + tid);
+            atomicAdd(a.acc1 + slot, (double)sums[0] * 0x1p-24);
+            if (accum2) atomicAdd(a.acc2 + slot, (double)sums[1] * 0x1p-21);
         }
     }
     return true;
