@@ -40,7 +40,7 @@ typedef int mpr_status;
 #define MPR_ERR_T_OUT_OF_RANGE   5  /* e_s outside the range of e(T)              */
 #define MPR_ERR_WORKSPACE        6  /* workspace missing, misaligned or too small */
 #define MPR_ERR_STATE            7  /* call not valid in the context's state      */
-#define MPR_ERR_DEVICE           8  /* a kernel reported an error (status word)   */
+#define MPR_ERR_DEVICE           8  /* a kernel reported an error (mpr_check)      */
 
 /* A CUDA stream (binary compatible with cudaStream_t); NULL = legacy stream. */
 typedef struct CUstream_st* mpr_stream;
@@ -326,6 +326,20 @@ mpr_status mpr_set_chain_a(mpr_ctx* ctx, const float* a, mpr_stream stream);
 mpr_status mpr_get_sweep_index(const mpr_ctx* ctx, uint32_t* sweep, uint32_t* equil_index);
 mpr_status mpr_set_sweep_index(mpr_ctx* ctx, uint32_t sweep, uint32_t equil_index,
                                mpr_stream stream);
+
+/* Whether a kernel of the context gave up: MPR_ERR_DEVICE if a wait of one of its
+ * runs has reached its limit (runs whose blocks wait for one another, see
+ * mpr_sweep_launches), MPR_OK otherwise.  Blocking.  Such a run ends early; its
+ * states, sums and everything after it are void, for the rest of the context's
+ * life.  The calls that return host values report it by themselves
+ * (MPR_ERR_DEVICE); what the others write to device memory is then NaN (mpr_predict,
+ * mpr_get_state and mpr_get_accumulators at the gap pixels, mpr_energy). */
+mpr_status mpr_check(mpr_ctx* ctx, mpr_stream stream);
+
+/* Reads after which a wait of a resident run gives up (2^21, about a second).  0 lets
+ * every such wait give up at once, which shows a caller's handling of MPR_ERR_DEVICE.
+ * Host only; runs already enqueued keep their limit. */
+mpr_status mpr_set_wait_limit(mpr_ctx* ctx, int polls);
 
 /* Releases the host descriptor.  The workspace stays the caller's. */
 void mpr_destroy(mpr_ctx* ctx);

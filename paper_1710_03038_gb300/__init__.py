@@ -335,6 +335,15 @@ class Context:
         a = np.broadcast_to(a, (self.n_img * self.chains,)).copy()
         call("mpr_set_chain_a", self._ctx, a.ctypes.data_as(C.POINTER(C.c_float)), _stream_ptr(stream))
 
+    def check(self, stream=None):
+        """Raise MprError if a kernel of this context has given up waiting (its device outputs
+        are NaN from then on); waits for the stream."""
+        call("mpr_check", self._ctx, _stream_ptr(stream))
+
+    def set_wait_limit(self, polls: int):
+        """Reads after which a wait of a resident run gives up (0: at once)."""
+        call("mpr_set_wait_limit", self._ctx, int(polls))
+
     def sweep_index(self):
         s, e = C.c_uint32(), C.c_uint32()
         call("mpr_get_sweep_index", self._ctx, C.byref(s), C.byref(e))

@@ -2,6 +2,7 @@
 // sweeps, temperature estimate, prediction and state access.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -240,6 +241,7 @@ struct mpr_ctx {
     bool resident = false;
     int steps = 1;  // warp steps of a block in a colour pass, at the tile with the most sites
     size_t res_smem = 0;
+    int polls = kDefaultPolls;  // reads of a wait of a resident run before it gives up
     mpr_ctx* sub = nullptr;   // unconditional lattices of the temperature estimate
     // instantiated CUDA graphs of sweep sequences, keyed by (n, phase, flags, stats, accumulate)
     std::vector<std::pair<long long, cudaGraphExec_t>> graphs;
@@ -406,8 +408,10 @@ __global__ void end_sweep_kernel(const ImgDev* img, ChainDev ch, Control* ctl, i
 // T <- T - (<e> - e_s) T^2 / (N_GP Var(e)), or the geometric bisection of the
 // bracket when the step leaves it.
 __global__ void newton_kernel(ImgDev* sub_img, ImgDev* main_img, ChainDev sub_ch, double* nst,
-                              int n_img, int K, int n_meas) {
+                              int n_img, int K, int n_meas, const Control* sub_ctl, Control* main_ctl) {
     const int im = blockIdx.x * blockDim.x + threadIdx.x;
+    // (a temperature from lattices cut short spoils the realisations too)
+    if (im == 0 && sub_ctl->status != 0) atomicOr(&main_ctl->status, sub_ctl->status);
     if (im >= n_img) return;
     double s = 0.0, s2 = 0.0;
     for (int k = 0; k < K; ++k) {
@@ -482,15 +486,18 @@ __global__ void energy_kernel(const ImgDev* img, const float* state, int n_chain
     if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(out + ic, s);
 }
 
-__global__ void energy_finish_kernel(const ImgDev* img, double* out, int n_chains, int nc) {
+__global__ void energy_finish_kernel(const ImgDev* img, const Control* ctl, double* out, int n_chains, int nc) {
     const int ic = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ic < nc) out[ic] /= img[ic / n_chains].n_bonds;
+    if (ic < nc)
+        out[ic] = ctl->status != 0 ? __longlong_as_double(0x7FF8000000000000LL)
+                                   : out[ic] / img[ic / n_chains].n_bonds;
 }
 
 // state <-> dense [chain][Ly][Lx] per image (dir 0: get, 1: set gap sites).
 __global__ void state_copy_kernel(const ImgDev* img, float* state, const float* samp,
-                                  const int* slot_map, int tiled, int n_chains, float* dense,
-                                  int dir, int ic0, float* plane) {
+                                  const int* slot_map, int tiled, int n_chains, const Control* ctl,
+                                  float* dense, int dir, int ic0, float* plane) {
+    const bool cut_short = dir == 0 && ctl->status != 0;
     const int ic = ic0 + blockIdx.y;
     const int im = ic / n_chains, chain = ic - im * n_chains;
     const ImgDev& I = img[im];
@@ -500,7 +507,8 @@ __global__ void state_copy_kernel(const ImgDev* img, float* state, const float* 
          i += (long long)gridDim.x * blockDim.x) {
         if (tiled) {
             const int s = slot_map[I.site_off + i];
-            if (dir == 0) d[i] = s >= 0 ? state[state_index(I, chain, s)] : samp[I.site_off + i];
+            if (dir == 0) d[i] = s < 0 ? samp[I.site_off + i] : cut_short ? __int_as_float(0x7FC00000)
+                                                              : state[state_index(I, chain, s)];
             else if (s >= 0) state[state_index(I, chain, s)] = d[i];
         } else {
             float* st = state + state_index(I, chain, 0);
@@ -537,7 +545,8 @@ __global__ void predict_kernel(const ImgDev* img, const double* acc1, const doub
 
 // Realisation sums <-> dense per-pixel arrays (dir 0: get, 1: set gap pixels).
 __global__ void acc_dense_kernel(const ImgDev* img, double* acc, const int* slot_map,
-                                 const float* samp, int tiled, double* dense, int dir) {
+                                 const float* samp, int tiled, const Control* ctl, double* dense, int dir) {
+    const bool cut_short = dir == 0 && ctl->status != 0;
     const ImgDev& I = img[blockIdx.y];
     const long long n = (long long)I.Lx * I.Ly;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -546,7 +555,8 @@ __global__ void acc_dense_kernel(const ImgDev* img, double* acc, const int* slot
         long long slot = -1;
         if (tiled) slot = slot_map[s];
         else if (samp[s] < 0.0f) slot = i;
-        if (dir == 0) dense[s] = slot < 0 ? 0.0 : acc[I.slot_off + slot];
+        if (dir == 0) dense[s] = slot < 0 ? 0.0 : cut_short ? __longlong_as_double(0x7FF8000000000000LL)
+                                                 : acc[I.slot_off + slot];
         else if (slot >= 0) acc[I.slot_off + slot] = dense[s];
     }
 }
@@ -1107,6 +1117,7 @@ mpr_status launch_resident_run(mpr_ctx* c, int n, int phase, int flags, bool sta
     r.epoch = at<uint32_t>(c->ws, c->L.res_epoch);
     r.packets = at<ulonglong2>(c->ws, c->L.res_packets);
     r.energies = at<ulonglong2>(c->ws, c->L.res_e);
+    r.polls = c->polls;
     const cudaError_t e = launch_resident(r, r.n_whole + (n_cr - 1), c->res_smem, s);
     if (e != cudaSuccess) return fail(MPR_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(e));
     return MPR_OK;
@@ -1488,7 +1499,7 @@ mpr_status mpr_estimate_T(mpr_ctx* c, double* T_out, mpr_stream stream) {
         MPR_TRY(run_sweeps(u, neq, MPR_EQUIL, 0, false, false, s));
         MPR_TRY(run_sweeps(u, c->topt.n_meas, MPR_MEASURE, MPR_RECORD_ENERGY, true, false, s));
         newton_kernel<<<grid_for(n_img), 256, 0, s>>>(u->d_img, c->d_img, u->ch, c->d_newton, n_img,
-                                                     K, c->topt.n_meas);
+                                                     K, c->topt.n_meas, u->d_ctl, c->d_ctl);
         MPR_CUDA(cudaGetLastError());
     }
     c->T_set = true;
@@ -1739,7 +1750,7 @@ mpr_status mpr_get_energy_history(mpr_ctx* c, double* out, mpr_stream stream) {
     MPR_CUDA(cudaMemcpyAsync(out, c->d_hist, sizeof(double) * kHist * c->g.n_img,
                              cudaMemcpyDeviceToHost, s));
     MPR_CUDA(cudaStreamSynchronize(s));
-    return MPR_OK;
+    return check_device_status(c, s);
 }
 
 mpr_status mpr_energy(mpr_ctx* c, double* e_out, mpr_mem where, mpr_stream stream) {
@@ -1761,11 +1772,12 @@ mpr_status mpr_energy(mpr_ctx* c, double* e_out, mpr_mem where, mpr_stream strea
             c->d_img, c->d_state, c->g.n_chains, (float)c->p.q, (float)c->p.J, gmrf, d_out);
         MPR_CUDA(cudaGetLastError());
     }
-    energy_finish_kernel<<<grid_for(nc), 256, 0, s>>>(c->d_img, d_out, c->g.n_chains, nc);
+    energy_finish_kernel<<<grid_for(nc), 256, 0, s>>>(c->d_img, c->d_ctl, d_out, c->g.n_chains, nc);
     MPR_CUDA(cudaGetLastError());
     if (where == MPR_HOST) {
         MPR_CUDA(cudaMemcpyAsync(e_out, d_out, sizeof(double) * nc, cudaMemcpyDeviceToHost, s));
         MPR_CUDA(cudaStreamSynchronize(s));
+        if (std::isnan(e_out[0])) return check_device_status(c, s);  // (NaN where the status is set)
     }
     return MPR_OK;
 }
@@ -1782,7 +1794,7 @@ mpr_status mpr_predict(mpr_ctx* c, float* z_hat, float* z_std, mpr_mem where, mp
     const double n_samples = (double)c->n_meas_done * c->g.n_chains;
     if (c->g.path == MPR_PATH_TILED) {
         MPR_CUDA(launch_predict_tiles(c->d_img, c->d_tiles, c->g.n_tiles, c->g.tx, c->g.ty, c->d_slot_pos,
-                                      c->d_acc1, c->d_acc2, c->d_zst, c->d_gst, n_samples, dh, ds, s));
+                                      c->d_acc1, c->d_acc2, c->d_zst, c->d_gst, n_samples, c->d_ctl, dh, ds, s));
     } else {
         predict_kernel<<<dim3(grid_for(maxn, 256, 2048), c->g.n_img), 256, 0, s>>>(
             c->d_img, c->d_acc1, c->d_acc2, c->d_zst, c->d_samp, n_samples, dh, ds);
@@ -1817,7 +1829,7 @@ static mpr_status acc_copy(mpr_ctx* c, double* acc, double* dense, mpr_mem where
     long long maxn = 0;
     for (int i = 0; i < c->g.n_img; ++i) maxn = std::max(maxn, (long long)c->g.Lx[i] * c->g.Ly[i]);
     acc_dense_kernel<<<dim3(grid_for(maxn, 256, 1024), c->g.n_img), 256, 0, s>>>(
-        c->d_img, acc, c->d_slot_map, c->d_samp, c->g.path == MPR_PATH_TILED ? 1 : 0, d, dir);
+        c->d_img, acc, c->d_slot_map, c->d_samp, c->g.path == MPR_PATH_TILED ? 1 : 0, c->d_ctl, d, dir);
     MPR_CUDA(cudaGetLastError());
     if (where == MPR_HOST) {
         if (dir == 0) MPR_CUDA(cudaMemcpyAsync(dense, d, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
@@ -1834,7 +1846,7 @@ mpr_status mpr_get_accumulators(mpr_ctx* c, double* sum, double* sum2, int64_t* 
     if (sum) MPR_TRY(acc_copy(c, c->d_acc1, sum, where, 0, s));
     if (sum2) MPR_TRY(acc_copy(c, c->d_acc2, sum2, where, 0, s));
     if (n_terms) *n_terms = (int64_t)c->n_meas_done * c->g.n_chains;
-    return MPR_OK;
+    return where == MPR_HOST && (sum || sum2) ? check_device_status(c, s) : MPR_OK;
 }
 
 mpr_status mpr_set_accumulators(mpr_ctx* c, const double* sum, const double* sum2,
@@ -1863,11 +1875,11 @@ static mpr_status state_copy(mpr_ctx* c, float* phi, mpr_mem where, int dir, cud
         if (tiled && maxn * nc >= (1LL << 18)) {
             MPR_CUDA(launch_state_tiles(c->d_img, c->d_tiles, c->g.n_tiles, c->g.tx, c->g.ty,
                                         std::min(c->g.tx * c->g.ty, c->n_cap[0] + c->n_cap[1]), c->d_slot_pos,
-                                        c->d_samp, c->d_state, c->g.n_chains, phi, dir == 1, s));
+                                        c->d_samp, c->d_state, c->g.n_chains, c->d_ctl, phi, dir == 1, s));
             return MPR_OK;
         }
         state_copy_kernel<<<dim3(grid_for(maxn, 256, 1024), nc), 256, 0, s>>>(
-            c->d_img, c->d_state, c->d_samp, c->d_slot_map, tiled, c->g.n_chains, phi, dir, 0,
+            c->d_img, c->d_state, c->d_samp, c->d_slot_map, tiled, c->g.n_chains, c->d_ctl, phi, dir, 0,
             nullptr);
         MPR_CUDA(cudaGetLastError());
         return MPR_OK;
@@ -1880,7 +1892,7 @@ static mpr_status state_copy(mpr_ctx* c, float* phi, mpr_mem where, int dir, cud
         float* h = phi + c->g.site_off[im] * c->g.n_chains + (long long)chain * n;
         if (dir == 1) MPR_CUDA(cudaMemcpyAsync(stage, h, sizeof(float) * n, cudaMemcpyHostToDevice, s));
         state_copy_kernel<<<dim3(grid_for(n, 256, 1024), 1), 256, 0, s>>>(
-            c->d_img, c->d_state, c->d_samp, c->d_slot_map, tiled, c->g.n_chains, nullptr, dir, ic,
+            c->d_img, c->d_state, c->d_samp, c->d_slot_map, tiled, c->g.n_chains, c->d_ctl, nullptr, dir, ic,
             stage);
         MPR_CUDA(cudaGetLastError());
         if (dir == 0) MPR_CUDA(cudaMemcpyAsync(h, stage, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
@@ -1891,7 +1903,9 @@ static mpr_status state_copy(mpr_ctx* c, float* phi, mpr_mem where, int dir, cud
 
 mpr_status mpr_get_state(mpr_ctx* c, float* phi, mpr_mem where, mpr_stream stream) {
     if (!c || !phi) return fail(MPR_ERR_INVALID_ARG, "NULL argument");
-    return state_copy(c, phi, where, 0, reinterpret_cast<cudaStream_t>(stream));
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    MPR_TRY(state_copy(c, phi, where, 0, s));
+    return where == MPR_HOST ? check_device_status(c, s) : MPR_OK;
 }
 
 mpr_status mpr_set_state(mpr_ctx* c, const float* phi, mpr_mem where, mpr_stream stream) {
@@ -1933,12 +1947,26 @@ mpr_status mpr_get_sweep_index(const mpr_ctx* c, uint32_t* sweep, uint32_t* equi
 
 mpr_status mpr_set_sweep_index(mpr_ctx* c, uint32_t sweep, uint32_t equil_index, mpr_stream stream) {
     if (!c) return fail(MPR_ERR_INVALID_ARG, "ctx is NULL");
-    Control h{sweep, equil_index, 0u, 0u};
+    // (the first two words: an error bit stays)
+    static_assert(offsetof(Control, sweep) == 0 && offsetof(Control, equil_index) == 4, "counters first");
+    const uint32_t h[2] = {sweep, equil_index};
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    MPR_CUDA(cudaMemcpyAsync(c->d_ctl, &h, sizeof(Control), cudaMemcpyHostToDevice, s));
+    MPR_CUDA(cudaMemcpyAsync(c->d_ctl, h, sizeof(h), cudaMemcpyHostToDevice, s));
     MPR_CUDA(cudaStreamSynchronize(s));
     c->sweep = sweep;
     c->equil_index = equil_index;
+    return MPR_OK;
+}
+
+mpr_status mpr_check(mpr_ctx* c, mpr_stream stream) {
+    if (!c) return fail(MPR_ERR_INVALID_ARG, "ctx is NULL");
+    return check_device_status(c, reinterpret_cast<cudaStream_t>(stream));
+}
+
+mpr_status mpr_set_wait_limit(mpr_ctx* c, int polls) {
+    if (!c || polls < 0) return fail(MPR_ERR_INVALID_ARG, "need a context and polls >= 0");
+    c->polls = polls;
+    if (c->sub) c->sub->polls = polls;
     return MPR_OK;
 }
 

@@ -21,8 +21,8 @@ __global__ void __launch_bounds__(128)
 predict_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix,
                     const uint32_t* __restrict__ slot_pos, const double* __restrict__ acc1,
                     const double* __restrict__ acc2, const float* __restrict__ zin,
-                    const uint8_t* __restrict__ gap, double inv_n, float* __restrict__ zhat,
-                    float* __restrict__ zstd) {
+                    const uint8_t* __restrict__ gap, double inv_n, const Control* ctl,
+                    float* __restrict__ zhat, float* __restrict__ zstd) {
     const TileDesc T = tiles[blockIdx.x];
     const ImgDev& I = img[T.img];
     const int Lx = I.Lx, Ly = I.Ly;
@@ -36,6 +36,8 @@ predict_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int np
         if (zstd) zstd[s] = 0.0f;
     }
     constexpr double kInvTwoPiD = 0.15915494309189533577;
+    const bool cut_short = ctl->status != 0;
+    if (cut_short) inv_n = __longlong_as_double(0x7FF8000000000000LL);
     const double per_rad = ((double)I.zmax - (double)I.zmin) * kInvTwoPiD;  // field units per rad
     const double scale = per_rad * inv_n, zmin = I.zmin;
     for (int j = threadIdx.x; j < T.cnt[0] + T.cnt[1]; j += 128) {
@@ -48,7 +50,7 @@ predict_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int np
             const double m = a * inv_n;
             const double v = fma(-m, m, acc2[k] * inv_n);
             const float vf = (float)v;
-            float sd = 0.0f;
+            float sd = cut_short ? __int_as_float(0x7FC00000) : 0.0f;
             if (vf > 1e30f) {  // (beyond the estimate's range: angles are below 2 pi)
                 sd = (float)(sqrt(v) * per_rad);
             } else if (vf > 1e-30f) {
@@ -68,7 +70,7 @@ template <bool SET>
 __global__ void __launch_bounds__(256)
 state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix,
                   int n_max, const uint32_t* __restrict__ slot_pos, const float* __restrict__ samp,
-                  float* __restrict__ state, int n_chains, float* __restrict__ dense) {
+                  float* __restrict__ state, int n_chains, const Control* ctl, float* __restrict__ dense) {
     extern __shared__ float rows[];  // [sites of the tile, at most n_max][33], then the tile's map
     uint16_t* map = reinterpret_cast<uint16_t*>(rows + n_max * 33);  // pixel -> site, 0xFFFF: a sample
     const TileDesc T = tiles[blockIdx.x];
@@ -85,8 +87,10 @@ state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix
     }
     float* st = state + T.state_off + r0 + lane;
     if (!SET && lane < nr) {
+        const bool cut_short = ctl->status != 0;
 #pragma unroll 8
-        for (int j = warp; j < n; j += 8) rows[j * 33 + lane] = st[(long long)slot_of(j) * T.cp];
+        for (int j = warp; j < n; j += 8)
+            rows[j * 33 + lane] = cut_short ? __int_as_float(0x7FC00000) : st[(long long)slot_of(j) * T.cp];
     }
     __syncthreads();
     const long long plane = (long long)Lx * Ly;
@@ -228,16 +232,16 @@ int log2_of(int v) {
 
 cudaError_t launch_predict_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tx, int ty,
                                  const uint32_t* slot_pos, const double* acc1, const double* acc2,
-                                 const float* z, const uint8_t* gap, double n_samples, float* zhat,
-                                 float* zstd, cudaStream_t s) {
+                                 const float* z, const uint8_t* gap, double n_samples,
+                                 const Control* ctl, float* zhat, float* zstd, cudaStream_t s) {
     predict_tile_kernel<<<n_tiles, 128, 0, s>>>(img, tiles, log2_of(tx), tx * ty, slot_pos, acc1, acc2, z,
-                                                gap, 1.0 / n_samples, zhat, zstd);
+                                                gap, 1.0 / n_samples, ctl, zhat, zstd);
     return cudaGetLastError();
 }
 
 cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tx, int ty,
                                int n_max, const uint32_t* slot_pos, const float* samp, float* state,
-                               int n_chains, float* dense, bool set, cudaStream_t s) {
+                               int n_chains, const Control* ctl, float* dense, bool set, cudaStream_t s) {
     n_max = (n_max + 3) & ~3;  // (the map after the rows starts on 16 bytes)
     const size_t smem = (size_t)n_max * 33 * sizeof(float) + (size_t)tx * ty * sizeof(uint16_t);
     const auto kernel = set ? state_tile_kernel<true> : state_tile_kernel<false>;
@@ -247,7 +251,7 @@ cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_t
         if (e != cudaSuccess) return e;
     }
     kernel<<<dim3(n_tiles, (n_chains + 31) / 32), 256, smem, s>>>(img, tiles, log2_of(tx), tx * ty, n_max,
-                                                                  slot_pos, samp, state, n_chains, dense);
+                                                                  slot_pos, samp, state, n_chains, ctl, dense);
     return cudaGetLastError();
 }
 

@@ -49,7 +49,8 @@ struct ImgDev {
 struct Control {
     uint32_t sweep;        // Philox sweep field of the next sweep
     uint32_t equil_index;  // i of Alg. 2 step 4.2 for the next equilibration sweep
-    uint32_t status;       // device-side error bits
+    uint32_t status;       // device-side error bits; while any is set, what is read out of the
+                           // context's state is NaN
     uint32_t ticket;       // blocks of the end-of-sweep kernel done (0 between launches)
 };
 
@@ -188,10 +189,12 @@ int tiled_blocks_per_sm(int tx, int ty);
 cudaError_t launch_predict_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tile_x,
                                  int tile_y, const uint32_t* slot_pos, const double* acc1,
                                  const double* acc2, const float* z, const uint8_t* gap,
-                                 double n_samples, float* zhat, float* zstd, cudaStream_t s);
+                                 double n_samples, const Control* ctl, float* zhat, float* zstd,
+                                 cudaStream_t s);
 cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tile_x,
                                int tile_y, int n_max, const uint32_t* slot_pos, const float* samp,
-                               float* state, int n_chains, float* dense, bool set, cudaStream_t s);
+                               float* state, int n_chains, const Control* ctl, float* dense, bool set,
+                               cudaStream_t s);
 cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles,
                                 int tile_x, int tile_y, const float* state, const float* samp,
                                 const int* slot_map, int n_chains, float q, float J, int gmrf,

@@ -179,6 +179,7 @@ mpr_status mpr_select_q(int Lx, int Ly, const float* z, const uint8_t* gap, cons
                 cudaStreamSynchronize(s) != cudaSuccess)
                 st = set_last_error(MPR_ERR_CUDA, "mpr_select_q: validation error");
         }
+        if (st == MPR_OK) st = mpr_check(ctx, stream);
         mpr_destroy(ctx);
         if (st != MPR_OK) return st;
         scores[k] = acc[0] / n_hold;

@@ -22,7 +22,11 @@ struct ResidentArgs {
     ulonglong2* packets;   // [3][tile][64 places][chain pairs]: (angle, epoch) words of both chains
     ulonglong2* energies;  // [3][tile][chain]: (half of a double, epoch) words
     uint32_t* epoch;       // epoch of the last launch's last pass
+    int polls;             // reads of a wait before it gives up
 };
+
+// (about a second)
+constexpr int kDefaultPolls = 1 << 21;
 
 // Shared memory of a block: the fixed part, the own sites' records and sums, the two
 // tables and the sites' packet places, for a tile of n0 red and n1 black sites with h0

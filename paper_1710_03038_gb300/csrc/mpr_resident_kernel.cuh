@@ -38,8 +38,9 @@
 // the launch per colour, so both give the same bits.
 //
 // Waiting.  The launch is cooperative (every block is resident), a block waits only
-// for blocks of its own launch, every wait has an iteration limit, and one that
-// gives up sets the status word and ends its block.
+// for blocks of its own launch, every wait has an iteration limit (ResidentArgs::polls),
+// and one that gives up sets the status word and ends its block.  The states and sums are
+// then those of a run cut short: whatever reads them out gives NaN (mpr_check).
 #pragma once
 
 #include "mpr_device.cuh"
@@ -53,7 +54,6 @@ using namespace tiled;
 
 constexpr int kNW = 4, kNT = kNW * 32;  // warps and threads of a block, as the 16 x 16 pass
 constexpr int kRing = 32;               // ring cells of one colour (16 + 16)
-constexpr int kPolls = 1 << 21;         // about a second
 constexpr unsigned kNoEdge = 0xFFu;
 constexpr int kRecorderChains = 4;
 // 72 registers a thread: at 64 the variants that record energies spill
@@ -105,16 +105,16 @@ __device__ __forceinline__ bool try_receive(const ulonglong2* pk, uint32_t epoch
 }
 
 // The packet's angles once both words carry the epoch; false when it never comes.
-__device__ __forceinline__ bool receive(const ulonglong2* pk, uint32_t epoch, float2& v) {
-    for (int k = 0; k < kPolls; ++k)
+__device__ __forceinline__ bool receive(const ulonglong2* pk, uint32_t epoch, float2& v, int polls) {
+    for (int k = 0; k < polls; ++k)
         if (try_receive(pk, epoch, v)) return true;
     return false;
 }
 
 // A chain's word once `tiles` arrivals (modulo 2^24) are in.
 __device__ __forceinline__ bool arrived(const unsigned long long* word, uint32_t tiles,
-                                        unsigned long long& v) {
-    for (int k = 0; k < kPolls; ++k) {
+                                        unsigned long long& v, int polls) {
+    for (int k = 0; k < polls; ++k) {
         asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
         // at most one sweep's arrivals beyond the awaited ones are in
         if ((((uint32_t)(v >> 40) - tiles) & 0xFFFFFFu) < 0x800000u) return true;
@@ -163,7 +163,7 @@ __device__ __forceinline__ bool run_recorder(const ResidentArgs& ra, unsigned ch
             for (int i = 0; i < 8; ++i) {
                 if (wait >> i & 1u)
                     there = there && receive(pk + (k % 3) * pk_buf + (long long)(t0 + i * t_step) * a.n_chains,
-                                             epoch, v[i]);
+                                             epoch, v[i], ra.polls);
                 E += __hiloint2double(__float_as_int(v[i].y), __float_as_int(v[i].x));
             }
         }
@@ -305,7 +305,7 @@ __device__ __forceinline__ bool run_tile(const ResidentArgs& ra, unsigned char* 
     const auto finished = [&](int k, int ch, int sp, unsigned long long& v) {
         return arrived(ra.words + (((k & 1) << ra.spread_log) + sp) * fx->word_step +
                            (long long)T.img * a.n_chains + r0 + ch,
-                       (uint32_t)((k >> 1) + 1) * arrivals_at(ra, tiles_img, sp, ENERGY), v);
+                       (uint32_t)((k >> 1) + 1) * arrivals_at(ra, tiles_img, sp, ENERGY), v, ra.polls);
     };
     // adds up the accepted proposals of every chain up to sweep k
     const auto count = [&](int k) {
@@ -350,7 +350,7 @@ __device__ __forceinline__ bool run_tile(const ResidentArgs& ra, unsigned char* 
                     float2 v;
                     if (c == 0 && k == 0) {
                         v = *reinterpret_cast<const float2*>(st + (long long)fx->slot[e] * cp);
-                    } else if (!receive(from + (long long)fx->ring[c][e] * np, epoch, v)) {
+                    } else if (!receive(from + (long long)fx->ring[c][e] * np, epoch, v, ra.polls)) {
                         there = false;
                         break;
                     }

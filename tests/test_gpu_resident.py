@@ -46,3 +46,56 @@ def test_sums_of_sampling_runs(R, cg, frac, model):
         assert torch.equal(got[0][0], want[0][0])
         assert torch.equal(got[1][0], want[1][0])
     assert torch.equal(alone.get_state()[0], launched.get_state()[0])
+
+
+# ------------------------------------------------------------------ a wait that gives up
+
+def device_error(call):
+    with pytest.raises(mpr._lib.MprError) as e:
+        call()
+    assert e.value.status == 8
+
+
+# (states of 1.5e5 values go out by pixel, of 3e5 by tile)
+@pytest.mark.parametrize("R,phase", [(8, "equil"), (8, "measure"), (16, "measure")])
+def test_a_run_that_gives_up_is_reported(R, phase):
+    """A wait limit of 0: every wait gives up.  Calls that return host values fail; what goes
+    to device memory is NaN at the gaps; the context stays unusable, others are not touched."""
+    z, g = image((130, 147), 0.3, 31)
+    gap, smp = torch.from_numpy(g).cuda() != 0, torch.from_numpy(z).cuda()
+    ctx = context([(z, g)], R, 8)
+    ctx.sweep(2, "measure")
+    ctx.check()
+    ctx.set_wait_limit(0)
+    ctx.sweep(3, phase)
+    zh, sd = ctx.predict(std=True)
+    s1, s2, _ = ctx.accumulators()
+    for t in (zh[0], sd[0], s1[0], s2[0], *ctx.get_state()[0]):
+        assert bool(torch.isnan(t[gap]).all()) and not bool(torch.isnan(t[~gap]).any())
+    assert torch.equal(zh[0][~gap], smp[~gap])
+    device_error(ctx.check)
+    device_error(ctx.energy)
+    device_error(ctx.chain_info)
+    device_error(ctx.get_T)
+    device_error(ctx.energy_history)
+    device_error(lambda: ctx.predict_host(torch.empty(z.size)))
+    ctx.set_wait_limit(1 << 21)
+    ctx.set_sweep_index(0, 0)  # (does not hide it)
+    device_error(ctx.check)
+    again = context([(z, g)], R, 8)
+    again.sweep(3, phase)
+    again.check()
+
+
+def test_a_temperature_that_gives_up_is_reported():
+    z, g = image((130, 147), 0.3, 31)
+    ctx = mpr.Context([z], [g], chains=4)
+    ctx.set_wait_limit(0)
+    device_error(ctx.estimate_T)
+    ctx = mpr.Context([z], [g], chains=4)
+    ctx.set_wait_limit(0)
+    ctx.estimate_T_async()
+    ctx.set_wait_limit(1 << 21)
+    ctx.sweep(2, "measure")
+    assert bool(torch.isnan(ctx.predict()[0][torch.from_numpy(g).cuda() != 0]).all())
+    device_error(ctx.check)
