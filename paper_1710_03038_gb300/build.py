@@ -20,7 +20,7 @@ SOURCES = ["mpr_api.cu", "mpr_setup.cu", "mpr_dense.cu", "mpr_tiled.cu", "mpr_ti
            "mpr_tiled_32x32.cu", "mpr_resident.cu", "mpr_resident_mpr.cu", "mpr_resident_gmrf.cu",
            "mpr_plain.cu", "mpr_lattice.cu", "mpr_noalloc.cu",
            "mpr_qcv.cu"]
-HEADERS = ["mpr_device.cuh", "mpr_internal.h", "mpr_resident.h", "mpr_async.cuh",
+HEADERS = ["mpr_device.cuh", "mpr_internal.h", "mpr_once.h", "mpr_resident.h", "mpr_async.cuh",
            "mpr_tiled_kernel.cuh", "mpr_resident_kernel.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-ftz=true", "-Xcompiler", "-fPIC",

@@ -35,16 +35,18 @@ cudaError_t resident_blocks(size_t smem, long long* blocks) {
 }
 
 cudaError_t resident_prepare(bool gmrf) {
-    static bool done[2] = {false, false};
-    if (done[gmrf]) return cudaSuccess;
-    int dev = 0, most = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    for (int v = 0; v < 4 && e == cudaSuccess; ++v)
-        e = cudaFuncSetAttribute(reinterpret_cast<const void*>(resident::pick(v & 1, v & 2, gmrf)),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    done[gmrf] = e == cudaSuccess;
-    return e;
+    static OncePerDevice limit[2];
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return limit[gmrf](dev, [&] {
+        int most = 0;
+        cudaError_t s = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        for (int v = 0; v < 4 && s == cudaSuccess; ++v)
+            s = cudaFuncSetAttribute(reinterpret_cast<const void*>(resident::pick(v & 1, v & 2, gmrf)),
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        return s;
+    });
 }
 
 cudaError_t launch_resident(const ResidentArgs& ra, int n_groups, size_t smem, cudaStream_t s) {

@@ -56,6 +56,7 @@
 #include "mpr_async.cuh"
 #include "mpr_device.cuh"
 #include "mpr_internal.h"
+#include "mpr_once.h"
 
 namespace mpr {
 namespace tiled {
@@ -480,13 +481,15 @@ cudaError_t launch_one(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     using Cf = Cfg<TX, TY, NW, MODEL>;
     static_assert(Cf::smem_max <= 227 * 1024, "shared memory");
     const auto kernel = tiled_pass_kernel<TX, TY, NW, P, ACC, MODEL, ENERGY, GROUPS>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)Cf::smem_max);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static OncePerDevice limit;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = limit(dev, [&] {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)Cf::smem_max);
+        });
+    if (e != cudaSuccess) return e;
     if (setup_only) return cudaSuccess;
     if (a.gt < 1 || a.gt > Cf::GT || a.n_cap < 0 || a.n_cap > Cf::NMAX) return cudaErrorInvalidValue;
     dim3 grid(a.n_list, (a.chain_end - a.chain0 + a.chain_group - 1) / a.chain_group);
