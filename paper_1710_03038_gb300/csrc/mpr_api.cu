@@ -43,7 +43,6 @@ constexpr size_t kAlign = 256;
 constexpr int kHist = 512;  // chain-mean energies kept per image for the equilibration test
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 constexpr double kPiD = 3.14159265358979323846;
-constexpr int kResidentBlocks = 2048;  // upper bound on the blocks that run at once (8 per SM)
 
 // ============================================================ layout
 
@@ -59,6 +58,7 @@ struct Layout {
 
 struct Geometry {
     int n_img = 0, n_chains = 0, path = 0, tx = 64, ty = 64, halo_cap = 128;
+    bool res_room = false;  // the batch may be resident: its workspace holds what that needs
     std::vector<int> Lx, Ly;
     std::vector<long long> site_off;
     std::vector<int> tile0, ntiles;
@@ -107,6 +107,15 @@ void make_geometry(Geometry& g, int n_img, const int* Lx, const int* Ly, int n_c
         g.max_Lx = std::max(g.max_Lx, Lx[i]);
         g.max_Ly = std::max(g.max_Ly, Ly[i]);
     }
+}
+
+// Batches that no choice of the chain groups can make resident get no room for it: other
+// tile shapes and the printed over-relaxation have no resident kernel, and groups are at
+// most 32 chains, recorders at most 4 (so resident_need is never below this sum).
+bool resident_room(const Geometry& g, int literal_or) {
+    const long long n = g.n_chains;
+    return g.path == MPR_PATH_TILED && g.tx == 16 && g.ty == 16 && !literal_or &&
+           g.n_tiles * ((n + 31) / 32) + g.n_img * ((n + 3) / 4) <= kResidentBlocks;
 }
 
 // Resident sweeps: 2^this words per chain, one per 64 tiles of the largest image.
@@ -162,10 +171,8 @@ Layout make_layout(const Geometry& g, const std::vector<long long>& slots_per_im
     L.state = take(sizeof(float) * L.n_state);
     L.newton = take(sizeof(double) * 4 * g.n_img);
     L.hist = take(sizeof(double) * kHist * g.n_img + sizeof(int) * (g.n_img + 3));
-    // resident sweeps: per-chain words, epoch, boundary and energy packets (none when the
-    // batch has more blocks than one wave)
-    const size_t RT = tiled && g.n_tiles * (long long)((g.n_chains + 31) / 32) <= kResidentBlocks
-                          ? (size_t)g.n_tiles : 0;
+    // resident sweeps: per-chain words, epoch, boundary and energy packets
+    const size_t RT = g.res_room ? (size_t)g.n_tiles : 0;
     L.res_words = take(RT ? 2 * (sizeof(unsigned long long) * NC << resident_spread_log(g)) : 0);
     L.res_epoch = take(RT ? sizeof(uint32_t) : 0);
     L.res_packets = take(3 * 64 * sizeof(ulonglong2) * RT * ((g.n_chains + 1) / 2));
@@ -766,7 +773,7 @@ mpr_status split_tiles(mpr_ctx* c, const TileStats& st, cudaStream_t s) {
 // the GMRF.
 long long resident_need(const mpr_ctx* c) {
     const Geometry& g = c->g;
-    if (g.path != MPR_PATH_TILED || g.tx != 16 || g.ty != 16 || (model_flags(c->p) & kLiteralOR)) return 0;
+    if (!g.res_room) return 0;
     ChainRange cr[2];
     const int n_cr = chain_ranges(c, cr);
     const long long groups = (cr[0].chain_end + cr[0].group - 1) / cr[0].group + (n_cr - 1);
@@ -823,6 +830,7 @@ mpr_status workspace_size_impl(int n_img, const int* Lx, const int* Ly, const in
         return fail(MPR_ERR_INVALID_ARG, "unsupported tile shape");
     Geometry g;
     make_geometry(g, n_img, Lx, Ly, n_chains, p.path, tx, ty);
+    g.res_room = resident_room(g, p.literal_or);
     std::vector<long long> slots(n_img);
     for (int i = 0; i < n_img; ++i)
         slots[i] = slot_bound(g, i, n_gap ? (long long)n_gap[i] : (long long)Lx[i] * Ly[i]);
@@ -886,6 +894,7 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
     c->img_tag = unconditional ? (1u << 30) : 0u;
     make_geometry(c->g, n_img, Lx, Ly, n_chains, c->p.path, tx, ty);
     Geometry& g = c->g;
+    g.res_room = resident_room(g, c->p.literal_or);
     const bool tiled = g.path == MPR_PATH_TILED;
     const bool staging = !unconditional;
     size_t sub_bytes = 0;

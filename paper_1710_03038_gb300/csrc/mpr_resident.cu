@@ -7,6 +7,8 @@
 namespace mpr {
 namespace resident {
 
+static_assert(kBlocksPerSM * 152 == kResidentBlocks, "room for as many blocks as fit");
+
 Kernel pick(bool acc, bool energy, bool gmrf) {
     return gmrf ? pick_gmrf(acc, energy) : pick_mpr(acc, energy);
 }

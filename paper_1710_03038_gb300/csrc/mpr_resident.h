@@ -25,6 +25,8 @@ struct ResidentArgs {
     int polls;             // reads of a wait before it gives up
 };
 
+// The most blocks that the device holds at once: 152 SMs of seven.
+constexpr int kResidentBlocks = 152 * 7;
 // (about a second)
 constexpr int kDefaultPolls = 1 << 21;
 

@@ -104,3 +104,40 @@ def test_no_cpu_fallback_in_product_package():
                     text = f.read()
                 assert "import oracle" not in text and "from oracle" not in text, fn
                 assert "mpr_oracle" not in text, fn
+
+
+def _workspace(lib, side, chains, images=1, **fields):
+    import ctypes as C
+    from paper_1710_03038_gb300 import _lib
+    p = _lib.MprParams()
+    lib.mpr_default_params(C.byref(p))
+    for k, v in fields.items():
+        setattr(p, k, v)
+    L, n = _lib.int_array([side] * images), C.c_size_t()
+    assert lib.mpr_workspace_size(images, L, L, None, chains, C.byref(p), None, C.byref(n)) == 0
+    return n.value
+
+
+@pytest.mark.parametrize("chains", [1, 4, 10, 32, 100])
+@pytest.mark.parametrize("side", [64, 200, 333, 512, 700, 1024, 1400])
+def test_the_smallest_tiles_need_the_largest_workspace(lib, side, chains):
+    """What mpr_autotune asks its callers to rely on: a workspace for 16 x 16 tiles holds
+    every candidate."""
+    for images in (1, 3):
+        want = _workspace(lib, side, chains, images, tile_x=16, tile_y=16)
+        assert _workspace(lib, side, chains, images, tile_x=32, tile_y=16) <= want
+        assert _workspace(lib, side, chains, images, tile_x=32, tile_y=32) <= want
+
+
+@pytest.mark.parametrize("side,chains", [(700, 32), (520, 64), (530, 4)])
+def test_batches_that_cannot_be_resident_reserve_no_packets(lib, side, chains):
+    """More than 1064 blocks (152 SMs of seven), or the printed over-relaxation: 16 x 16 tiles
+    need what their slots and lists add to those of 32 x 32 tiles, and no packets."""
+    tiles = (-(-side // 16)) ** 2
+    for fields in (dict(), dict(literal_or=1)):
+        extra = (_workspace(lib, side, chains, tile_x=16, tile_y=16, **fields)
+                 - _workspace(lib, side, chains, tile_x=32, tile_y=32))
+        # 8 slots of padding, their records, the ring lists and the tile's own records
+        assert extra < tiles * (8 * (4 * ((chains + 31) // 32 * 32) + 64) + 1024)
+    assert (_workspace(lib, 128, 32, tile_x=16, tile_y=16, literal_or=1)
+            < _workspace(lib, 128, 32, tile_x=16, tile_y=16))
