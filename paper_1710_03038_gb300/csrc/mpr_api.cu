@@ -1103,8 +1103,8 @@ SweepArgs sweep_args(const mpr_ctx* c, int phase, bool accumulate) {
 }
 
 // n sweeps as one launch
-mpr_status launch_resident_run(mpr_ctx* c, int n, int phase, int flags, bool stats, bool accumulate,
-                               cudaStream_t s) {
+cudaError_t launch_resident_run(mpr_ctx* c, int n, int phase, int flags, bool stats, bool accumulate,
+                                cudaStream_t s) {
     ResidentArgs r{};
     r.a = sweep_args(c, phase, accumulate);
     if (flags & MPR_RECORD_ENERGY) r.a.flags |= kEnergy;
@@ -1127,9 +1127,7 @@ mpr_status launch_resident_run(mpr_ctx* c, int n, int phase, int flags, bool sta
     r.packets = at<ulonglong2>(c->ws, c->L.res_packets);
     r.energies = at<ulonglong2>(c->ws, c->L.res_e);
     r.polls = c->polls;
-    const cudaError_t e = launch_resident(r, r.n_whole + (n_cr - 1), c->res_smem, s);
-    if (e != cudaSuccess) return fail(MPR_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(e));
-    return MPR_OK;
+    return launch_resident(r, r.n_whole + (n_cr - 1), c->res_smem, s);
 }
 
 mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool accumulate,
@@ -1254,21 +1252,36 @@ bool graphs_usable(const mpr_ctx* c, cudaStream_t s) {
     return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
 }
 
-// n sweeps: as one launch (resident sweeps), launched directly, or (sequences of at least 4 sweeps on a stream
-// that may be captured) through a CUDA graph captured once per context and
+// The host's counters after n enqueued sweeps.
+void count_sweeps(mpr_ctx* c, int n, int phase, bool accumulate) {
+    c->sweep += (uint32_t)n;
+    if (phase == MPR_EQUIL) c->equil_index += (uint32_t)n;
+    if (phase != MPR_EQUIL && accumulate) c->n_meas_done += n;
+}
+
+// n sweeps: as one launch (resident sweeps), launched directly, or (sequences of at least
+// 4 sweeps on a stream that may be captured) through a CUDA graph captured once per context and
 // replayed.  Every argument of the launches is fixed for the context's life
 // (temperatures, a, the sweep counter live in device memory), so a graph
 // stays valid.
 mpr_status run_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool accumulate,
                       cudaStream_t s) {
+    int done = 0;  // sweeps that went to resident launches
+    if (resident_runs(c, phase, flags)) {
+        const cudaError_t e = resident_chunks(
+            n, [&](int m) { return launch_resident_run(c, m, phase, flags, stats, accumulate, s); }, &done);
+        if (e != cudaSuccess) return fail(MPR_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(e));
+        if (done < n) {  // refused: launches per colour from here on
+            cudaGetLastError();
+            c->resident = false;
+        }
+    }
+    count_sweeps(c, done, phase, accumulate);
+    n -= done;
+    if (n == 0) return MPR_OK;
     // (a caller that is capturing gets the launches in its own capture)
     const bool graph = n >= 4 && graphs_usable(c, s);
-    if (n > 0 && resident_runs(c, phase, flags)) {
-        // (a chain's word holds 2^40 accepted proposals: 2^20 sweeps of 2048 tiles)
-        constexpr int kMost = 1 << 20;
-        for (int k = 0; k < n; k += kMost)
-            MPR_TRY(launch_resident_run(c, std::min(n - k, kMost), phase, flags, stats, accumulate, s));
-    } else if (!graph) {
+    if (!graph) {
         MPR_TRY(launch_sweeps(c, n, phase, flags, stats, accumulate, s));
     } else {
         const long long key = ((long long)n << 8) | (phase << 4) | ((flags & 1) << 3) |
@@ -1294,9 +1307,7 @@ mpr_status run_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool 
         }
         MPR_CUDA(cudaGraphLaunch(exec, s));
     }
-    c->sweep += (uint32_t)n;
-    if (phase == MPR_EQUIL) c->equil_index += (uint32_t)n;
-    if (phase != MPR_EQUIL && accumulate) c->n_meas_done += n;
+    count_sweeps(c, n, phase, accumulate);
     return MPR_OK;
 }
 

@@ -44,6 +44,24 @@ __host__ __device__ inline unsigned resident_smem(int n0, int n1, int h0, int h1
     return (unsigned)kResidentFixed + 32u * n + resident_sum_bytes(n0 > n1 ? n0 : n1) +
            (tables > 1024u ? tables : 1024u);
 }
+// n sweeps as resident launches of at most kMost each (a chain's word holds 2^40 accepted
+// proposals: 2^20 sweeps of 2048 tiles).  *done: the sweeps launched.  A launch that is
+// refused because the blocks cannot run at once is no error: a context may use fewer SMs
+// than the device has, by which residency was decided, and the sweeps left over can go as
+// launches per colour (*done < n).
+constexpr int kMostSweeps = 1 << 20;
+template <typename Launch>
+cudaError_t resident_chunks(int n, Launch launch, int* done) {
+    for (*done = 0; *done < n;) {
+        const int m = n - *done < kMostSweeps ? n - *done : kMostSweeps;
+        const cudaError_t e = launch(m);
+        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) return cudaSuccess;
+        if (e != cudaSuccess) return e;
+        *done += m;
+    }
+    return cudaSuccess;
+}
+
 // Blocks that record the energies of a group of that many chains.
 int resident_recorders(int group);
 // Blocks of that size that the device holds at once (0: no cooperative launches, or
