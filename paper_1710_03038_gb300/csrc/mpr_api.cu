@@ -465,26 +465,33 @@ __global__ void newton_init_kernel(ImgDev* sub_img, const ImgDev* main_img, doub
 
 // ======================================================= dense views
 
-// H of every (image, chain) (blockIdx.y) of the plain path, FP64 sums of FP32 bond terms.
-__global__ void energy_kernel(const ImgDev* img, const float* state, int n_chains, float q, float J,
-                              int gmrf, double* out) {
+// H of every (image, chain) (blockIdx.y), a thread per pixel, FP64 sums of FP32 bond terms:
+// the plain path, and small batches or single chains of the tiled one (mpr_energy).
+template <bool TILED>
+__global__ void energy_kernel(const ImgDev* img, const float* state, const float* samp, const int* slot_map,
+                              int n_chains, float q, float J, int gmrf, double* out) {
     const int ic = blockIdx.y;
     const int im = ic / n_chains, chain = ic - im * n_chains;
     const ImgDev& I = img[im];
     const float* st = state + state_index(I, chain, 0);
+    const auto value = [&](long long i) {
+        if (!TILED) return fabsf(st[i]);
+        const int s = slot_map[I.site_off + i];
+        return s >= 0 ? st[s * I.sstride] : samp[I.site_off + i];
+    };
     const long long n = (long long)I.Lx * I.Ly;
     double s = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(i % I.Lx), y = (int)(i / I.Lx);
-        const float v = fabsf(st[i]);
+        const float v = value(i);
         float e = 0.0f;
         if (x + 1 < I.Lx) {
-            const float d = v - fabsf(st[i + 1]);
+            const float d = v - value(i + 1);
             e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
         }
         if (y + 1 < I.Ly) {
-            const float d = v - fabsf(st[i + I.Lx]);
+            const float d = v - value(i + I.Lx);
             e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
         }
         s += (double)e;
@@ -1782,14 +1789,22 @@ mpr_status mpr_energy(mpr_ctx* c, double* e_out, mpr_mem where, mpr_stream strea
     long long maxn = 0;
     for (int i = 0; i < c->g.n_img; ++i) maxn = std::max(maxn, (long long)c->g.Lx[i] * c->g.Ly[i]);
     const int gmrf = c->p.model == MPR_MODEL_GMRF ? 1 : 0;
-    if (c->g.path == MPR_PATH_TILED) {
+    // a block per tile, but a thread per pixel where that is the shorter way: batches of fewer
+    // than 2^16 pixels x chains (us, tile / pixel: 64^2 x 10 11.4 / 10.2, x 16 11.8 / 12.1; 128^2
+    // x 2 12.3 / 10.7, x 4 12.2 / 12.8) and single chains of large maps (1000 x 777 27.8 / 21.3,
+    // 2048^2 81 / 53; 256^2 11.8 / 13.1)
+    const bool by_tile = c->g.path == MPR_PATH_TILED && c->g.n_sites * c->g.n_chains >= (1 << 16) &&
+                         (c->g.n_chains > 1 || maxn < (1 << 18));
+    if (by_tile) {
         const int most = *std::max_element(c->g.ntiles.begin(), c->g.ntiles.end());
         MPR_CUDA(launch_energy_tiles(c->d_img, c->d_tiles, c->g.n_img, most, c->g.tx, c->g.ty, c->d_state,
                                      c->d_samp, c->d_slot_map, c->g.n_chains, (float)c->p.q, (float)c->p.J,
                                      gmrf, d_out, s));
     } else {
-        energy_kernel<<<dim3(grid_for(maxn, 256, 512), nc), 256, 0, s>>>(
-            c->d_img, c->d_state, c->g.n_chains, (float)c->p.q, (float)c->p.J, gmrf, d_out);
+        const auto kernel = c->g.path == MPR_PATH_TILED ? energy_kernel<true> : energy_kernel<false>;
+        kernel<<<dim3(grid_for(maxn, 256, 512), nc), 256, 0, s>>>(c->d_img, c->d_state, c->d_samp, c->d_slot_map,
+                                                                  c->g.n_chains, (float)c->p.q, (float)c->p.J,
+                                                                  gmrf, d_out);
         MPR_CUDA(cudaGetLastError());
     }
     energy_finish_kernel<<<grid_for(nc), 256, 0, s>>>(c->d_img, c->d_ctl, d_out, c->g.n_chains, nc);

@@ -144,75 +144,102 @@ state_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int npix
     }
 }
 
-// H of 32 chains of an image (blockIdx.y, z): a lane is a chain, a block walks strips of
-// STRIP rows of a tile.  The strip's angles and those right of and below it lie in
-// shared memory, a row of 32 chains per pixel.  FP32 bond terms as before; their sum in
-// two FP32 words (TwoSum: the rounding error of every addition is kept), FP64 from
-// there: an FP64 addition per pixel and chain ran at 1/32 of the rate.  Bound by the
-// two cosines per pixel and chain; small batches by the chain of a warp's pixels: they
-// take strips of two rows, four warps to a row (64^2 x 32: 23 us with whole tiles).
-template <int STRIP, int NW>
+// H of the chains r_base to r_end of an image (blockIdx.z), C to a block (blockIdx.y): a lane
+// is a pixel and a chain, C chains (a power of two) beside one another and 32 / C pixels,
+// so that batches of few chains leave few lanes idle.  A block walks strips of STRIP rows
+// of a tile.  The strip's angles and those right of and below it lie in shared memory, a
+// row of C chains per pixel.  FP32 bond terms; their sum in two FP32 words (two_sum), FP64
+// from the strip on: an FP64 addition per pixel and chain ran at 1/32 of the rate.  Bound
+// by the two cosines per pixel and chain; small batches by the chain of a warp's pixels.
+// 1000 x 777, us a call with 2, 4, 10, 16 and 24 chains: a thread per pixel and chain 35, 46,
+// 85, 126, 176; a lane per chain whatever their number 107, 107, 115, 115, 116; this 32, 39,
+// 75, 75, 112.
+template <int STRIP, int NW, int C>
 __global__ void __launch_bounds__(NW * 32)
 energy_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int ty, const float* state,
-                   const float* samp, const int* slot_map, int n_chains, float q, float J, int gmrf,
-                   double* out) {
-    extern __shared__ float ang[];  // [(STRIP + 1) x (tx + 1)][32]
-    __shared__ double part[NW][32];
-    constexpr int kParts = NW > STRIP ? NW / STRIP : 1;  // warps to a row
+                   const float* samp, const int* slot_map, int n_chains, int r_base, int r_end, float q,
+                   float J, int gmrf, double* out) {
+    extern __shared__ float ang[];  // [(STRIP + 1) x (tx + 1)][C]
+    __shared__ double part[NW][C];
+    constexpr int kPixels = 32 / C;  // pixels of a warp side by side
     const ImgDev& I = img[blockIdx.z];
     const int Lx = I.Lx, Ly = I.Ly, tx = 1 << tx_log, ew = tx + 1, strips = ty / STRIP;
-    const int r0 = blockIdx.y * 32, nr = min(32, n_chains - r0);
+    const int r0 = r_base + blockIdx.y * C, nr = min(C, r_end - r0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = min(lane, nr - 1);  // idle lanes repeat the last chain
+    const int ch = lane & (C - 1), px = lane / C;
+    const int r = min(ch, nr - 1);  // lanes without a chain repeat the last one
     double sum = 0.0;
     for (int t = blockIdx.x; t < I.ntiles * strips; t += gridDim.x) {
         const TileDesc& T = tiles[I.tile0 + t / strips];
         const int x00 = T.x0, y00 = T.y0 + t % strips * STRIP;
         // with the neighbours that exist (rows below the image: nothing to do)
         const int w = min(ew, Lx - x00), h = min(STRIP + 1, Ly - y00);
+        const float* st = state + I.state_off + r0 + r;
         __syncthreads();
         for (int y = warp; y < h; y += NW) {
-            // a row's slots and samples by lane, then its cells' rows of chains, all in flight
             const long long s0 = I.site_off + (long long)(y00 + y) * Lx + x00;
-            for (int x0 = 0; x0 < w; x0 += 32) {
-                const bool in = x0 + lane < w;
-                const int slot = in ? slot_map[s0 + x0 + lane] : -1;
-                const float sample = in ? samp[s0 + x0 + lane] : 0.0f;
+            if (C == 32) {
+                // a row's slots and samples by lane, then its cells' rows of chains, all in flight
+                for (int x0 = 0; x0 < w; x0 += 32) {
+                    const bool in = x0 + lane < w;
+                    const int slot = in ? slot_map[s0 + x0 + lane] : -1;
+                    const float sample = in ? samp[s0 + x0 + lane] : 0.0f;
 #pragma unroll 8
-                for (int x = 0; x < min(32, w - x0); ++x) {
-                    const int s = __shfl_sync(0xffffffffu, slot, x);
-                    const float v = __shfl_sync(0xffffffffu, sample, x);
-                    ang[(y * ew + x0 + x) * 32 + lane] =
-                        s >= 0 ? state[I.state_off + (long long)s * I.sstride + r0 + r] : v;
+                    for (int x = 0; x < min(32, w - x0); ++x) {
+                        const int s = __shfl_sync(0xffffffffu, slot, x);
+                        const float v = __shfl_sync(0xffffffffu, sample, x);
+                        ang[(y * ew + x0 + x) * C + lane] = s >= 0 ? st[(long long)s * I.sstride] : v;
+                    }
+                }
+            } else {
+#pragma unroll 4
+                for (int x = px; x < w; x += kPixels) {
+                    const int s = slot_map[s0 + x];
+                    ang[(y * ew + x) * C + ch] = s >= 0 ? st[(long long)s * I.sstride] : samp[s0 + x];
                 }
             }
         }
         __syncthreads();
-        const int hn = min(STRIP, Ly - y00), x_lo = warp % kParts * (tx / kParts);
-        const int x_hi = min(x_lo + tx / kParts, Lx - x00);
+        const int hn = min(STRIP, Ly - y00);
         float hi = 0.0f, lo = 0.0f;
-        for (int y = warp / kParts; y < hn; y += NW / kParts) {
-            const float* a = ang + y * ew * 32 + lane;
-            float v = x_lo < x_hi ? a[x_lo * 32] : 0.0f;
+        // the bonds to the right of and below pixel x of row y
+        const auto bonds = [&](const float* a, int x, int y, float v, float right) {
+            float e = 0.0f;
+            if (x + 1 < w) {
+                const float d = v - right;
+                e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
+            }
+            if (y + 1 < h) {
+                const float d = v - a[ew * C];
+                e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
+            }
+            two_sum(hi, lo, e);
+        };
+        if (C == 32) {
+            const int x_hi = min(tx, Lx - x00);
+            for (int y = warp; y < hn; y += NW) {
+                const float* a = ang + y * ew * C + lane;
+                float v = *a;
 #pragma unroll 4
-            for (int x = x_lo; x < x_hi; ++x) {
-                float e = 0.0f, right = 0.0f;
-                if (x + 1 < w) {
-                    right = a[(x + 1) * 32];
-                    const float d = v - right;
-                    e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
+                for (int x = 0; x < x_hi; ++x, a += C) {
+                    const float right = x + 1 < w ? a[C] : 0.0f;
+                    bonds(a, x, y, v, right);
+                    v = right;
                 }
-                if (y + 1 < h) {
-                    const float d = v - a[(ew + x) * 32];
-                    e += gmrf ? J * gmrf_bond(d) : -J * cosf(q * d);
-                }
-                two_sum(hi, lo, e);
-                v = right;
+            }
+        } else {
+            for (int i = warp * kPixels + px; i < hn * tx; i += NW * kPixels) {
+                const int x = i & (tx - 1), y = i >> tx_log;
+                if (x00 + x >= Lx) continue;
+                const float* a = ang + (y * ew + x) * C + ch;
+                bonds(a, x, y, *a, x + 1 < w ? a[C] : 0.0f);
             }
         }
         sum += two_sum_value(hi, lo);
     }
-    part[warp][lane] = sum;
+#pragma unroll
+    for (int o = C; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane < C) part[warp][lane] = sum;
     __syncthreads();
     if (warp == 0 && lane < nr) {
         double s = 0.0;
@@ -258,23 +285,46 @@ cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_t
 cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles, int tx,
                                 int ty, const float* state, const float* samp, const int* slot_map,
                                 int n_chains, float q, float J, int gmrf, double* out, cudaStream_t s) {
-    const int groups = (n_chains + 31) / 32;
-    const auto launch = [&](auto kernel, int strip, int nw, int per_sm) {
-        const size_t smem = (size_t)(tx + 1) * (strip + 1) * 32 * sizeof(float);
+    const auto launch = [&](auto kernel, int strip, int C, int r_base, int chains) {
+        const int groups = (chains + C - 1) / C;
+        const size_t smem = (size_t)(tx + 1) * (strip + 1) * C * sizeof(float);
         if (smem > 48 * 1024) {  // (32 x 32 tiles)
             const cudaError_t e =
                 cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        const long long most = 152LL * per_sm / std::max(1, groups * n_img) + 1;
+        const long long most = 152LL * 8 / std::max(1, groups * n_img) + 1;
         const int blocks = (int)std::max(1LL, std::min((long long)max_tiles * (ty / strip), most));
-        kernel<<<dim3(blocks, groups, n_img), nw * 32, smem, s>>>(img, tiles, log2_of(tx), ty, state, samp,
-                                                                  slot_map, n_chains, q, J, gmrf, out);
+        kernel<<<dim3(blocks, groups, n_img), 256, smem, s>>>(img, tiles, log2_of(tx), ty, state, samp, slot_map,
+                                                              n_chains, r_base, r_base + chains, q, J, gmrf, out);
         return cudaGetLastError();
     };
-    // the line: below four blocks per SM of whole tiles the strips are the shorter chain
-    if ((long long)max_tiles * groups * n_img < 152 * 4) return launch(energy_tile_kernel<2, 8>, 2, 8, 8);
-    return launch(energy_tile_kernel<16, 8>, 16, 8, 8);
+    const auto chains_to_lanes = [](int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : 32; };
+    // below a tile per SM strips of two rows are the shorter chain (us, strips / tiles: 128^2 x 16
+    // 14.5 / 18.8, x 4 12.2 / 14.5; 256^2 x 4 20.6 / 15.4, x 16 20.9 / 20.4), by at most 16
+    // chains (64^2 x 20 14.4 by 32, 11.6 by 16)
+    if ((long long)max_tiles * ((n_chains + 31) / 32) * n_img < 152) {
+        switch (chains_to_lanes(n_chains)) {
+            case 1: return launch(energy_tile_kernel<2, 8, 1>, 2, 1, 0, n_chains);
+            case 2: return launch(energy_tile_kernel<2, 8, 2>, 2, 2, 0, n_chains);
+            case 4: return launch(energy_tile_kernel<2, 8, 4>, 2, 4, 0, n_chains);
+            case 8: return launch(energy_tile_kernel<2, 8, 8>, 2, 8, 0, n_chains);
+            default: return launch(energy_tile_kernel<2, 8, 16>, 2, 16, 0, n_chains);
+        }
+    }
+    // whole groups of 32 chains, then the chains left over by as many lanes as they need
+    const int rest = n_chains % 32, whole = rest > 16 ? n_chains : n_chains - rest;
+    if (whole) {
+        const cudaError_t e = launch(energy_tile_kernel<16, 8, 32>, 16, 32, 0, whole);
+        if (e != cudaSuccess || whole == n_chains) return e;
+    }
+    switch (chains_to_lanes(rest)) {
+        case 1: return launch(energy_tile_kernel<16, 8, 1>, 16, 1, whole, rest);
+        case 2: return launch(energy_tile_kernel<16, 8, 2>, 16, 2, whole, rest);
+        case 4: return launch(energy_tile_kernel<16, 8, 4>, 16, 4, whole, rest);
+        case 8: return launch(energy_tile_kernel<16, 8, 8>, 16, 8, whole, rest);
+        default: return launch(energy_tile_kernel<16, 8, 16>, 16, 16, whole, rest);
+    }
 }
 
 }  // namespace mpr

@@ -231,3 +231,26 @@ def test_states_out_by_quads_and_by_pixels(shape, R):
     torch.cuda.synchronize()
     assert float(flat[0]) == -7.0
     assert torch.equal(flat[1:].view(R, h, w), out[0][1])
+
+
+# chains to a block 1, 2, 4, 8, 16 and 32, with and without lanes left over, and a last group
+# of each width; fewer than 2^16 values by pixel, up to 151 tiles by strips, more by tiles
+@pytest.mark.parametrize("R", [1, 2, 3, 4, 5, 8, 9, 16, 17, 31, 32, 33, 34, 36, 40, 48, 49])
+@pytest.mark.parametrize("shape,tile,model", [((53, 37), (16, 16), "mpr"), ((150, 130), (16, 16), "mpr"),
+                                              ((211, 203), (16, 16), "mpr"), ((211, 203), (16, 16), "gmrf"),
+                                              ((520, 515), (32, 32), "mpr")])
+def test_chain_energies_of_every_lane_split(R, shape, tile, model):
+    """Energies of every chain against torch in FP64 on the states read back."""
+    h, w = shape
+    z = synthetic.grf(shape, nu=0.5, ell=6.0, mean=50, std=10, seed=7).astype(np.float32)
+    g = synthetic.uniform_gaps(shape, 0.5, 8).astype(np.uint8)
+    ctx = mpr.Context([z], [g], chains=R, params=mpr.Params(seed=9, tile=tile, model=model))
+    d = ctx.get_state()[0].double()
+    dx, dy = d[:, :, 1:] - d[:, :, :-1], d[:, 1:] - d[:, :-1]
+    if model == "gmrf":
+        want = sum((t * t / (2 * np.pi ** 2) - 1).sum((1, 2)) for t in (dx, dy))
+    else:
+        want = -sum(torch.cos(0.5 * t).sum((1, 2)) for t in (dx, dy))
+    want /= h * (w - 1) + w * (h - 1)
+    # FP32 differences and bonds of angles below 2 pi: 5e-7 a bond
+    assert np.max(np.abs(ctx.energy()[0] - want.cpu().numpy())) < 5e-7
