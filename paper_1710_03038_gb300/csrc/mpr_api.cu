@@ -1905,9 +1905,13 @@ static mpr_status state_copy(mpr_ctx* c, float* phi, mpr_mem where, int dir, cud
     if (where == MPR_DEVICE) {
         long long maxn = 0;
         for (int i = 0; i < c->g.n_img; ++i) maxn = std::max(maxn, (long long)c->g.Lx[i] * c->g.Ly[i]);
-        // (below 2^18 values a thread per pixel and chain is the shorter chain: 64^2 x 32 4.6
-        // against 6.6 us, 128^2 x 16 6.4 against 6.5)
-        if (tiled && maxn * nc >= (1LL << 18)) {
+        // By tile, 32 chains to a block, or a thread per pixel and chain: the latter below 2^18
+        // values (64^2 x 32 4.6 against 6.6 us) and where a tile holds fewer than 4.5 chains of all
+        // its pixels (the block's lanes are chains).  us out, pixel / tile: 2000^2 x 1 19 / 56, x 4
+        // 63 / 87, x 6 121 / 101, x 16 427 / 126; 1000 x 777 x 4 15 / 17, x 8 25 / 21; 65535 x 2 x 8
+        // 11 / 19, x 32 29 / 27; the line lies where large maps cross it.
+        const double values = (double)c->g.n_sites * c->g.n_chains;
+        if (tiled && maxn * nc >= (1LL << 18) && values > 4.5 * c->g.n_tiles * (c->g.tx * c->g.ty)) {
             MPR_CUDA(launch_state_tiles(c->d_img, c->d_tiles, c->g.n_tiles, c->g.tx, c->g.ty,
                                         std::min(c->g.tx * c->g.ty, c->n_cap[0] + c->n_cap[1]), c->d_slot_pos,
                                         c->d_samp, c->d_state, c->g.n_chains, c->d_ctl, phi, dir == 1, s));

@@ -254,3 +254,24 @@ def test_chain_energies_of_every_lane_split(R, shape, tile, model):
     want /= h * (w - 1) + w * (h - 1)
     # FP32 differences and bonds of angles below 2 pi: 5e-7 a bond
     assert np.max(np.abs(ctx.energy()[0] - want.cpu().numpy())) < 5e-7
+
+
+# either side of the line between the two ways (4.5 chains of a whole tile): few chains, a
+# thin map with few pixels to a tile, more than one group of chains
+@pytest.mark.parametrize("shape,R", [((256, 256), 4), ((256, 256), 5), ((512, 515), 1), ((20000, 3), 20),
+                                     ((3, 20000), 40), ((20000, 3), 33)])
+def test_states_in_and_out_by_tile_and_by_pixel(shape, R):
+    z = synthetic.grf((64, 64), nu=0.5, ell=6.0, mean=50, std=10, seed=3).astype(np.float32)
+    z = np.resize(z, shape)
+    g = synthetic.uniform_gaps(shape, 0.4, 5).astype(np.uint8)
+    gap = torch.from_numpy(g).cuda() != 0
+    gen = torch.Generator(device="cuda").manual_seed(R)
+    new = torch.rand(R, *shape, device="cuda", generator=gen) * 6.28
+    out = []
+    for path in ("plain", "tiled"):
+        ctx = mpr.Context([z], [g], chains=R, params=mpr.Params(seed=5, path=path))
+        start = ctx.get_state()[0]
+        ctx.set_state([new])
+        out.append((start, ctx.get_state()[0]))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert torch.equal(out[1][1][:, gap], new[:, gap])
