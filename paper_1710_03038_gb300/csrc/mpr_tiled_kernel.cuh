@@ -524,12 +524,18 @@ cudaError_t launch_groups(const SweepArgs& a, cudaStream_t s, bool setup_only) {
 // 2048^2 at 40 % x 4 chains 83 / 99 -> 61 / 61 (one warp), x 16 159 / 173 -> 143 / 156
 // (two); x 8 sampling 128 -> 102, but equilibration 57 -> 62 at 1500^2 x 7: two warps for
 // sampling only; 1024^2 at 50 % x 16 sampling 51 -> 53 with 24 warps per SM: 26 asked for.
+// Launches of less than a wave of four-warp blocks (eight per SM) keep the four warps: their
+// SMs are not full, and a dense tile's steps fall to fewer warps (four warps / fewer /
+// launches before: GMRF 462 x 367 x 10 with a block of gaps 15.6 / 19.1 / 16.2 equilibrating,
+// 11.8 / 16.7 / 17.5 sampling; 500^2 at 40 % x 16, 625 blocks, 17.4 / 20.7 / 20.1; 640 x 480 x
+// 16, 1200 blocks, 18.9 / 20.1 / 19.8; 600^2 x 4, 1444 blocks, 16.1 / 15.2 / 19.7).
 // Passes that record energies keep the four warps, which fix the order of their sums,
 // and so do launches beside another (1024^2 x 100: 276 -> 285).
 constexpr int small_group_warps(int P, bool acc) {
     return P == 2 ? 1 : P == 4 && acc ? 2 : P == 8 ? 2 : 4;
 }
 constexpr int kSmallGroupSmWarps = 26;
+constexpr long long kSmallGroupBlocks = 152 * 8;
 
 template <int TX, int TY, int NW, int P, bool ACC, int MODEL>
 cudaError_t launch_acc(const SweepArgs& a, cudaStream_t s, bool setup_only) {
@@ -541,7 +547,8 @@ cudaError_t launch_acc(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     }
     if (a.flags & kEnergy) return launch_groups<TX, TY, NW, P, ACC, MODEL, true>(a, s, false);
     constexpr size_t kSmBytes = 228 * 1024, kReserved = 1024;  // of an SM, per block
-    if (kFew != NW && a.chain_end - a.chain0 == a.n_chains &&
+    const long long groups = (a.chain_end - a.chain0 + a.chain_group - 1) / a.chain_group;
+    if (kFew != NW && a.chain_end - a.chain0 == a.n_chains && a.n_list * groups >= kSmallGroupBlocks &&
         (Cfg<TX, TY, kFew, MODEL>::smem_for(a.gt, a.n_cap, P) + kReserved) *
                 ((kSmallGroupSmWarps + kFew - 1) / kFew) <= kSmBytes)
         return launch_groups<TX, TY, kFew, P, ACC, MODEL, false>(a, s, false);

@@ -275,3 +275,22 @@ def test_states_in_and_out_by_tile_and_by_pixel(shape, R):
         out.append((start, ctx.get_state()[0]))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
     assert torch.equal(out[1][1][:, gap], new[:, gap])
+
+
+@pytest.mark.parametrize("R,model", [(4, "mpr"), (3, "gmrf"), (8, "mpr"), (7, "mpr"), (16, "mpr"), (13, "gmrf")])
+def test_blocks_of_fewer_warps_equal_the_plain_path(R, model):
+    """1404 tiles: more than a wave of blocks, where small chain groups take fewer warps."""
+    z = synthetic.grf((610, 575), nu=0.5, ell=9.0, mean=50, std=10, seed=63).astype(np.float32)
+    g = synthetic.uniform_gaps((610, 575), 0.35, 64).astype(np.uint8)
+    out = []
+    for path in ("plain", "tiled"):
+        ctx = mpr.Context([z], [g], chains=R, params=mpr.Params(seed=80, path=path, model=model))
+        ctx.set_T([0.1])
+        ctx.sweep(3, "equil")
+        ctx.sweep(3, "measure")
+        out.append((ctx.get_state()[0], ctx.chain_info(), ctx.predict()[0]))
+    assert torch.equal(out[0][0], out[1][0])
+    for k in ("a", "accepted"):
+        assert np.array_equal(out[0][1][k], out[1][1][k])
+    # the mean of angles rounded to 2^-24 rad, mapped back and rounded to FP32
+    assert torch.allclose(out[0][2], out[1][2], rtol=1e-6, atol=1e-5)
