@@ -315,7 +315,6 @@ def run_gpu(args):
 
     sweep_events = []
     equil_events = []
-    launches = []
 
     def step(z_in, g_in, host_out=None, timed=False):
         ctx = mpr.Context([z_in], [g_in], chains=R, params=params, topts=topts, device=dev)
@@ -329,8 +328,6 @@ def run_gpu(args):
             q0 = torch.cuda.Event(enable_timing=True)
             q1 = torch.cuda.Event(enable_timing=True)
             q0.record(stream)
-        if not launches:
-            launches.extend(ctx.sweep_launches())
         ctx.sweep(ne, "equil")
         if timed:
             q1.record(stream)
@@ -365,10 +362,13 @@ def run_gpu(args):
     torch.cuda.synchronize()
     t0 = torch.cuda.Event(enable_timing=True)
     t1 = torch.cuda.Event(enable_timing=True)
+    # kernels of the timed steps, as the library launched them
+    gpu_launches = mpr.launch_count()
     t0.record(stream)
     for _ in range(args.steps):
         step(z_d, g_d, timed=True)
     t1.record(stream)
+    gpu_launches = mpr.launch_count() - gpu_launches
     torch.cuda.synchronize()
     barrier()
     ms = t0.elapsed_time(t1)
@@ -430,13 +430,7 @@ def run_gpu(args):
                 "d2h_bytes_per_step": N * 4},
         "clocks": clocks,
     }
-    # kernel launches of one step: the library's per-sweep count for the realisations,
-    # two runs of the temperature lattices per Newton step (each one launch), the Newton
-    # steps (and their set-up), the 16 initialisation kernels of the two contexts (map,
-    # extremes, sample energy, tile tables, hot starts, chain set-up) and the prediction
-    # (the sampling sweeps of a run share one bookkeeping launch)
-    line["gpu_launches"] = args.steps * (launches[0] * (ne + nm) - (nm - 1) + 2 * topts.iters
-                                         + topts.iters + 1 + 16 + 1)
+    line["gpu_launches"] = gpu_launches
     if not args.no_plain:
         # the plain single-image path on the same job (one warm-up, one timed step)
         plain = mpr.Params(seed=12345 + rank, path="plain")

@@ -243,6 +243,12 @@ mpr_status mpr_select_q(int Lx, int Ly, const float* z, const uint8_t* gap, cons
  * Host only. */
 mpr_status mpr_sweep_launches(const mpr_ctx* ctx, int* per_sweep, int* per_T_sweep);
 
+/* Kernels that this thread's calls into the library have enqueued so far: runs of sweeps as
+ * they went (resident, launched, or a graph replay's kernels), set-up, estimates and
+ * reads alike.  A call made while the caller captures counts once, at the capture.
+ * Host only. */
+int64_t mpr_launch_count(void);
+
 /* Sets / reads the reduced temperature of every image (host [n_img]). */
 mpr_status mpr_set_T(mpr_ctx* ctx, const double* T, mpr_stream stream);
 mpr_status mpr_get_T(mpr_ctx* ctx, double* T, mpr_stream stream);

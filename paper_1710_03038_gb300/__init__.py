@@ -519,6 +519,11 @@ class MPREnergy(torch.autograd.Function):
         return g_phi, g_J, None
 
 
+def launch_count() -> int:
+    """Kernels that this thread's calls into the library have enqueued so far."""
+    return int(_lib.load().mpr_launch_count())
+
+
 def math_probe(fn: int, a: torch.Tensor, b: torch.Tensor = None) -> torch.Tensor:
     """The library's own approximations (fn 0: atan2, 2: series sine) or CUDA's (1, 3)."""
     a = a.to(torch.float32).contiguous()

@@ -37,7 +37,7 @@ EXPORTS = (
     "mpr_get_accumulators", "mpr_set_accumulators",
     "mpr_eT_table_workspace_size", "mpr_eT_table", "mpr_set_T_from_table", "mpr_autotune",
     "mpr_select_q_workspace_size", "mpr_select_q", "mpr_sweep_launches",
-    "mpr_check", "mpr_set_wait_limit",
+    "mpr_check", "mpr_set_wait_limit", "mpr_launch_count",
 )
 
 
@@ -121,6 +121,7 @@ def load(path: str = LIB_PATH):
             "mpr_sample_energy_noalloc": (i, [i, ip, ip, vp, vp, d, d, vp, vp, vp, vp, vp]),
             "mpr_select_q_workspace_size": (i, [i, i, i, pp, tp, C.POINTER(sz)]),
             "mpr_sweep_launches": (i, [vp, ip, ip]),
+            "mpr_launch_count": (C.c_int64, []),
             "mpr_check": (i, [vp, vp]),
             "mpr_set_wait_limit": (i, [vp, i]),
             "mpr_select_q": (i, [i, i, vp, vp, vp, i, i, dp, i, i, i, pp, tp, vp, sz, dp, dp, dp,

@@ -20,6 +20,7 @@ using namespace mpr;
 namespace {
 
 thread_local std::string g_last_error;
+thread_local long long g_launches = 0;
 
 mpr_status fail(mpr_status s, const std::string& msg) {
     g_last_error = msg;
@@ -196,6 +197,7 @@ int default_T_side(int Lx, int Ly, const mpr_T_opts& o) {
 }  // namespace
 
 mpr_status mpr::set_last_error(mpr_status s, const std::string& msg) { return fail(s, msg); }
+long long& mpr::launch_total() { return g_launches; }
 
 // ============================================================== context
 
@@ -251,18 +253,23 @@ struct mpr_ctx {
     int polls = kDefaultPolls;  // reads of a wait of a resident run before it gives up
     mpr_ctx* sub = nullptr;   // unconditional lattices of the temperature estimate
     // instantiated CUDA graphs of sweep sequences, keyed by (n, phase, flags, stats, accumulate)
-    std::vector<std::pair<long long, cudaGraphExec_t>> graphs;
+    struct SweepGraph {
+        long long key;
+        cudaGraphExec_t exec;
+        long long kernels;
+    };
+    std::vector<SweepGraph> graphs;
     // the equilibration with its stop rule as one device-side while loop, keyed by
     // (n_f, n_fit, i_max)
     cudaGraphExec_t eq_exec = nullptr;
-    long long eq_key = -1;
+    long long eq_key = -1, eq_kernels = 0;  // (kernels of an iteration)
     // tiled path: a second stream and two events, so that a colour pass's launch
     // for its heavy tiles and the one for the chains left over by the chain
     // groups run beside the main launch (they touch other tiles or chains)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     ~mpr_ctx() {
-        for (auto& g : graphs) cudaGraphExecDestroy(g.second);
+        for (auto& g : graphs) cudaGraphExecDestroy(g.exec);
         if (eq_exec) cudaGraphExecDestroy(eq_exec);
         if (ev_fork) cudaEventDestroy(ev_fork);
         if (ev_join) cudaEventDestroy(ev_join);
@@ -1024,12 +1031,12 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
         } else {
             init_plain_kernel<<<grid_for((long long)Lx[i] * Ly[i] * n_chains), 256, 0, s>>>(
                 c->d_img, c->d_samp, c->d_state, i, n_chains, key, c->img_tag);
+            MPR_CUDA(launched());
         }
-        MPR_CUDA(cudaGetLastError());
     }
     const int nc = n_img * n_chains;
     init_chains_kernel<<<grid_for(nc), 256, 0, s>>>(c->ch, nc);
-    MPR_CUDA(cudaGetLastError());
+    MPR_CUDA(launched());
     MPR_CUDA(cudaMemsetAsync(c->d_ctl, 0, sizeof(Control), s));
     MPR_CUDA(cudaMemsetAsync(c->d_acc1, 0, sizeof(double) * c->L.n_slots, s));
     MPR_CUDA(cudaMemsetAsync(c->d_acc2, 0, sizeof(double) * c->L.n_slots, s));
@@ -1213,7 +1220,7 @@ mpr_status launch_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bo
         end_sweep_kernel<<<std::min((nc + 7) / 8, 1024), 256, 0, s>>>(
             c->d_img, c->ch, c->d_ctl, c->g.n_img, c->g.n_chains, equil ? 1 : 0, record ? 1 : 0,
             stats ? 1 : 0, tiled ? 1 : 0, c->p.A_targ, c->p.k_a, once ? n : 1);
-        MPR_CUDA(cudaGetLastError());
+        MPR_CUDA(launched());
     }
     return MPR_OK;
 }
@@ -1294,12 +1301,16 @@ mpr_status run_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool 
         const long long key = ((long long)n << 8) | (phase << 4) | ((flags & 1) << 3) |
                               ((stats ? 1 : 0) << 2) | ((accumulate ? 1 : 0) << 1);
         cudaGraphExec_t exec = nullptr;
+        long long kernels = 0;
         for (auto& g : c->graphs)
-            if (g.first == key) exec = g.second;
+            if (g.key == key) { exec = g.exec; kernels = g.kernels; }
         if (!exec) {
             MPR_TRY(prepare_capture(c, s));
             MPR_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+            const long long before = launch_total();
             const mpr_status st = launch_sweeps(c, n, phase, flags, stats, accumulate, s);
+            kernels = launch_total() - before;
+            launch_total() = before;
             cudaGraph_t g = nullptr;
             const cudaError_t e = cudaStreamEndCapture(s, &g);
             if (st != MPR_OK) {
@@ -1310,9 +1321,10 @@ mpr_status run_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool 
             const cudaError_t ei = cudaGraphInstantiate(&exec, g, 0);
             cudaGraphDestroy(g);
             if (ei != cudaSuccess) return fail(MPR_ERR_CUDA, std::string("instantiate: ") + cudaGetErrorString(ei));
-            c->graphs.emplace_back(key, exec);
+            c->graphs.push_back({key, exec, kernels});
         }
         MPR_CUDA(cudaGraphLaunch(exec, s));
+        launch_total() += kernels;
     }
     count_sweeps(c, n, phase, accumulate);
     return MPR_OK;
@@ -1482,7 +1494,7 @@ mpr_status mpr_set_T(mpr_ctx* c, const double* T, mpr_stream stream) {
     double* tmp = c->d_newton;  // 4 doubles per image of room
     MPR_CUDA(cudaMemcpyAsync(tmp, T, sizeof(double) * c->g.n_img, cudaMemcpyHostToDevice, s));
     set_T_kernel<<<grid_for(c->g.n_img), 256, 0, s>>>(c->d_img, tmp, c->g.n_img);
-    MPR_CUDA(cudaGetLastError());
+    MPR_CUDA(launched());
     MPR_CUDA(cudaStreamSynchronize(s));
     for (int i = 0; i < c->g.n_img; ++i) { c->h_img[i].T = T[i]; c->h_img[i].invT = (float)(1.0 / T[i]); }
     c->T_set = true;
@@ -1520,14 +1532,14 @@ mpr_status mpr_estimate_T(mpr_ctx* c, double* T_out, mpr_stream stream) {
     const int K = u->g.n_chains;
     newton_init_kernel<<<grid_for(n_img), 256, 0, s>>>(u->d_img, c->d_img, c->d_newton, n_img,
                                                       c->topt.T_lo, c->topt.T_hi, J);
-    MPR_CUDA(cudaGetLastError());
+    MPR_CUDA(launched());
     for (int it = 0; it < c->topt.iters; ++it) {
         const int neq = it == 0 ? 2 * c->topt.n_equil : c->topt.n_equil;
         MPR_TRY(run_sweeps(u, neq, MPR_EQUIL, 0, false, false, s));
         MPR_TRY(run_sweeps(u, c->topt.n_meas, MPR_MEASURE, MPR_RECORD_ENERGY, true, false, s));
         newton_kernel<<<grid_for(n_img), 256, 0, s>>>(u->d_img, c->d_img, u->ch, c->d_newton, n_img,
                                                      K, c->topt.n_meas, u->d_ctl, c->d_ctl);
-        MPR_CUDA(cudaGetLastError());
+        MPR_CUDA(launched());
     }
     c->T_set = true;
     if (T_out) MPR_TRY(mpr_get_T(c, T_out, stream));
@@ -1641,7 +1653,7 @@ mpr_status mpr_eT_table(int L, int n_T, const double* T, int chains, int n_equil
     u.img_tag = 1u << 29;  // a stream of its own
     MPR_CUDA(cudaMemcpyAsync(u.d_newton, T, sizeof(double) * n_T, cudaMemcpyHostToDevice, s));
     set_T_kernel<<<grid_for(n_T), 256, 0, s>>>(u.d_img, u.d_newton, n_T);
-    MPR_CUDA(cudaGetLastError());
+    MPR_CUDA(launched());
     MPR_TRY(run_sweeps(&u, n_equil, MPR_EQUIL, 0, false, false, s));
     MPR_TRY(run_sweeps(&u, n_meas, MPR_MEASURE, MPR_RECORD_ENERGY, true, false, s));
     const int nc = n_T * chains;
@@ -1721,12 +1733,15 @@ mpr_status mpr_equilibrate(mpr_ctx* c, int n_f, int n_fit, int i_max, int* n_don
                 e = cudaStreamBeginCaptureToGraph(s, np.conditional.phGraph_out[0], nullptr, nullptr,
                                                   0, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {
+                const long long before = launch_total();
                 st = launch_sweeps(c, 1, MPR_EQUIL, MPR_RECORD_ENERGY, false, true, s);
                 if (st == MPR_OK) {
                     sg_step_kernel<<<1, 256, 0, s>>>(c->ch, c->d_hist, c->d_sg, n_img, c->g.n_chains,
                                                      n_fit, n_f, i_max, h, 1);
-                    e = cudaGetLastError();
+                    e = launched();
                 }
+                c->eq_kernels = launch_total() - before;
+                launch_total() = before;
                 cudaGraph_t body = nullptr;
                 const cudaError_t ee = cudaStreamEndCapture(s, &body);
                 if (e == cudaSuccess) e = ee;
@@ -1741,6 +1756,7 @@ mpr_status mpr_equilibrate(mpr_ctx* c, int n_f, int n_fit, int i_max, int* n_don
         MPR_CUDA(cudaGraphLaunch(c->eq_exec, s));
         MPR_CUDA(cudaMemcpyAsync(&done, c->d_sg + n_img + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
         MPR_CUDA(cudaStreamSynchronize(s));
+        launch_total() += c->eq_kernels * done;
         c->sweep += (uint32_t)done;
         c->equil_index += (uint32_t)done;
     } else {
@@ -1749,7 +1765,7 @@ mpr_status mpr_equilibrate(mpr_ctx* c, int n_f, int n_fit, int i_max, int* n_don
             MPR_TRY(run_sweeps(c, 1, MPR_EQUIL, MPR_RECORD_ENERGY, false, true, s));
             sg_step_kernel<<<1, 256, 0, s>>>(c->ch, c->d_hist, c->d_sg, n_img, c->g.n_chains, n_fit,
                                              n_f, i_max, cudaGraphConditionalHandle{}, 0);
-            MPR_CUDA(cudaGetLastError());
+            MPR_CUDA(launched());
             done = i + 1;
             if (i >= n_fit && i % n_f == 0) {
                 int stop = 0;
@@ -1769,6 +1785,8 @@ mpr_status mpr_sweep_launches(const mpr_ctx* c, int* per_sweep, int* per_T_sweep
     if (per_T_sweep) *per_T_sweep = c->sub ? sweep_launch_count(c->sub) : 0;
     return MPR_OK;
 }
+
+int64_t mpr_launch_count(void) { return launch_total(); }
 
 mpr_status mpr_get_energy_history(mpr_ctx* c, double* out, mpr_stream stream) {
     static_assert(kHist == MPR_HISTORY, "history length");
@@ -1805,10 +1823,10 @@ mpr_status mpr_energy(mpr_ctx* c, double* e_out, mpr_mem where, mpr_stream strea
         kernel<<<dim3(grid_for(maxn, 256, 512), nc), 256, 0, s>>>(c->d_img, c->d_state, c->d_samp, c->d_slot_map,
                                                                   c->g.n_chains, (float)c->p.q, (float)c->p.J,
                                                                   gmrf, d_out);
-        MPR_CUDA(cudaGetLastError());
+        MPR_CUDA(launched());
     }
     energy_finish_kernel<<<grid_for(nc), 256, 0, s>>>(c->d_img, c->d_ctl, d_out, c->g.n_chains, nc);
-    MPR_CUDA(cudaGetLastError());
+    MPR_CUDA(launched());
     if (where == MPR_HOST) {
         MPR_CUDA(cudaMemcpyAsync(e_out, d_out, sizeof(double) * nc, cudaMemcpyDeviceToHost, s));
         MPR_CUDA(cudaStreamSynchronize(s));
@@ -1833,7 +1851,7 @@ mpr_status mpr_predict(mpr_ctx* c, float* z_hat, float* z_std, mpr_mem where, mp
     } else {
         predict_kernel<<<dim3(grid_for(maxn, 256, 2048), c->g.n_img), 256, 0, s>>>(
             c->d_img, c->d_acc1, c->d_acc2, c->d_zst, c->d_samp, n_samples, dh, ds);
-        MPR_CUDA(cudaGetLastError());
+        MPR_CUDA(launched());
     }
     if (where == MPR_HOST) {
         MPR_CUDA(cudaMemcpyAsync(z_hat, dh, sizeof(float) * N, cudaMemcpyDeviceToHost, s));
@@ -1865,7 +1883,7 @@ static mpr_status acc_copy(mpr_ctx* c, double* acc, double* dense, mpr_mem where
     for (int i = 0; i < c->g.n_img; ++i) maxn = std::max(maxn, (long long)c->g.Lx[i] * c->g.Ly[i]);
     acc_dense_kernel<<<dim3(grid_for(maxn, 256, 1024), c->g.n_img), 256, 0, s>>>(
         c->d_img, acc, c->d_slot_map, c->d_samp, c->g.path == MPR_PATH_TILED ? 1 : 0, c->d_ctl, d, dir);
-    MPR_CUDA(cudaGetLastError());
+    MPR_CUDA(launched());
     if (where == MPR_HOST) {
         if (dir == 0) MPR_CUDA(cudaMemcpyAsync(dense, d, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
         MPR_CUDA(cudaStreamSynchronize(s));
@@ -1920,7 +1938,7 @@ static mpr_status state_copy(mpr_ctx* c, float* phi, mpr_mem where, int dir, cud
         state_copy_kernel<<<dim3(grid_for(maxn, 256, 1024), nc), 256, 0, s>>>(
             c->d_img, c->d_state, c->d_samp, c->d_slot_map, tiled, c->g.n_chains, c->d_ctl, phi, dir, 0,
             nullptr);
-        MPR_CUDA(cudaGetLastError());
+        MPR_CUDA(launched());
         return MPR_OK;
     }
     // host buffers: one (image, chain) plane at a time through the output staging area
@@ -1933,7 +1951,7 @@ static mpr_status state_copy(mpr_ctx* c, float* phi, mpr_mem where, int dir, cud
         state_copy_kernel<<<dim3(grid_for(n, 256, 1024), 1), 256, 0, s>>>(
             c->d_img, c->d_state, c->d_samp, c->d_slot_map, tiled, c->g.n_chains, c->d_ctl, nullptr, dir, ic,
             stage);
-        MPR_CUDA(cudaGetLastError());
+        MPR_CUDA(launched());
         if (dir == 0) MPR_CUDA(cudaMemcpyAsync(h, stage, sizeof(float) * n, cudaMemcpyDeviceToHost, s));
     }
     MPR_CUDA(cudaStreamSynchronize(s));
@@ -1972,7 +1990,7 @@ mpr_status mpr_set_chain_a(mpr_ctx* c, const float* a, mpr_stream stream) {
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     MPR_CUDA(cudaMemcpyAsync(c->ch.a, a, sizeof(float) * nc, cudaMemcpyHostToDevice, s));
     set_alpha_kernel<<<grid_for(nc), 256, 0, s>>>(c->ch, nc);
-    MPR_CUDA(cudaGetLastError());
+    MPR_CUDA(launched());
     MPR_CUDA(cudaStreamSynchronize(s));
     return MPR_OK;
 }

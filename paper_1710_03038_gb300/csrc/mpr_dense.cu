@@ -263,7 +263,7 @@ cudaError_t launch_predict_tiles(const ImgDev* img, const TileDesc* tiles, int n
                                  const Control* ctl, float* zhat, float* zstd, cudaStream_t s) {
     predict_tile_kernel<<<n_tiles, 128, 0, s>>>(img, tiles, log2_of(tx), tx * ty, slot_pos, acc1, acc2, z,
                                                 gap, 1.0 / n_samples, ctl, zhat, zstd);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_tiles, int tx, int ty,
@@ -279,7 +279,7 @@ cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_t
     }
     kernel<<<dim3(n_tiles, (n_chains + 31) / 32), 256, smem, s>>>(img, tiles, log2_of(tx), tx * ty, n_max,
                                                                   slot_pos, samp, state, n_chains, ctl, dense);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles, int tx,
@@ -297,7 +297,7 @@ cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_
         const int blocks = (int)std::max(1LL, std::min((long long)max_tiles * (ty / strip), most));
         kernel<<<dim3(blocks, groups, n_img), 256, smem, s>>>(img, tiles, log2_of(tx), ty, state, samp, slot_map,
                                                               n_chains, r_base, r_base + chains, q, J, gmrf, out);
-        return cudaGetLastError();
+        return launched();
     };
     const auto chains_to_lanes = [](int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : 32; };
     // below a tile per SM strips of two rows are the shorter chain (us, strips / tiles: 128^2 x 16

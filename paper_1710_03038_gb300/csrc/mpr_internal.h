@@ -120,6 +120,14 @@ struct SweepArgs {
 // Records the message returned by mpr_last_error() for this thread; returns s.
 mpr_status set_last_error(mpr_status s, const std::string& msg);
 
+// Kernels that this thread has launched (mpr_launch_count).
+long long& launch_total();
+// After n launches: counts them; the error of any.
+inline cudaError_t launched(int n = 1) {
+    launch_total() += n;
+    return cudaGetLastError();
+}
+
 // ---- launchers ------------------------------------------------------------
 // setup_only: set the kernel's attributes without launching (before a capture)
 // (chain_group: even and at most 32, or covering every chain)

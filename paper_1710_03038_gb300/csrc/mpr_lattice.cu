@@ -196,7 +196,7 @@ mpr_status mpr_lattice_energy(int n, const int* Lx, const int* Ly, const float* 
         return MPR_ERR_CUDA;
     return for_chunks(n, Lx, Ly, [&](const Grids& G, int k0, int m, int blocks) {
         lattice_energy_kernel<<<dim3(blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, H_out);
-        return cudaGetLastError();
+        return launched();
     });
 }
 
@@ -207,7 +207,7 @@ mpr_status mpr_lattice_torque(int n, const int* Lx, const int* Ly, const float* 
     return for_chunks(n, Lx, Ly, [&](const Grids& G, int k0, int m, int blocks) {
         lattice_grad_kernel<true, false><<<dim3(blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, g,
                                                                           grad, nullptr);
-        return cudaGetLastError();
+        return launched();
     });
 }
 
@@ -221,7 +221,7 @@ mpr_status mpr_lattice_grad(int n, const int* Lx, const int* Ly, const float* ph
         const auto kernel = !grad_J ? lattice_grad_kernel<true, false>
                             : grad_phi ? lattice_grad_kernel<true, true> : lattice_grad_kernel<false, true>;
         kernel<<<dim3(blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, g, grad_phi, grad_J);
-        return cudaGetLastError();
+        return launched();
     });
 }
 
@@ -231,7 +231,7 @@ mpr_status mpr_philox(int n, const uint32_t* ctr, const uint32_t* key, uint32_t*
     if (n == 0) return MPR_OK;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     philox_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, ctr, make_uint2(key[0], key[1]), out, reference);
-    return cudaGetLastError() == cudaSuccess ? MPR_OK : MPR_ERR_CUDA;
+    return launched() == cudaSuccess ? MPR_OK : MPR_ERR_CUDA;
 }
 
 mpr_status mpr_math_probe(int fn, int n, const float* a, const float* b, float* out,
@@ -240,7 +240,7 @@ mpr_status mpr_math_probe(int fn, int n, const float* a, const float* b, float* 
     if (n == 0) return MPR_OK;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     math_probe_kernel<<<(n + 255) / 256, 256, 0, s>>>(fn, n, a, b, out);
-    return cudaGetLastError() == cudaSuccess ? MPR_OK : MPR_ERR_CUDA;
+    return launched() == cudaSuccess ? MPR_OK : MPR_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -261,7 +261,7 @@ extern "C" mpr_status mpr_sample_energy_noalloc(int n_img, const int* Lx, const 
     noalloc_pairs_kernel<<<grid, kPairThreads, 0, s>>>(S, z, gap, stat, (float)q, (float)J, part);
     noalloc_final_kernel<<<n_img, kNoAllocBlocks, 0, s>>>(part, stat, e_s, reinterpret_cast<long long*>(n_sp),
                                               z_min, z_max);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launched(3);
     if (e != cudaSuccess)
         return set_last_error(MPR_ERR_CUDA, std::string("mpr_sample_energy_noalloc: ") +
                                                 cudaGetErrorString(e));

@@ -168,7 +168,7 @@ cudaError_t launch_plain_pass(const SweepArgs& a, int max_Lx, int max_Ly, cudaSt
     const int half = (max_Lx + 1) / 2;
     dim3 grid((half + kPlainBX - 1) / kPlainBX, max_Ly, a.n_img * ((a.n_chains + 1) / 2));
     plain_pass_kernel<<<grid, kPlainBX, 0, s>>>(a);
-    return cudaGetLastError();
+    return launched();
 }
 
 }  // namespace mpr

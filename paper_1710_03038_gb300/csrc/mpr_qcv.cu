@@ -142,7 +142,7 @@ mpr_status mpr_select_q(int Lx, int Ly, const float* z, const uint8_t* gap, cons
     // gcv is both the image's gap input and the merged output: each element is read
     // and written by the same thread
     qcv_mask_kernel<<<qcv_blocks(N), 256, 0, s>>>(N, dgcv, dhold, dgcv, dacc);
-    if (cudaGetLastError() != cudaSuccess) return set_last_error(MPR_ERR_CUDA, "mpr_select_q: mask kernel");
+    if (mpr::launched() != cudaSuccess) return set_last_error(MPR_ERR_CUDA, "mpr_select_q: mask kernel");
     double acc[2];
     if (cudaMemcpyAsync(acc, dacc, sizeof(acc), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
@@ -174,7 +174,7 @@ mpr_status mpr_select_q(int Lx, int Ly, const float* z, const uint8_t* gap, cons
             st = set_last_error(MPR_ERR_CUDA, "mpr_select_q: memset");
         if (st == MPR_OK) {
             qcv_abs_error_kernel<<<qcv_blocks(N), 256, 0, s>>>(N, dz, dzhat, dhold, dacc);
-            if (cudaGetLastError() != cudaSuccess ||
+            if (mpr::launched() != cudaSuccess ||
                 cudaMemcpyAsync(acc, dacc, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
                 cudaStreamSynchronize(s) != cudaSuccess)
                 st = set_last_error(MPR_ERR_CUDA, "mpr_select_q: validation error");

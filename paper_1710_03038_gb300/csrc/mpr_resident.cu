@@ -57,8 +57,10 @@ cudaError_t launch_resident(const ResidentArgs& ra, int n_groups, size_t smem, c
                           (ra.a.flags & kGMRF) != 0);
     void* args[] = {const_cast<ResidentArgs*>(&ra)};
     const int x = ra.n_tiles + ((ra.a.flags & kEnergy) ? ra.a.n_img * ra.recorders : 0);
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(f), dim3(x, n_groups), dim3(kNT), args,
-                                       smem, s);
+    const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(f), dim3(x, n_groups),
+                                                      dim3(kNT), args, smem, s);
+    if (e == cudaSuccess) ++launch_total();
+    return e;
 }
 
 }  // namespace mpr

@@ -519,7 +519,7 @@ cudaError_t launch_put(void* dst, const void* src, size_t bytes, cudaStream_t s)
         const size_t n = std::min(sizeof(Blob), bytes - o);
         std::memcpy(b.w, static_cast<const char*>(src) + o, n);
         put_kernel<<<1, 256, 0, s>>>(b, reinterpret_cast<uint32_t*>(static_cast<char*>(dst) + o), (int)(n / 4));
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launched();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -528,23 +528,23 @@ cudaError_t launch_put(void* dst, const void* src, size_t bytes, cudaStream_t s)
 cudaError_t launch_minmax(const ImgDev* img, int n_img, long long max_sites, const float* z,
                           const uint8_t* gap, ImgScan* scan, cudaStream_t s) {
     minmax_kernel<<<dim3(blocks_for(max_sites, 4096, 608), n_img), 256, 0, s>>>(img, z, gap, scan);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_tile_count(const ImgDev* img, int n_img, TileDesc* tiles, int n_tiles, const uint8_t* gap,
                               int tx, int ty, int* counts, ImgScan* scan, cudaStream_t s) {
     tile_count_kernel<<<n_tiles, 256, 0, s>>>(img, n_img, tiles, gap, log2_of(tx), tx * ty, ty, counts);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launched();
     if (e != cudaSuccess) return e;
     tile_scan_kernel<<<n_img, 1024, 0, s>>>(img, tiles, counts, scan);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_map(const ImgDev* img, int n_img, long long max_sites, const float* z, const uint8_t* gap,
                        float* samp, bool unconditional, cudaStream_t s) {
     map_kernel<<<dim3(blocks_for(max_sites, 256, 2048), n_img), 256, 0, s>>>(img, z, gap, samp,
                                                                               unconditional ? 1 : 0);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_tile_tables(const ImgDev* img, TileDesc* tiles, int n_tiles, const uint8_t* gap, int tx,
@@ -552,24 +552,24 @@ cudaError_t launch_tile_tables(const ImgDev* img, TileDesc* tiles, int n_tiles, 
                                const float* samp, float q, int gmrf, int literal, uint2* slot_ref,
                                float4* slot_cs, int res_P, TileStats* stats, cudaStream_t s) {
     tile_fill_kernel<<<n_tiles, 256, 0, s>>>(img, tiles, gap, log2_of(tx), tx * ty, slot_pos, slot_map);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launched();
     if (e != cudaSuccess) return e;
     tile_link_kernel<<<n_tiles, 128, sizeof(uint16_t) * (tx + 2) * (ty + 2), s>>>(
         img, tiles, log2_of(tx), ty, slot_pos, slot_map, halo, halo_cap, samp, q, gmrf, literal, slot_ref,
         slot_cs, res_P, stats);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_tile_hist(const TileDesc* tiles, int n_tiles, int* hist, cudaStream_t s) {
     tile_hist_kernel<<<blocks_for(n_tiles, 256, 152), 256, 0, s>>>(tiles, n_tiles, hist);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_tile_split(const TileDesc* tiles, int n_tiles, const int e_max[2], const int own_max[2],
                               int* list, int* n_light, cudaStream_t s) {
     tile_split_kernel<<<2, 1024, 0, s>>>(tiles, n_tiles, make_int2(e_max[0], own_max[0]),
                                          make_int2(e_max[1], own_max[1]), list, n_light);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_hot_start(const ImgDev* img, const uint32_t* slot_pos, float* state, long long slots,
@@ -578,17 +578,17 @@ cudaError_t launch_hot_start(const ImgDev* img, const uint32_t* slot_pos, float*
     if (n == 0) return cudaSuccess;
     hot_start_kernel<<<blocks_for(n, 1024, 152 * 32), 256, 0, s>>>(img, slot_pos, state, slots, img_i, n_chains,
                                                                    key, img_tag, cold ? 1 : 0);
-    return cudaGetLastError();
+    return launched();
 }
 
 cudaError_t launch_sample_energy(ImgDev* img, int n_img, long long max_sites, const float* samp, float q,
                                  float J, int gmrf, double* sums, unsigned long long* npairs, cudaStream_t s) {
     sample_energy_kernel<<<dim3(blocks_for(max_sites, 31 * 64, 152 * 8), n_img), 256, 0, s>>>(
         img, samp, q, J, gmrf, sums, npairs);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launched();
     if (e != cudaSuccess) return e;
     sample_energy_finish_kernel<<<(n_img + 127) / 128, 128, 0, s>>>(img, sums, npairs, n_img);
-    return cudaGetLastError();
+    return launched();
 }
 
 }  // namespace mpr

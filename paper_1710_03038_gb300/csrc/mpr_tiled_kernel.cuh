@@ -494,7 +494,7 @@ cudaError_t launch_one(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     if (a.gt < 1 || a.gt > Cf::GT || a.n_cap < 0 || a.n_cap > Cf::NMAX) return cudaErrorInvalidValue;
     dim3 grid(a.n_list, (a.chain_end - a.chain0 + a.chain_group - 1) / a.chain_group);
     kernel<<<grid, Cf::NT, Cf::smem_for(a.gt, a.n_cap, P), s>>>(a);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <int TX, int TY, int NW, int P, bool ACC, int MODEL, bool ENERGY>

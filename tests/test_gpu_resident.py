@@ -99,3 +99,37 @@ def test_a_temperature_that_gives_up_is_reported():
     ctx.sweep(2, "measure")
     assert bool(torch.isnan(ctx.predict()[0][torch.from_numpy(g).cuda() != 0]).all())
     device_error(ctx.check)
+
+
+# ------------------------------------------------------------------ what was launched
+
+def kernels(call):
+    before = mpr.launch_count()
+    call()
+    return mpr.launch_count() - before
+
+
+@pytest.mark.parametrize("use_graphs", [True, False])
+def test_launch_count(use_graphs):
+    """One kernel for a resident run; two passes and the bookkeeping for a launched sweep, the
+    bookkeeping once for sampling sweeps without energies; replays like the launches."""
+    img, side = image((130, 147), 0.3, 41), torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        alone = context([img], 8, 8, use_graphs=use_graphs)
+        big = context([img, image(*FILLER)], 8, 8, use_graphs=use_graphs)
+        plain = context([img], 8, 0, path="plain")
+        assert big.sweep_launches()[0] == 3
+        for n in (1, 5, 5):
+            assert kernels(lambda: alone.sweep(n, "measure")) == 1
+            assert kernels(lambda: alone.sweep(n, "equil")) == 1
+            assert kernels(lambda: big.sweep(n, "measure")) == 2 * n + 1
+            assert kernels(lambda: big.sweep(n, "equil")) == 3 * n
+            assert kernels(lambda: big.sweep(n, "measure", record_energy=True)) == 3 * n
+            assert kernels(lambda: plain.sweep(n, "measure")) == 3 * n
+        # (per sweep the stop rule's kernel too)
+        done = []
+        got = kernels(lambda: done.append(big.equilibrate(i_max=30)))
+        assert got == 4 * done[0]
+        assert kernels(lambda: big.predict()) == 1
+        assert kernels(lambda: big.image_info()) == 0
+    assert kernels(lambda: context([img], 8, 8)) > 20
