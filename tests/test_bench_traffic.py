@@ -8,6 +8,8 @@ import sys
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 sys.path.insert(0, ROOT)
 
+import pytest  # noqa: E402
+
 import bench  # noqa: E402
 
 
@@ -69,3 +71,34 @@ def test_record_is_written_from_an_ncu_raw_page(monkeypatch, tmp_path):
     assert got["dram_bytes_per_gap_update"] == round(2.5e6 / updates, 4)
     assert got["kernel_sources_sha16"] == bench.kernel_sources_hash()
     assert bench.recorded_traffic_per_update() == got["dram_bytes_per_gap_update"]
+
+
+def test_record_takes_the_colour_pass_as_it_is_named_now(monkeypatch, tmp_path):
+    """The kernel's eight template arguments (tile, warps, pairs, accumulation, model, energies,
+    groups): the sampling launch is taken whatever its warps and groups, an equilibration
+    launch and other kernels are not."""
+    import csv
+    import synthetic
+    wl = synthetic.workload("lognormal4096", L=64)
+    updates = int(wl.gap[0].sum()) * wl.chains / 2.0
+    monkeypatch.setattr(bench, "TRAFFIC_RECORD", str(tmp_path / "traffic.json"))
+    for k, name in enumerate(("16, 16, 4, 16, 1, 0, 0, 2", "16, 16, 2, 8, 1, 0, 0, 0", "32, 32, 8, 16, 1, 0, 1, 0")):
+        raw = tmp_path / f"raw{k}.csv"
+        with open(raw, "w", newline="") as f:
+            w = csv.writer(f)
+            w.writerow(["ID", "Kernel Name", "dram__bytes_read.sum", "dram__bytes_write.sum"])
+            w.writerow(["", "", "Mbyte", "Mbyte"])
+            w.writerow(["0", "void resident::resident_kernel<1, 0, 0>(mpr::ResidentArgs)", "7.0", "7.0"])
+            w.writerow(["1", "void tiled::tiled_pass_kernel<16, 16, 4, 16, 0, 0, 0, 2>(SweepArgs)", "9.0", "9.0"])
+            w.writerow(["2", f"void tiled::tiled_pass_kernel<{name}>(SweepArgs)", "2.0", "0.5"])
+        bench.record_traffic(str(raw), 64, "ncu ...")
+        with open(bench.TRAFFIC_RECORD) as f:
+            assert json.load(f)["dram_bytes_per_gap_update"] == round(2.5e6 / updates, 4)
+    # an equilibration launch alone is refused
+    with open(raw, "w", newline="") as f:
+        w = csv.writer(f)
+        w.writerow(["ID", "Kernel Name", "dram__bytes_read.sum", "dram__bytes_write.sum"])
+        w.writerow(["", "", "Mbyte", "Mbyte"])
+        w.writerow(["1", "void tiled::tiled_pass_kernel<16, 16, 2, 8, 0, 0, 0, 1>(SweepArgs)", "9.0", "9.0"])
+    with pytest.raises(SystemExit):
+        bench.record_traffic(str(raw), 64, "ncu ...")
