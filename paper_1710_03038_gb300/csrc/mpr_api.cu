@@ -248,6 +248,8 @@ struct mpr_ctx {
     // tiled: every tile and chain group fits the GPU at once, so a run of sweeps is one
     // launch (resident sweeps) with this much shared memory per block
     bool resident = false;
+    bool res_twice = false;  // two such runs fit at once
+    int most_tiles = 0;      // of an image
     int steps = 1;  // warp steps of a block in a colour pass, at the tile with the most sites
     size_t res_smem = 0;
     int polls = kDefaultPolls;  // reads of a wait of a resident run before it gives up
@@ -804,6 +806,8 @@ mpr_status choose_resident(mpr_ctx* c, const TileStats& st, cudaStream_t s) {
     long long blocks = 0;
     MPR_CUDA(resident_blocks(st.res_smem, &blocks));
     c->resident = need <= blocks;
+    c->res_twice = 2 * need <= blocks;
+    c->most_tiles = *std::max_element(c->g.ntiles.begin(), c->g.ntiles.end());
     ChainRange cr[2];
     chain_ranges(c, cr);
     // (four warps, 32 (site, pair) lanes each)
@@ -816,20 +820,34 @@ mpr_status choose_resident(mpr_ctx* c, const TileStats& st, cudaStream_t s) {
     return MPR_OK;
 }
 
-// Whether a run of sweeps goes to the resident kernel.  What it saves is the launches;
+// Whether a run of n sweeps goes to the resident kernel.  What it saves is the launches;
 // against it stand that its blocks hold their places on the SMs from the first sweep to
 // the last, which keeps other streams' work out, and that a sweep that adapts a or
-// records energies ends in a wait of every tile for the slowest one.  The more warp
-// steps a block has in a pass, the less the launches matter.  us per sweep, launches ->
-// resident, at up to two steps: 256^2 x 16 chains 15.9 -> 9.0 equilibrating, 12.7 -> 8.2
-// sampling; three: 400^2 x 8 at 60 % gaps 14.1 -> 11.3, 13.0 -> 9.5; four: 462 x 367 x 7
-// with a block of gaps at 23 % 12.6 -> 12.8 equilibrating, 12.5 -> 9.2 sampling, and two
-// such contexts in turn on two streams took 8.6 a sweep launched, 11.2 resident; six and
-// eight: GMRF 462 x 367 x 10 with recorded energies 21.6 -> 24.9, 20.6 -> 29.0, sampling
-// 16.1 -> 13.6, 16.6 -> 13.7; twelve (x 32) sampling 19.6 -> 20.8.
-bool resident_runs(const mpr_ctx* c, int phase, int flags) {
-    const bool waits = phase == MPR_EQUIL || (flags & MPR_RECORD_ENERGY);
-    return c->resident && c->steps <= (waits ? 3 : 8);
+// records energies ends in a wait of every tile for the slowest one.  The line lies where
+// two contexts, in turn on two streams, take no longer than launches per colour took
+// before there were resident runs.  us per sweep, one context / two in turn, those
+// launches -> today's launches -> resident:
+//  - images of at most 256 tiles, or two such runs fit the GPU at once: 64^2 x 7 12.5 / 6.6 ->
+//    10.8 / 5.8 -> 4.1 / 2.1 equilibrating; 350^2 x 4 12.2 / 7.1 -> 12.1 / 7.2 -> 6.6 / 3.7; the
+//    temperature lattices' size, 256^2 x 16 at 97 % gaps, 16.8 / 10.5 -> 15.8 / 9.3 -> 9.5 / 8.8;
+//    at three steps (128^2 x 100) 17.6 / 10.2 -> 15.3 / 9.1 -> 8.1 / 7.9.  Up to three steps;
+//    sampling runs up to seven (200^2 x 100 22.6 / 13.4 -> 15.1 / 10.5 -> 14.0 / 12.4; at eight
+//    GMRF 462 x 367 x 10 18.9 / 10.4 -> 16.6 / 9.5 -> 12.3 / 11.2).
+//  - others: equilibration waits for the slowest of more tiles, 400^2 x 4 13.8 / 8.0 -> 12.5 /
+//    6.9 -> 7.4 / 8.7, 500^2 x 4 15.0 / 8.5 -> 13.1 / 7.9 -> 9.9 / 9.6: never.  Sampling runs at
+//    two steps 500^2 x 4 16.1 / 9.4 -> 11.8 / 7.0 -> 8.1 / 7.6, at three 400^2 x 8 18.1 / 10.2 ->
+//    13.1 / 9.2 -> 8.8 / 10.6.
+// Three contexts in turn on three streams are the price: 256^2 x 16 at 50 % gaps takes 8.0 a
+// sweep equilibrating (7.5 before there were resident runs, 6.2 with today's launches), 6.6
+// sampling (8.5, 5.8).
+// Single recorded sweeps (mpr_equilibrate outside graphs) also pay for the records'
+// set-up, by the tiles: 128^2 x 48 24.9 -> 22.2 -> 18.6, 200^2 x 8 of four images 24.8 -> 22.8 ->
+// 21.1, but 256^2 x 16 at 97 % 23.8 -> 24.9 -> 24.3, 500^2 x 4 22.8 -> 22.8 -> 28.2.
+bool resident_runs(const mpr_ctx* c, int n, int phase, int flags) {
+    const bool record = (flags & MPR_RECORD_ENERGY) != 0;
+    if (!c->resident || (n == 1 && record && c->most_tiles > 200)) return false;
+    if (c->most_tiles <= 256 || c->res_twice) return c->steps <= (phase == MPR_EQUIL || record ? 3 : 7);
+    return phase != MPR_EQUIL && c->steps <= 2;
 }
 
 mpr_status sub_workspace_size(const mpr_params& p, const mpr_T_opts& o, int n_img, const int* Lx,
@@ -1281,7 +1299,7 @@ void count_sweeps(mpr_ctx* c, int n, int phase, bool accumulate) {
 mpr_status run_sweeps(mpr_ctx* c, int n, int phase, int flags, bool stats, bool accumulate,
                       cudaStream_t s) {
     int done = 0;  // sweeps that went to resident launches
-    if (resident_runs(c, phase, flags)) {
+    if (resident_runs(c, n, phase, flags)) {
         const cudaError_t e = resident_chunks(
             n, [&](int m) { return launch_resident_run(c, m, phase, flags, stats, accumulate, s); }, &done);
         if (e != cudaSuccess) return fail(MPR_ERR_CUDA, std::string("sweep launch: ") + cudaGetErrorString(e));

@@ -9,13 +9,10 @@
 // both colours stay in shared memory, and so do the two tables of cells.  A pass
 // writes its new cells straight into the table that the other colour's pass reads.
 // Equilibration / sampling sweeps, us, launches per colour -> resident: 64^2 x 7
-// chains at 30 % gaps 11.3 / 11.4 -> 4.2 / 4.4; 256^2 x 16 12.4 / 12.8 -> 7.4 / 5.7;
-// 330^2 x 32 at 40 % 18.0 / 19.1 -> 12.4 / 12.2; 500^2 x 32 at 20 % 18.8 / 19.9 ->
-// 17.8 / 15.3 (close to one wave of blocks, the most there is room for; which runs of a
-// batch come here is decided by their warp steps, at the last two sizes the sampling
-// runs only: resident_runs).  What is left of a
-// 64^2 pass (2 us) is latency: about 1 us of dependent instructions of one warp step,
-// the rest the trip of the packets through L2.
+// chains at 30 % gaps 10.8 / 7.2 -> 4.1 / 4.3; 256^2 x 16 at 50 % 13.8 / 11.9 -> 8.4 /
+// 7.1; 350^2 x 4 12.1 / 10.8 -> 6.6 / 5.5.  Which runs come here: resident_runs.  What is
+// left of a 64^2 pass (2 us) is latency: about 1 us of dependent instructions of one warp
+// step, the rest the trip of the packets through L2.
 //
 // Exchange.  Only the ring cells come from other blocks.  A block publishes its
 // boundary sites as packets of two 64-bit words (angle, epoch), one per chain of the

@@ -133,3 +133,48 @@ def test_launch_count(use_graphs):
         assert kernels(lambda: big.predict()) == 1
         assert kernels(lambda: big.image_info()) == 0
     assert kernels(lambda: context([img], 8, 8)) > 20
+
+
+# tiles per image: 484 (two runs fit the GPU at once), 361 and 625 (one does), 90
+@pytest.mark.parametrize("shape,R,frac,want", [
+    ((130, 147), 8, 0.3, dict(equil=1, measure=1, equil_rec=1, measure_rec=1, single_rec=1)),
+    ((350, 350), 4, 0.4, dict(equil=1, measure=1, equil_rec=1, measure_rec=1, single_rec=0)),
+    ((300, 300), 16, 0.2, dict(equil=0, measure=1, equil_rec=0, measure_rec=1, single_rec=0)),
+    ((400, 400), 8, 0.2, dict(equil=0, measure=1, equil_rec=0, measure_rec=1, single_rec=0)),
+])
+def test_which_runs_are_resident(shape, R, frac, want):
+    ctx = context([image(shape, frac, 51)], R, 0)
+    got = {}
+    for name, n, phase, record in (("equil", 3, "equil", False), ("measure", 3, "measure", False),
+                                   ("equil_rec", 3, "equil", True), ("measure_rec", 3, "measure", True),
+                                   ("single_rec", 1, "equil", True)):
+        got[name] = int(kernels(lambda: ctx.sweep(n, phase, record_energy=record)) == 1)
+    assert got == want
+
+
+# more than 64 tiles to an image: several words to a chain, recorders of many packets;
+# chain groups of 4 with and without a rest, one group of all chains
+@pytest.mark.parametrize("shape,R,model", [((350, 350), 4, "mpr"), ((256, 256), 16, "mpr"), ((250, 250), 10, "mpr"),
+                                           ((251, 173), 16, "gmrf"), ((300, 300), 6, "gmrf")])
+def test_images_of_many_tiles(shape, R, model):
+    img, other = image(shape, 0.4, 61), image(FILLER[0], 0.3, 71)
+    out = []
+    for images, cg in (([img], 0), ([img, other], 4)):
+        ctx = context(images, R, cg, model=model)
+        if len(images) == 1:
+            assert kernels(lambda: ctx.sweep(2, "measure")) == 1
+        else:
+            ctx.sweep(2, "measure")
+        records = []
+        for n, phase, record in ((3, "equil", False), (4, "equil", True), (3, "measure", True), (5, "measure", False),
+                                 (1, "equil", True)):
+            ctx.sweep(n, phase, record_energy=record)
+            info = ctx.chain_info()
+            records.append({k: v[0] for k, v in info.items()})
+        out.append((ctx.get_state()[0], ctx.accumulators(), records))
+    assert torch.equal(out[0][0], out[1][0])
+    assert torch.equal(out[0][1][0][0], out[1][1][0][0]) and torch.equal(out[0][1][1][0], out[1][1][1][0])
+    for a, b in zip(out[0][2], out[1][2]):
+        assert np.array_equal(a["a"], b["a"]) and np.array_equal(a["accepted"], b["accepted"])
+        # the tiles' sums are the same bits; their FP64 total in another order
+        assert np.allclose(a["e_last"], b["e_last"], rtol=0, atol=1e-10, equal_nan=True)
