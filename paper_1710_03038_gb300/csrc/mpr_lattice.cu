@@ -42,11 +42,11 @@ struct Column {
 };
 
 __device__ __forceinline__ Column column_of(const GridTable& g, const float* phi) {
-    const int nx = (g.Lx + kCols - 1) / kCols;
+    const unsigned nx = ((unsigned)g.Lx + kCols - 1u) / kCols;
     Column c;
-    c.x = (int)(blockIdx.x % nx) * kCols + threadIdx.x;
+    c.x = (int)min((unsigned)(blockIdx.x % nx) * kCols + threadIdx.x, (unsigned)g.Lx);
     c.y0 = (int)min((long long)(blockIdx.x / nx) * kRows, (long long)g.Ly);  // (past its last chunk: nothing)
-    c.y1 = min(c.y0 + kRows, g.Ly);
+    c.y1 = (int)min((long long)c.y0 + kRows, (long long)g.Ly);
     c.Lx = g.Lx;
     c.Ly = g.Ly;
     c.in = c.x < g.Lx && c.y0 < g.Ly;
@@ -64,6 +64,62 @@ __device__ __forceinline__ void add_block(double v, double* out) {
 #pragma unroll
         for (int k = 1; k < kCols / 32; ++k) v += part[k];
         if (v != 0.0) atomicAdd(out, v);
+    }
+}
+
+// By site: a thread per pixel, FP64 sums.  The shorter way for small batches and for grids
+// that leave a block's columns or rows idle (by_columns).
+__global__ void lattice_energy_site_kernel(const __grid_constant__ Grids G, int k0,
+                                           const float* __restrict__ phi, float q, float J, double* H) {
+    const GridTable g = G.g[blockIdx.y];
+    const long long n = (long long)g.Lx * g.Ly;
+    const float* p = phi + g.off;
+    double s = 0.0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int x = (int)(i % g.Lx), y = (int)(i / g.Lx);
+        const float v = p[i];
+        float e = 0.0f;
+        if (x + 1 < g.Lx) e -= J * cosf(q * (v - p[i + 1]));
+        if (y + 1 < g.Ly) e -= J * cosf(q * (v - p[i + g.Lx]));
+        s += (double)e;
+    }
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(H + k0 + blockIdx.y, s);
+}
+
+template <bool GRAD, bool GJ>
+__global__ void lattice_grad_site_kernel(const __grid_constant__ Grids G, int k0,
+                                         const float* __restrict__ phi, float q, float J, const double* up,
+                                         float* __restrict__ grad, double* gJ) {
+    const GridTable g = G.g[blockIdx.y];
+    const long long n = (long long)g.Lx * g.Ly;
+    const float* p = phi + g.off;
+    const double uk = up[k0 + blockIdx.y];
+    const float w = (float)uk * J * q;
+    double sJ = 0.0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int x = (int)(i % g.Lx), y = (int)(i / g.Lx);
+        const float v = p[i];
+        if (GRAD) {
+            float s = 0.0f;
+            if (y > 0) s += sinf(q * (v - p[i - g.Lx]));
+            if (y + 1 < g.Ly) s += sinf(q * (v - p[i + g.Lx]));
+            if (x > 0) s += sinf(q * (v - p[i - 1]));
+            if (x + 1 < g.Lx) s += sinf(q * (v - p[i + 1]));
+            grad[g.off + i] = w * s;
+        }
+        if (GJ) {
+            float e = 0.0f;
+            if (x + 1 < g.Lx) e -= cosf(q * (v - p[i + 1]));
+            if (y + 1 < g.Ly) e -= cosf(q * (v - p[i + g.Lx]));
+            sJ += (double)e;
+        }
+    }
+    if (GJ) {
+        sJ = warp_sum(sJ) * uk;
+        if ((threadIdx.x & 31) == 0 && sJ != 0.0) atomicAdd(gJ, sJ);
     }
 }
 
@@ -163,6 +219,20 @@ __global__ void math_probe_kernel(int fn, int n, const float* a, const float* b,
     out[i] = v;
 }
 
+// A launch's grids: blocks to a grid by columns and by site, pixels of all of them.
+struct Chunk {
+    int blocks, site_blocks;
+    double sites, fill;  // fill: share of the columns' threads and rows that have a pixel
+};
+
+// By columns or by site.  us, columns / site (energy, both gradients): 12 x 128^2 11.5 / 14.4,
+// 14.9 / 17.0; 40 x 64^2 11.8 / 10.4, 14.9 / 15.0; 1 x 256^2 13.2 / 9.7, 16.8 / 10.6; 12 x 509 x
+// 383 14.9 / 105, 24.7 / 117.  Thin grids leave most of a block idle: 10^6 x 2 162 / 25, 543 / 31;
+// 10^5 x 32 28.9 / 28.9, 65 / 46; 30000 x 64 15.0 / 24.6, 30.4 / 30.3.  The torque alone sums
+// nothing and is the shorter by site up to larger batches: 4 x 512^2 12.9 / 11.9, 12 x 509 x 383
+// 17.0 / 20.9, 1 x 2048^2 27 / 36.
+bool by_columns(const Chunk& c, bool sums) { return c.fill >= 0.45 && c.sites >= (sums ? 1.8e5 : 2e6); }
+
 template <typename F>
 mpr_status for_chunks(int n, const int* Lx, const int* Ly, F launch) {
     if (n < 1 || !Lx || !Ly) return MPR_ERR_INVALID_ARG;
@@ -170,18 +240,38 @@ mpr_status for_chunks(int n, const int* Lx, const int* Ly, F launch) {
     for (int k0 = 0; k0 < n; k0 += kMaxGrids) {
         Grids G;
         const int m = std::min(kMaxGrids, n - k0);
-        long long blocks = 1;
+        long long blocks = 1, most = 1;
+        const long long first = off;
         for (int j = 0; j < m; ++j) {
             const int i = k0 + j;
             if (Lx[i] < 1 || Ly[i] < 1) return MPR_ERR_INVALID_ARG;
             G.g[j] = GridTable{Lx[i], Ly[i], off};
             off += (long long)Lx[i] * Ly[i];
-            blocks = std::max(blocks, (long long)((Lx[i] + kCols - 1) / kCols) * ((Ly[i] + kRows - 1) / kRows));
+            most = std::max(most, (long long)Lx[i] * Ly[i]);
+            blocks = std::max(blocks, ((kCols - 1LL + Lx[i]) / kCols) * ((kRows - 1LL + Ly[i]) / kRows));
         }
-        if (blocks > 0x7FFFFFFFLL) return MPR_ERR_INVALID_ARG;
-        if (launch(G, k0, m, (int)blocks) != cudaSuccess) return MPR_ERR_CUDA;
+        Chunk c;
+        c.sites = (double)(off - first);
+        c.fill = blocks > 0x7FFFFFFFLL ? 0.0 : c.sites / ((double)blocks * m * kCols * kRows);
+        c.blocks = (int)std::min(blocks, 0x7FFFFFFFLL);
+        c.site_blocks = (int)std::min((most + 255) / 256, 1024LL);
+        if (launch(G, k0, m, c) != cudaSuccess) return MPR_ERR_CUDA;
     }
     return MPR_OK;
+}
+
+template <bool GRAD, bool GJ>
+mpr_status gradients(int n, const int* Lx, const int* Ly, const float* phi, double q, double J, const double* g,
+                     float* grad, double* gJ, cudaStream_t s) {
+    return for_chunks(n, Lx, Ly, [&](const Grids& G, int k0, int m, const Chunk& c) {
+        if (by_columns(c, GJ))
+            lattice_grad_kernel<GRAD, GJ><<<dim3(c.blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, g,
+                                                                             grad, gJ);
+        else
+            lattice_grad_site_kernel<GRAD, GJ><<<dim3(c.site_blocks, m), 256, 0, s>>>(G, k0, phi, (float)q,
+                                                                                     (float)J, g, grad, gJ);
+        return launched();
+    });
 }
 
 }  // namespace
@@ -194,8 +284,12 @@ mpr_status mpr_lattice_energy(int n, const int* Lx, const int* Ly, const float* 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(H_out, 0, sizeof(double) * (n > 0 ? n : 0), s) != cudaSuccess)
         return MPR_ERR_CUDA;
-    return for_chunks(n, Lx, Ly, [&](const Grids& G, int k0, int m, int blocks) {
-        lattice_energy_kernel<<<dim3(blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, H_out);
+    return for_chunks(n, Lx, Ly, [&](const Grids& G, int k0, int m, const Chunk& c) {
+        if (by_columns(c, true))
+            lattice_energy_kernel<<<dim3(c.blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, H_out);
+        else
+            lattice_energy_site_kernel<<<dim3(c.site_blocks, m), 256, 0, s>>>(G, k0, phi, (float)q, (float)J,
+                                                                              H_out);
         return launched();
     });
 }
@@ -203,12 +297,7 @@ mpr_status mpr_lattice_energy(int n, const int* Lx, const int* Ly, const float* 
 mpr_status mpr_lattice_torque(int n, const int* Lx, const int* Ly, const float* phi, double q,
                               double J, const double* g, float* grad, mpr_stream stream) {
     if (!phi || !g || !grad) return MPR_ERR_INVALID_ARG;
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    return for_chunks(n, Lx, Ly, [&](const Grids& G, int k0, int m, int blocks) {
-        lattice_grad_kernel<true, false><<<dim3(blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, g,
-                                                                          grad, nullptr);
-        return launched();
-    });
+    return gradients<true, false>(n, Lx, Ly, phi, q, J, g, grad, nullptr, reinterpret_cast<cudaStream_t>(stream));
 }
 
 mpr_status mpr_lattice_grad(int n, const int* Lx, const int* Ly, const float* phi, double q,
@@ -217,12 +306,9 @@ mpr_status mpr_lattice_grad(int n, const int* Lx, const int* Ly, const float* ph
     if (!phi || !g || (!grad_phi && !grad_J)) return MPR_ERR_INVALID_ARG;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (grad_J && cudaMemsetAsync(grad_J, 0, sizeof(double), s) != cudaSuccess) return MPR_ERR_CUDA;
-    return for_chunks(n, Lx, Ly, [&](const Grids& G, int k0, int m, int blocks) {
-        const auto kernel = !grad_J ? lattice_grad_kernel<true, false>
-                            : grad_phi ? lattice_grad_kernel<true, true> : lattice_grad_kernel<false, true>;
-        kernel<<<dim3(blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, g, grad_phi, grad_J);
-        return launched();
-    });
+    if (!grad_J) return gradients<true, false>(n, Lx, Ly, phi, q, J, g, grad_phi, nullptr, s);
+    if (!grad_phi) return gradients<false, true>(n, Lx, Ly, phi, q, J, g, nullptr, grad_J, s);
+    return gradients<true, true>(n, Lx, Ly, phi, q, J, g, grad_phi, grad_J, s);
 }
 
 mpr_status mpr_philox(int n, const uint32_t* ctr, const uint32_t* key, uint32_t* out, int reference,
