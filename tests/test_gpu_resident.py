@@ -178,3 +178,34 @@ def test_images_of_many_tiles(shape, R, model):
         assert np.array_equal(a["a"], b["a"]) and np.array_equal(a["accepted"], b["accepted"])
         # the tiles' sums are the same bits; their FP64 total in another order
         assert np.allclose(a["e_last"], b["e_last"], rtol=0, atol=1e-10, equal_nan=True)
+
+
+# ------------------------------------------------------------------ graphs of launches
+
+@pytest.mark.parametrize("R,hole", [(6, False), (36, False), (8, True)])
+def test_replayed_graphs_of_a_launched_batch(R, hole):
+    """A batch that is launched per colour: runs captured once and replayed (also sampling runs,
+    whose launches carry their place in the run and share one bookkeeping launch) give the
+    bits of direct launches.  36 chains leave a group of 4 to a launch of its own, a hole
+    makes heavy tiles."""
+    z, g = image((530, 545), 0.35, 81)
+    if hole:
+        g[100:160, 200:270] = 1
+    side, out = torch.cuda.Stream(), []
+    for use_graphs in (True, False):
+        with torch.cuda.stream(side):
+            ctx = context([(z, g)], R, 32 if R > 32 else 0, use_graphs=use_graphs)
+            assert kernels(lambda: ctx.sweep(6, "equil")) >= 18
+            for n, phase, record in ((5, "measure", False), (5, "measure", False), (6, "equil", True),
+                                     (5, "measure", False), (7, "measure", True), (6, "equil", True),
+                                     (7, "measure", True), (5, "measure", False)):
+                ctx.sweep(n, phase, record_energy=record)
+            ctx.sweep(7, "measure", record_energy=True)
+            out.append((ctx.get_state()[0], ctx.accumulators(), ctx.chain_info(), ctx.sweep_index()))
+        side.synchronize()
+    assert torch.equal(out[0][0], out[1][0])
+    assert torch.equal(out[0][1][0][0], out[1][1][0][0]) and torch.equal(out[0][1][1][0], out[1][1][1][0])
+    assert np.array_equal(out[0][2]["a"], out[1][2]["a"]) and np.array_equal(out[0][2]["accepted"], out[1][2]["accepted"])
+    # FP64 totals of the tiles' sums, added in any order
+    assert np.allclose(out[0][2]["e_last"], out[1][2]["e_last"], rtol=0, atol=1e-10)
+    assert out[0][3] == out[1][3]
