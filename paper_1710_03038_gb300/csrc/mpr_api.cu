@@ -69,17 +69,19 @@ struct Geometry {
 };
 
 // Floats per slot of the state buffer: the tiled layout interleaves the chains, rounded
-// up to 4, 8, 16 or a multiple of 32, so that a chain group's row of a slot starts on
-// its own size and never straddles a 128-byte line (1024^2 at 50 % gaps: 100 chains in
-// rows of 400 bytes 296 us an equilibration and 316 a sampling sweep, in rows of 512
-// bytes 276 and 299).  Batches whose states would pass 16 GB that way keep to a multiple
-// of 4, so that the rounding costs 8 GB at most (by the pixels alone: the choice must
-// not depend on the gaps or the tile shape).
+// up to a multiple of 4, or of 32 where there are more than 32 chains and that adds at
+// most 30 %: a group's row of a slot then starts on a 128-byte line (1024^2 at 50 % gaps,
+// us per equilibration / sampling sweep, rows of a multiple of 4 -> of 32: 100 chains 296 /
+// 316 -> 278 / 301, 52 chains 187 / 199 -> 181 / 193).  Wider rounding costs more memory
+// traffic than it saves (36 chains 115 / 125 -> 134 / 141, 33 112 / 120 -> 131 / 137), and
+// below 32 chains it gives up to 3 % (10 chains 54.1 / 55.5 -> 52.6 / 55.3) for up to twice
+// the memory.  Batches whose states would pass 16 GB that way keep to a multiple of 4 (by
+// the pixels alone: the choice must not depend on the gaps or the tile shape).
 long long state_chains(const Geometry& g) {
     const long long n = g.n_chains;
     if (g.path != MPR_PATH_TILED) return n;
-    const long long wide = n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : (n + 31) & ~31LL;
-    return g.n_sites * wide * 4 <= 16LL << 30 ? wide : (n + 3) & ~3LL;
+    const long long wide = (n + 31) & ~31LL;
+    return n > 32 && wide * 10 <= n * 13 && g.n_sites * wide * 4 <= 16LL << 30 ? wide : (n + 3) & ~3LL;
 }
 
 void make_geometry(Geometry& g, int n_img, const int* Lx, const int* Ly, int n_chains, int path,

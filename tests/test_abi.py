@@ -141,3 +141,11 @@ def test_batches_that_cannot_be_resident_reserve_no_packets(lib, side, chains):
         assert extra < tiles * (8 * (4 * ((chains + 31) // 32 * 32) + 64) + 1024)
     assert (_workspace(lib, 128, 32, tile_x=16, tile_y=16, literal_or=1)
             < _workspace(lib, 128, 32, tile_x=16, tile_y=16))
+
+
+@pytest.mark.parametrize("chains", [5, 9, 17, 21, 33, 36, 40, 65, 100])
+def test_states_are_rounded_by_less_than_a_third(lib, chains):
+    """A workspace's states: within 30 % of 4 bytes per chain and pixel (and 4 chains)."""
+    side = 1024
+    states = _workspace(lib, side, chains) - _workspace(lib, side, 1)
+    assert states <= 4.0 * side * side * (1.3 * chains + 4) + 2 ** 24
