@@ -529,13 +529,17 @@ cudaError_t launch_groups(const SweepArgs& a, cudaStream_t s, bool setup_only) {
 // launches before: GMRF 462 x 367 x 10 with a block of gaps 15.6 / 19.1 / 16.2 equilibrating,
 // 11.8 / 16.7 / 17.5 sampling; 500^2 at 40 % x 16, 625 blocks, 17.4 / 20.7 / 20.1; 640 x 480 x
 // 16, 1200 blocks, 18.9 / 20.1 / 19.8; 600^2 x 4, 1444 blocks, 16.1 / 15.2 / 19.7).
+// The counting pass of a sampling run (its last sweep) keeps the four warps in large launches:
+// its blocks' counts and realisation sums queue at the same L2 slices, the more the faster
+// the blocks go by (single sampling sweeps of 2000^2 x 4, 15625 blocks: 156 with one warp, 143
+// with four, 146 before there were fewer; 1000^2 x 4, 3969 blocks, 37 and 39).
 // Passes that record energies keep the four warps, which fix the order of their sums,
 // and so do launches beside another (1024^2 x 100: 276 -> 285).
 constexpr int small_group_warps(int P, bool acc) {
     return P == 2 ? 1 : P == 4 && acc ? 2 : P == 8 ? 2 : 4;
 }
 constexpr int kSmallGroupSmWarps = 26;
-constexpr long long kSmallGroupBlocks = 152 * 8;
+constexpr long long kSmallGroupBlocks = 152 * 8, kCountBlocks = 8192;
 
 template <int TX, int TY, int NW, int P, bool ACC, int MODEL>
 cudaError_t launch_acc(const SweepArgs& a, cudaStream_t s, bool setup_only) {
@@ -548,7 +552,9 @@ cudaError_t launch_acc(const SweepArgs& a, cudaStream_t s, bool setup_only) {
     if (a.flags & kEnergy) return launch_groups<TX, TY, NW, P, ACC, MODEL, true>(a, s, false);
     constexpr size_t kSmBytes = 228 * 1024, kReserved = 1024;  // of an SM, per block
     const long long groups = (a.chain_end - a.chain0 + a.chain_group - 1) / a.chain_group;
-    if (kFew != NW && a.chain_end - a.chain0 == a.n_chains && a.n_list * groups >= kSmallGroupBlocks &&
+    const long long launch_blocks = a.n_list * groups;
+    const bool counts = ACC && (a.flags & kCount) && launch_blocks >= kCountBlocks;
+    if (kFew != NW && a.chain_end - a.chain0 == a.n_chains && launch_blocks >= kSmallGroupBlocks && !counts &&
         (Cfg<TX, TY, kFew, MODEL>::smem_for(a.gt, a.n_cap, P) + kReserved) *
                 ((kSmallGroupSmWarps + kFew - 1) / kFew) <= kSmBytes)
         return launch_groups<TX, TY, kFew, P, ACC, MODEL, false>(a, s, false);

@@ -294,3 +294,22 @@ def test_blocks_of_fewer_warps_equal_the_plain_path(R, model):
         assert np.array_equal(out[0][1][k], out[1][1][k])
     # the mean of angles rounded to 2^-24 rad, mapped back and rounded to FP32
     assert torch.allclose(out[0][2], out[1][2], rtol=1e-6, atol=1e-5)
+
+
+@pytest.mark.parametrize("R", [4, 16])
+def test_counting_passes_of_large_launches_equal_the_plain_path(R):
+    """8281 tiles: the last sweep of a sampling run takes four warps, the others fewer."""
+    z = np.resize(synthetic.grf((256, 256), nu=0.5, ell=9.0, mean=50, std=10, seed=65), (1450, 1449)).astype(np.float32)
+    g = synthetic.uniform_gaps((1450, 1449), 0.3, 66).astype(np.uint8)
+    out = []
+    for path in ("plain", "tiled"):
+        ctx = mpr.Context([z], [g], chains=R, params=mpr.Params(seed=81, path=path))
+        ctx.set_T([0.1])
+        ctx.sweep(1, "equil")
+        ctx.sweep(1, "measure")
+        ctx.sweep(2, "measure")
+        out.append((ctx.get_state()[0], ctx.chain_info(), ctx.predict()[0]))
+    assert torch.equal(out[0][0], out[1][0])
+    assert np.array_equal(out[0][1]["accepted"], out[1][1]["accepted"])
+    # the mean of angles rounded to 2^-24 rad, mapped back and rounded to FP32
+    assert torch.allclose(out[0][2], out[1][2], rtol=1e-6, atol=1e-5)
