@@ -1834,10 +1834,10 @@ mpr_status mpr_energy(mpr_ctx* c, double* e_out, mpr_mem where, mpr_stream strea
     const int gmrf = c->p.model == MPR_MODEL_GMRF ? 1 : 0;
     // a block per tile, but a thread per pixel where that is the shorter way: batches of fewer
     // than 2^16 pixels x chains (us, tile / pixel: 64^2 x 10 11.4 / 10.2, x 16 11.8 / 12.1; 128^2
-    // x 2 12.3 / 10.7, x 4 12.2 / 12.8) and single chains of large maps (1000 x 777 27.8 / 21.3,
-    // 2048^2 81 / 53; 256^2 11.8 / 13.1)
+    // x 2 12.3 / 10.7, x 4 12.2 / 12.8) and one or two chains of large maps (one: 1000 x 777 27.8 /
+    // 21.3, 2048^2 81 / 53, 256^2 11.8 / 13.1; two: 2048^2 114 / 119, 4000^2 586 / 564)
     const bool by_tile = c->g.path == MPR_PATH_TILED && c->g.n_sites * c->g.n_chains >= (1 << 16) &&
-                         (c->g.n_chains > 1 || maxn < (1 << 18));
+                         (c->g.n_chains > 2 || maxn < (c->g.n_chains == 1 ? 1 << 18 : 1 << 23));
     if (by_tile) {
         const int most = *std::max_element(c->g.ntiles.begin(), c->g.ntiles.end());
         MPR_CUDA(launch_energy_tiles(c->d_img, c->d_tiles, c->g.n_img, most, c->g.tx, c->g.ty, c->d_state,
