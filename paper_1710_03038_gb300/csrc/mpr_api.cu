@@ -1069,7 +1069,7 @@ mpr_status init_impl(mpr_ctx* c, int n_img, const int* Lx, const int* Ly, int n_
         double* sums = scratch + 2 * n_img;
         unsigned long long* npairs = reinterpret_cast<unsigned long long*>(scratch + 3 * n_img);
         MPR_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * 2 * n_img, s));
-        MPR_CUDA(launch_sample_energy(c->d_img, n_img, maxn, c->d_samp, (float)c->p.q, (float)c->p.J,
+        MPR_CUDA(launch_sample_energy(c->d_img, n_img, maxn, c->d_samp, (float)c->p.q, c->p.J,
                                       c->p.model == MPR_MODEL_GMRF ? 1 : 0, sums, npairs, s));
     }
     c->sweep = 0;
@@ -1841,7 +1841,7 @@ mpr_status mpr_energy(mpr_ctx* c, double* e_out, mpr_mem where, mpr_stream strea
     if (by_tile) {
         const int most = *std::max_element(c->g.ntiles.begin(), c->g.ntiles.end());
         MPR_CUDA(launch_energy_tiles(c->d_img, c->d_tiles, c->g.n_img, most, c->g.tx, c->g.ty, c->d_state,
-                                     c->d_samp, c->d_slot_map, c->g.n_chains, (float)c->p.q, (float)c->p.J,
+                                     c->d_samp, c->d_slot_map, c->g.n_chains, (float)c->p.q, c->p.J,
                                      gmrf, d_out, s));
     } else {
         const auto kernel = c->g.path == MPR_PATH_TILED ? energy_kernel<true> : energy_kernel<false>;

@@ -158,7 +158,7 @@ template <int STRIP, int NW, int C>
 __global__ void __launch_bounds__(NW * 32)
 energy_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int ty, const float* state,
                    const float* samp, const int* slot_map, int n_chains, int r_base, int r_end, float q,
-                   float J, int gmrf, double* out) {
+                   float J, double scale, int gmrf, double* out) {
     extern __shared__ float ang[];  // [(STRIP + 1) x (tx + 1)][C]
     __shared__ double part[NW][C];
     constexpr int kPixels = 32 / C;  // pixels of a warp side by side
@@ -245,7 +245,7 @@ energy_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int ty,
         double s = 0.0;
 #pragma unroll
         for (int k = 0; k < NW; ++k) s += part[k][lane];
-        atomicAdd(out + (long long)blockIdx.z * n_chains + r0 + lane, s);
+        atomicAdd(out + (long long)blockIdx.z * n_chains + r0 + lane, s * scale);
     }
 }
 
@@ -284,7 +284,8 @@ cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_t
 
 cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles, int tx,
                                 int ty, const float* state, const float* samp, const int* slot_map,
-                                int n_chains, float q, float J, int gmrf, double* out, cudaStream_t s) {
+                                int n_chains, float q, double J, int gmrf, double* out, cudaStream_t s) {
+    const ScaledJ j(J);
     const auto launch = [&](auto kernel, int strip, int C, int r_base, int chains) {
         const int groups = (chains + C - 1) / C;
         const size_t smem = (size_t)(tx + 1) * (strip + 1) * C * sizeof(float);
@@ -296,7 +297,7 @@ cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_
         const long long most = 152LL * 8 / std::max(1, groups * n_img) + 1;
         const int blocks = (int)std::max(1LL, std::min((long long)max_tiles * (ty / strip), most));
         kernel<<<dim3(blocks, groups, n_img), 256, smem, s>>>(img, tiles, log2_of(tx), ty, state, samp, slot_map,
-                                                              n_chains, r_base, r_base + chains, q, J, gmrf, out);
+                                                              n_chains, r_base, r_base + chains, q, j.m, j.scale, gmrf, out);
         return launched();
     };
     const auto chains_to_lanes = [](int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : 32; };

@@ -2,6 +2,7 @@
 // translation units of the library provide to each other.
 #pragma once
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <string>
@@ -128,6 +129,21 @@ inline cudaError_t launched(int n = 1) {
     return cudaGetLastError();
 }
 
+// J of a kernel that sums FP32 bond terms in two FP32 words, as m 2^e with 1/2 <= m < 1: the
+// terms are those of J but for the power of two, and neither overflow in the sum (J
+// above 1e36) nor lose its low word to the flush of denormals (below 1e-30).
+struct ScaledJ {
+    float m;
+    double scale;  // 2^e
+    explicit ScaledJ(double J) : m((float)J), scale(1.0) {
+        int e = 0;
+        if (std::isfinite(m)) {
+            m = std::frexp(m, &e);
+            scale = std::ldexp(1.0, e);
+        }
+    }
+};
+
 // ---- launchers ------------------------------------------------------------
 // setup_only: set the kernel's attributes without launching (before a capture)
 // (chain_group: even and at most 32, or covering every chain)
@@ -182,7 +198,7 @@ cudaError_t launch_hot_start(const ImgDev* img, const uint32_t* slot_pos, float*
                              cudaStream_t s);
 // e_s, E_ss and n_sp of every image (sums, npairs: zeroed scratch)
 cudaError_t launch_sample_energy(ImgDev* img, int n_img, long long max_sites, const float* samp, float q,
-                                 float J, int gmrf, double* sums, unsigned long long* npairs,
+                                 double J, int gmrf, double* sums, unsigned long long* npairs,
                                  cudaStream_t s);
 // Dynamic shared memory of a colour-pass block of tile shape tx x ty for a
 // launch whose largest tiles have gt table entries and n_cap own sites; flags: the model bits of
@@ -205,7 +221,7 @@ cudaError_t launch_state_tiles(const ImgDev* img, const TileDesc* tiles, int n_t
                                cudaStream_t s);
 cudaError_t launch_energy_tiles(const ImgDev* img, const TileDesc* tiles, int n_img, int max_tiles,
                                 int tile_x, int tile_y, const float* state, const float* samp,
-                                const int* slot_map, int n_chains, float q, float J, int gmrf,
+                                const int* slot_map, int n_chains, float q, double J, int gmrf,
                                 double* out, cudaStream_t s);
 
 // float offset of gap slot k (tiled) or site k (plain) of a realisation

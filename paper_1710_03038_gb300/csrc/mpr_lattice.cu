@@ -126,7 +126,7 @@ __global__ void lattice_grad_site_kernel(const __grid_constant__ Grids G, int k0
 // H_k = -J sum_<ij> cos(q (phi_i - phi_j)) over the right and down bonds of grid k.
 __global__ void __launch_bounds__(kCols)
 lattice_energy_kernel(const __grid_constant__ Grids G, int k0, const float* __restrict__ phi, float q,
-                      float J, double* H) {
+                      float J, double scale, double* H) {
     const Column c = column_of(G.g[blockIdx.y], phi);
     float hi = 0.0f, lo = 0.0f;
     if (c.in) {
@@ -144,7 +144,7 @@ lattice_energy_kernel(const __grid_constant__ Grids G, int k0, const float* __re
             v = below;
         }
     }
-    add_block(two_sum_value(hi, lo), H + k0 + blockIdx.y);
+    add_block(two_sum_value(hi, lo) * scale, H + k0 + blockIdx.y);
 }
 
 // Gradients of L = sum_k g_k H_k: GRAD the torque of every site, dL/dphi_i = g_k J q
@@ -284,9 +284,10 @@ mpr_status mpr_lattice_energy(int n, const int* Lx, const int* Ly, const float* 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(H_out, 0, sizeof(double) * (n > 0 ? n : 0), s) != cudaSuccess)
         return MPR_ERR_CUDA;
+    const ScaledJ j(J);
     return for_chunks(n, Lx, Ly, [&](const Grids& G, int k0, int m, const Chunk& c) {
         if (by_columns(c, true))
-            lattice_energy_kernel<<<dim3(c.blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, (float)J, H_out);
+            lattice_energy_kernel<<<dim3(c.blocks, m), kCols, 0, s>>>(G, k0, phi, (float)q, j.m, j.scale, H_out);
         else
             lattice_energy_site_kernel<<<dim3(c.site_blocks, m), 256, 0, s>>>(G, k0, phi, (float)q, (float)J,
                                                                               H_out);

@@ -110,7 +110,8 @@ constexpr int kRows = 8, kPairThreads = 256;
 
 __global__ void __launch_bounds__(kPairThreads)
 noalloc_pairs_kernel(const __grid_constant__ Shapes S, const float* __restrict__ z,
-                     const uint8_t* __restrict__ gap, ImgStat* stat, float q, float J, Partial* part) {
+                     const uint8_t* __restrict__ gap, ImgStat* stat, float q, float J, double scale_J,
+                     Partial* part) {
     __shared__ unsigned long long shu[32];
     __shared__ double shd[32];
     __shared__ ImgStat st;
@@ -177,7 +178,7 @@ noalloc_pairs_kernel(const __grid_constant__ Shapes S, const float* __restrict__
     const unsigned long long rc = block_reduce<unsigned long long>(cnt, add_u, shu, 0ull);
     if (threadIdx.x == 0) {
         Partial& p = part[im * kNoAllocBlocks + blockIdx.x];
-        p.sum = rs;
+        p.sum = rs * scale_J;
         p.n_pair = rc;
     }
 }
@@ -257,8 +258,9 @@ extern "C" mpr_status mpr_sample_energy_noalloc(int n_img, const int* Lx, const 
     ImgStat* stat = reinterpret_cast<ImgStat*>(part + kNoAllocMaxImages * kNoAllocBlocks);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     dim3 grid(kNoAllocBlocks, n_img);
+    const ScaledJ j(J);
     noalloc_extremes_kernel<<<grid, 256, 0, s>>>(S, z, gap, part);
-    noalloc_pairs_kernel<<<grid, kPairThreads, 0, s>>>(S, z, gap, stat, (float)q, (float)J, part);
+    noalloc_pairs_kernel<<<grid, kPairThreads, 0, s>>>(S, z, gap, stat, (float)q, j.m, j.scale, part);
     noalloc_final_kernel<<<n_img, kNoAllocBlocks, 0, s>>>(part, stat, e_s, reinterpret_cast<long long*>(n_sp),
                                               z_min, z_max);
     const cudaError_t e = launched(3);

@@ -431,8 +431,8 @@ __device__ __forceinline__ float bond_energy(float d, float q, float J, int gmrf
 }
 
 __global__ void __launch_bounds__(256)
-sample_energy_kernel(const ImgDev* img, const float* __restrict__ samp, float q, float J, int gmrf,
-                     double* sums, unsigned long long* npairs) {
+sample_energy_kernel(const ImgDev* img, const float* __restrict__ samp, float q, float J, double scale,
+                     int gmrf, double* sums, unsigned long long* npairs) {
     constexpr int kRows = 8;
     __shared__ double s_sum[8];
     __shared__ unsigned s_cnt[8];
@@ -478,7 +478,7 @@ sample_energy_kernel(const ImgDev* img, const float* __restrict__ samp, float q,
         s += s_sum[k];
         c += s_cnt[k];
     }
-    if (s != 0.0) atomicAdd(sums + blockIdx.y, s);
+    if (s != 0.0) atomicAdd(sums + blockIdx.y, s * scale);
     if (c) atomicAdd(npairs + blockIdx.y, c);
 }
 
@@ -582,9 +582,10 @@ cudaError_t launch_hot_start(const ImgDev* img, const uint32_t* slot_pos, float*
 }
 
 cudaError_t launch_sample_energy(ImgDev* img, int n_img, long long max_sites, const float* samp, float q,
-                                 float J, int gmrf, double* sums, unsigned long long* npairs, cudaStream_t s) {
+                                 double J, int gmrf, double* sums, unsigned long long* npairs, cudaStream_t s) {
+    const ScaledJ j(J);
     sample_energy_kernel<<<dim3(blocks_for(max_sites, 31 * 64, 152 * 8), n_img), 256, 0, s>>>(
-        img, samp, q, J, gmrf, sums, npairs);
+        img, samp, q, j.m, j.scale, gmrf, sums, npairs);
     cudaError_t e = launched();
     if (e != cudaSuccess) return e;
     sample_energy_finish_kernel<<<(n_img + 127) / 128, 128, 0, s>>>(img, sums, npairs, n_img);

@@ -70,3 +70,27 @@ def test_the_longest_lines(lx, ly):
     _lib.call("mpr_lattice_energy", 1, _lib.int_array([lx]), _lib.int_array([ly]), mpr._ptr(phi), Q, 1.0,
               mpr._ptr(H), mpr._stream_ptr())
     assert float(H) == -(2.0 ** 31 - 2)
+
+
+@pytest.mark.parametrize("big", [1e37, 1e-33])
+def test_energies_of_extreme_exchange(big):
+    """J near the ends of FP32: the sums of energies scale with J (FP32 terms, wider sums).
+    Every sum that is kept in two FP32 words: grids by column, the sample energy of a
+    context and of the allocation-free entry point, the chains' energies by tile."""
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    phi = 6.28 * torch.rand(1, 600, 513, device="cuda", generator=gen)
+    z = 50 + 10 * torch.randn(211, 203, device="cuda", generator=gen)
+    g = (torch.rand(211, 203, device="cuda", generator=gen) < 0.4).to(torch.uint8)
+    got = []
+    for j in (1.0, big):
+        H = mpr.lattice_energy(phi, q=Q, J=j)
+        ns = mpr.sample_energy_noalloc([z], [g], J=j)["e_s"]
+        out = [H.cpu().numpy(), ns.cpu().numpy()]
+        for model in ("mpr", "gmrf"):
+            ctx = mpr.Context([z], [g], chains=10, params=mpr.Params(J=j, model=model, seed=4))
+            out += [ctx.image_info()["e_s"], ctx.energy().reshape(-1)]
+        got.append(out)
+    for k, (a, b) in enumerate(zip(*got)):
+        # J and every bond's product with it are rounded to FP32 once each, 6e-8 of a bond; the
+        # first is a sum over bonds, the others are means
+        assert abs(b / big - a).max() <= 1.2e-7 * (2 * phi.numel() if k == 0 else 1)
