@@ -51,7 +51,7 @@ predict_tile_kernel(const ImgDev* img, const TileDesc* tiles, int tx_log, int np
             const double v = fma(-m, m, acc2[k] * inv_n);
             const float vf = (float)v;
             float sd = cut_short ? __int_as_float(0x7FC00000) : 0.0f;
-            if (vf > 1e30f) {  // (beyond the estimate's range: angles are below 2 pi)
+            if (vf > 1e30f || (vf <= 1e-30f && v > 0.0)) {  // (beyond the estimate's range)
                 sd = (float)(sqrt(v) * per_rad);
             } else if (vf > 1e-30f) {
                 const double r = (double)rsqrtf(vf), y = v * r;

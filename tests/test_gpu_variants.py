@@ -313,3 +313,23 @@ def test_counting_passes_of_large_launches_equal_the_plain_path(R):
     assert np.array_equal(out[0][1]["accepted"], out[1][1]["accepted"])
     # the mean of angles rounded to 2^-24 rad, mapped back and rounded to FP32
     assert torch.allclose(out[0][2], out[1][2], rtol=1e-6, atol=1e-5)
+
+
+def test_spread_of_the_smallest_and_largest_variances():
+    """Restored sums far from any angle's: the spread is the square root of the variance, in
+    FP64, for a map whose range makes it visible."""
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    z = torch.rand(40, 48, device="cuda", generator=gen) * 1e28
+    g = (torch.rand(40, 48, device="cuda", generator=gen) < 0.5).to(torch.uint8)
+    ctx = mpr.Context([z], [g], chains=4, params=mpr.Params(seed=5))
+    gap = g != 0
+    var = 10.0 ** (80 * torch.rand(40, 48, dtype=torch.float64, device="cuda", generator=gen) - 48)
+    var[0] = 0.0
+    ctx.set_accumulators([torch.zeros_like(var)], [var * 8], 8)
+    sd = ctx.predict(std=True)[1][0]
+    info = ctx.image_info()
+    want = (torch.sqrt(var) * (float(info["zmax"][0]) - float(info["zmin"][0])) / (2 * np.pi))[gap]
+    # FP64 throughout and one rounding to FP32 (infinite beyond its range)
+    over = torch.isinf(want.float())
+    assert torch.isinf(sd[gap][over]).all()
+    assert ((sd[gap].double() - want)[~over].abs() <= 1.2e-7 * want[~over]).all()
