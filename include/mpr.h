@@ -238,8 +238,8 @@ mpr_status mpr_select_q(int Lx, int Ly, const float* z, const uint8_t* gap, cons
  * sweep (the plain path: two passes and the bookkeeping).  A graph replay of n
  * sweeps runs n times that many kernels, less the bookkeeping of all but the last of
  * n sampling sweeps without recorded energies.  Batches whose tiles and chain groups fit
- * the GPU at once run n sweeps of mpr_sweep or mpr_estimate_T as one launch instead where
- * a block's share of a tile is small.
+ * the GPU at once run n sweeps of mpr_sweep or mpr_estimate_T as one (cooperative) launch
+ * instead where that is the shorter way; mpr_launch_count() tells what was launched.
  * Host only. */
 mpr_status mpr_sweep_launches(const mpr_ctx* ctx, int* per_sweep, int* per_T_sweep);
 

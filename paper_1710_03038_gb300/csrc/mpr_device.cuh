@@ -351,8 +351,10 @@ __device__ __forceinline__ float gmrf_bond(float d) {
 }
 
 // --------------------------------------------------------- reductions
-// (hi, lo) += e without loss: hi takes the rounded sum, lo its rounding error (TwoSum,
-// Knuth, The Art of Computer Programming 2, 4.2.2).
+// (hi, lo) += e: hi takes the rounded sum and lo adds its rounding error, which TwoSum
+// (Knuth, The Art of Computer Programming 2, 4.2.2) gives exactly.  lo is rounded itself:
+// over the few dozen additions of a strip the pair holds about 48 bits of the sum, against
+// terms of 24.
 __device__ __forceinline__ void two_sum(float& hi, float& lo, float e) {
     const float s = __fadd_rn(hi, e), b = __fsub_rn(s, hi);
     lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(e, b)));

@@ -29,8 +29,8 @@ struct Grids {
 // grid, blockIdx.y: the grid), so that no pixel index is divided, the pixel below is
 // the next row's own pixel, and a bond's sine serves both of its ends (sin is odd, bit
 // for bit): the bond above comes from the row before, the one on the left from the
-// lane before.  Bond terms in FP32; their sums in two FP32 words (no rounding error
-// lost), FP64 from the end of the column on: an FP64 addition per pixel alone would
+// lane before.  Bond terms in FP32; their sums in two FP32 words (two_sum:
+// about 48 bits), FP64 from the end of the column on: an FP64 addition per pixel alone would
 // take as long as everything else (12 grids of 509 x 383: energy 102 us, gradient 115
 // us before, with a 64-bit division and an FP64 addition per pixel).
 constexpr int kRows = 16, kCols = 128;

@@ -386,8 +386,8 @@ __global__ void map_kernel(const ImgDev* img, const float* z, const uint8_t* gap
 }
 
 // Start of the tiled state: hot (slot -> 2 pi u with the site's first uniform
-// at sweep 0xFFFFFFFF) or cold (every gap angle pi); padding slots and padding chains
-// hold 0.  One thread per (slot, four chains): two Philox blocks (words 0 and 2 of the
+// at sweep 0xFFFFFFFF) or cold (every gap angle pi); padding slots and the padding chains up
+// to the next multiple of 4 hold 0, what wider rows have beyond them stays undefined.  One thread per (slot, four chains): two Philox blocks (words 0 and 2 of the
 // pair's) and one 16-byte store; bound by the stores (2048^2 x 32: 215 MB).  A thread per
 // pair with a 64-bit division took 75 us of it.
 __global__ void __launch_bounds__(256)
