@@ -434,7 +434,11 @@ def select_q(z, gap, holdout, qs, chains: int = 16, n_equil: int = 100, n_meas: 
 
 def fill(z, gap, chains: int, n_equil: int, n_meas: int, params: Params = None,
          topts: TOpts = None, T=None, std: bool = False):
-    """Whole gap fill (Alg. 2): init, SEM temperature (unless T given), sweeps, prediction."""
+    """Whole gap fill (Alg. 2): init, SEM temperature (unless T given), sweeps, prediction.
+
+    Returns without waiting for the GPU.  Should a kernel have given up waiting for
+    another, every gap pixel is NaN and the context's check() raises.
+    """
     ctx = Context(z, gap, chains, params, topts)
     if T is None:
         ctx.estimate_T_async()
